@@ -85,7 +85,7 @@ struct StatusDev {
     CountersDev live, last;
 };
 
-enum : int32_t { ST_OK = 0, ST_CAPACITY = 4, ST_LIST = 5, ST_NONFINITE = 6 };
+enum : int32_t { ST_OK = 0, ST_CAPACITY = 4, ST_LIST = 5, ST_NONFINITE = 6, ST_STUCK = 7 };
 #define DEM_HALT 2
 
 // Step control, read and written only by kernels (the host never needs to know, while
@@ -101,7 +101,25 @@ struct CtrlDev {
     uint32_t nsorts;     // sorts performed since the particles were set
     uint32_t cond_sorts; // sorts run as the conditional body of a step graph (launch accounting)
     uint32_t steps_done; // steps completed (not void) since the control block was set
-    int32_t pad;
+    int32_t sorted;      // the sort tail of this step has run (read and cleared by its bookkeeping)
+    // list mode
+    int32_t hcur;        // history buffer the next step reads
+    int32_t hlast;       // history buffer the last force pass wrote
+    uint32_t left;       // step loop: steps still to take (written with `stop` before the loop starts)
+    int32_t stop;        // step loop: LOOP_* below
+    uint32_t seen;       // step loop: `left` at the last end of a turn, and turns since it changed
+    uint32_t idle;
+    int32_t pad[2];
+};
+
+// State of the step loop (CtrlDev::stop). A force pass of the loop idles unless it is GO.
+enum : int32_t {
+    LOOP_GO = 0,       // the next step may run
+    LOOP_SORT = 1,     // the last step ends with a sort that has not run yet
+    LOOP_VOID = 2,     // the last step is void (DEM_HALT)
+    LOOP_DONE = 3,     // no steps left
+    LOOP_KEEP = 4,     // between decision and bookkeeping: a step that does not sort
+    LOOP_TOSORT = 5    // ... a step that sorts
 };
 
 __device__ __forceinline__ void raise_status(StatusDev* st, int32_t code, int32_t where) {

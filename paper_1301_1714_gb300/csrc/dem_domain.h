@@ -79,26 +79,29 @@ struct Domain {
     uint32_t diag_part_cap = 0;
     double* diag_out = nullptr;
 
+    int in_loop = 0;      // 1 while the step loop is being captured
+    cudaGraphConditionalHandle loop_inner{}, loop_outer{};   // of the loop being captured
     int64_t launches = 0;
 
     std::vector<void*> allocations;   // every cudaMalloc of this domain (freed together)
 };
 
-// A CUDA graph of two captured timesteps and the kernel launches it holds.
+// The captured steps of a domain: a graph of two timesteps, or (list mode) the step loop.
 struct StepGraph {
     cudaGraphExec_t exec = nullptr;
-    int64_t launches = 0;        // kernels every replay launches
+    bool loop = false;           // exec is the step loop (takes ctrl->left steps) and not two steps
+    bool no_loop = false;        // the driver refused conditional nodes
+    int64_t launches = 0;        // kernels every replay launches (loop: every step)
     int64_t body_launches = 0;   // kernels of one conditional sort body (list mode)
-    cudaGraphExec_t sort_exec[2] = {nullptr, nullptr};   // phase timing: the sort tail per history parity
+    cudaGraphExec_t sort_exec = nullptr;   // phase timing: the sort tail
     int64_t sort_launches = 0;   // kernels every sort-tail replay launches
     cudaStream_t side = nullptr; // stream on which the conditional bodies are captured
     void reset() {
         if (exec) cudaGraphExecDestroy(exec);
         exec = nullptr;
-        for (auto& x : sort_exec) {
-            if (x) cudaGraphExecDestroy(x);
-            x = nullptr;
-        }
+        if (sort_exec) cudaGraphExecDestroy(sort_exec);
+        sort_exec = nullptr;
+        loop = false;
         sort_launches = 0;
         launches = 0;
         body_launches = 0;
@@ -114,7 +117,9 @@ cudaError_t run_check_input(Domain& d, uint32_t n, const double* x, const double
                             uint32_t* out);
 cudaError_t run_hash(Domain& d);      // cell key + in-cell rank of the next state (if sorting)
 cudaError_t run_rebuild(Domain& d);   // scan, scatter, (cell, id) gather, lists (if sorting)
-cudaError_t run_end_step(Domain& d);  // step bookkeeping (swap or keep, counters)
+// step bookkeeping outside the loop (swap or keep, counters); step = false: after an import
+cudaError_t run_end_step(Domain& d, bool step = true);
+cudaError_t run_loop_end(Domain& d);  // decision and bookkeeping after a force pass of the step loop
 cudaError_t run_sort_cond(Domain& d, cudaGraphConditionalHandle h);  // graph condition = this step sorts
 cudaError_t run_force(Domain& d, bool eval, double* dbgF, double* dbgT);
 // list mode (dem_list.cu): the neighbour lists of a sort, and the force pass over them

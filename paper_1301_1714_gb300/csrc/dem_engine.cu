@@ -386,6 +386,10 @@ dem_status sync_status(dem_handle* h) {
                      where, DEM_LIST_CAP);
             return fail(h, DEM_ERR_CAPACITY, buf);
         }
+        if (code == ST_STUCK) {
+            snprintf(buf, sizeof buf, "the step loop stopped with %d steps left", where);
+            return fail(h, DEM_ERR_TIMEOUT, buf);
+        }
         snprintf(buf, sizeof buf, "non-finite position or velocity at sorted position %d", where);
         return fail(h, DEM_ERR_NONFINITE, buf);
     }
@@ -569,7 +573,7 @@ dem_status load_particles(dem_handle* h, int64_t n64, const double* x, const dou
         CK(h, run_import(d, xd, vd, wd, rd));
         CK(h, run_hash(d));
         CK(h, run_rebuild(d));
-        CK(h, run_end_step(d));
+        CK(h, run_end_step(d, false));
     }
     h->has_particles = true;
     h->eval_valid = false;
@@ -589,127 +593,134 @@ cudaError_t enqueue_step(Domain& d) {
     return run_end_step(d);
 }
 
-// One step for a graph in list mode: force pass, the kernel that sets the condition, a
-// conditional node whose body (captured on the side stream) is the sort and the new
-// lists, then the bookkeeping. A step that does not sort launches three kernels.
-// The part of a list-mode step after the force pass, while d.stream is capturing: the
-// condition kernel, the conditional sort node (body captured on g->side), bookkeeping.
-cudaError_t capture_sort_tail(Domain& d, StepGraph* g, int64_t& body) {
-    cudaError_t e;
-    cudaStreamCaptureStatus cs;
-    cudaGraph_t graph = nullptr;
-    const cudaGraphNode_t* deps = nullptr;
-    size_t ndeps = 0;
-    if ((e = cudaStreamGetCaptureInfo(d.stream, &cs, nullptr, &graph, &deps, nullptr, &ndeps)) != cudaSuccess) return e;
-    if (cs != cudaStreamCaptureStatusActive) return cudaErrorStreamCaptureInvalidated;
-    cudaGraphConditionalHandle hc;
-    if ((e = cudaGraphConditionalHandleCreate(&hc, graph, 0, 0)) != cudaSuccess) return e;
-    if ((e = run_sort_cond(d, hc)) != cudaSuccess) return e;
-    if ((e = cudaStreamGetCaptureInfo(d.stream, &cs, nullptr, &graph, &deps, nullptr, &ndeps)) != cudaSuccess) return e;
-    cudaGraphNodeParams p{};
-    p.type = cudaGraphNodeTypeConditional;
-    p.conditional.handle = hc;
-    p.conditional.type = cudaGraphCondTypeIf;
-    p.conditional.size = 1;
-    cudaGraphNode_t node;
-    if ((e = cudaGraphAddNode(&node, graph, deps, nullptr, ndeps, &p)) != cudaSuccess) return e;
-    if ((e = cudaStreamUpdateCaptureDependencies(d.stream, &node, nullptr, 1, cudaStreamSetCaptureDependencies)) !=
-        cudaSuccess)
-        return e;
-    cudaGraph_t bg = p.conditional.phGraph_out[0];
-    if ((e = cudaStreamBeginCaptureToGraph(g->side, bg, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal)) !=
-        cudaSuccess)
-        return e;
-    const cudaStream_t main = d.stream;
-    const int64_t l0 = d.launches;
-    d.stream = g->side;
-    cudaError_t e1 = run_hash(d);
-    if (e1 == cudaSuccess) e1 = run_rebuild(d);
-    d.stream = main;
-    body = d.launches - l0;
-    d.launches = l0;
-    cudaGraph_t out = nullptr;
-    e = cudaStreamEndCapture(g->side, &out);
-    if (e1 != cudaSuccess) return e1;
-    if (e != cudaSuccess) return e;
-    return run_end_step(d);
-}
-
-cudaError_t capture_step_cond(Domain& d, StepGraph* g, int64_t& body) {
-    cudaError_t e;
-    if ((e = run_force(d, false, nullptr, nullptr)) != cudaSuccess) return e;
-    d.h_cur = 1 - d.h_cur;
-    return capture_sort_tail(d, g, body);
-}
-
-// Phase timing in list mode: the sort tail of a step as its own graph, one per history
-// parity (the tail reads the contact counts of the buffer the force pass just wrote).
-cudaError_t capture_sort_graphs(Domain& d, StepGraph* g) {
-    cudaError_t e;
-    if (!g->side && (e = cudaStreamCreateWithFlags(&g->side, cudaStreamNonBlocking)) != cudaSuccess) {
-        g->side = nullptr;
-        return e;
-    }
-    const int64_t l0 = d.launches;
-    const int hc0 = d.h_cur;
-    for (int par = 0; par < 2; ++par) {
-        d.h_cur = par;
-        if ((e = cudaStreamBeginCapture(d.stream, cudaStreamCaptureModeThreadLocal)) != cudaSuccess) break;
-        int64_t b = 0;
-        cudaError_t e1 = capture_sort_tail(d, g, b);
-        cudaGraph_t graph = nullptr;
-        e = cudaStreamEndCapture(d.stream, &graph);
-        if (e1 == cudaSuccess && e == cudaSuccess) e = cudaGraphInstantiate(&g->sort_exec[par], graph, 0);
-        if (graph) cudaGraphDestroy(graph);
-        if (e1 != cudaSuccess) e = e1;
-        if (e != cudaSuccess) break;
-        g->body_launches = b;
-        g->sort_launches = d.launches - l0;
-        d.launches = l0;
-    }
-    d.h_cur = hc0;
-    d.launches = l0;
-    if (e != cudaSuccess) {
-        for (int par = 0; par < 2; ++par)
-            if (g->sort_exec[par]) cudaGraphExecDestroy(g->sort_exec[par]);
-        g->sort_exec[0] = g->sort_exec[1] = nullptr;
-    }
+cudaError_t side_stream(StepGraph* g) {
+    if (g->side) return cudaSuccess;
+    const cudaError_t e = cudaStreamCreateWithFlags(&g->side, cudaStreamNonBlocking);
+    if (e != cudaSuccess) g->side = nullptr;
     return e;
 }
 
-// Two timesteps captured once as a CUDA graph (two, so that the history buffers return
-// to their starting roles) and replayed; plain launches on the legacy default stream.
-// In list mode the sort of each step is a conditional node (see capture_step_cond); if
-// the driver refuses conditional nodes the plain two-step graph is used.
-cudaError_t capture_cond_graph(Domain& d, StepGraph* g) {
+// Captures fn's launches on g->side into graph, after deps.
+template <class F>
+cudaError_t capture_into(Domain& d, StepGraph* g, cudaGraph_t graph, const cudaGraphNode_t* deps, size_t ndeps, F fn) {
+    cudaError_t e = cudaStreamBeginCaptureToGraph(g->side, graph, deps, nullptr, ndeps, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return e;
+    const cudaStream_t main = d.stream;
+    d.stream = g->side;
+    const cudaError_t e1 = fn();
+    d.stream = main;
+    cudaGraph_t out = nullptr;
+    e = cudaStreamEndCapture(g->side, &out);
+    return e1 != cudaSuccess ? e1 : e;
+}
+
+cudaError_t add_conditional(cudaGraphNode_t* node, cudaGraph_t graph, const cudaGraphNode_t* deps, size_t ndeps,
+                            cudaGraphConditionalHandle h, cudaGraphConditionalNodeType type, cudaGraph_t* body) {
+    cudaGraphNodeParams p{};
+    p.type = cudaGraphNodeTypeConditional;
+    p.conditional.handle = h;
+    p.conditional.type = type;
+    p.conditional.size = 1;
+    const cudaError_t e = cudaGraphAddNode(node, graph, deps, nullptr, ndeps, &p);
+    if (e == cudaSuccess) *body = p.conditional.phGraph_out[0];
+    return e;
+}
+
+// Phase timing in list mode: the sort tail of a step as its own graph (the condition
+// kernel, a conditional node whose body is the sort and the new lists, bookkeeping).
+cudaError_t capture_sort_graph(Domain& d, StepGraph* g) {
     cudaError_t e;
-    if (!g->side && (e = cudaStreamCreateWithFlags(&g->side, cudaStreamNonBlocking)) != cudaSuccess) {
-        g->side = nullptr;
+    if ((e = side_stream(g)) != cudaSuccess) return e;
+    const int64_t l0 = d.launches;
+    int64_t body = 0;
+    cudaGraph_t graph = nullptr, bg = nullptr;
+    cudaGraphConditionalHandle hc;
+    cudaGraphNode_t first = nullptr, node = nullptr;
+    size_t one = 1;
+    if ((e = cudaGraphCreate(&graph, 0)) != cudaSuccess) return e;
+    e = cudaGraphConditionalHandleCreate(&hc, graph, 0, 0);
+    if (e == cudaSuccess) e = capture_into(d, g, graph, nullptr, 0, [&] { return run_sort_cond(d, hc); });
+    if (e == cudaSuccess) e = cudaGraphGetNodes(graph, &first, &one);
+    if (e == cudaSuccess) e = add_conditional(&node, graph, &first, 1, hc, cudaGraphCondTypeIf, &bg);
+    if (e == cudaSuccess) {
+        const int64_t l1 = d.launches;
+        e = capture_into(d, g, bg, nullptr, 0, [&] {
+            const cudaError_t e1 = run_hash(d);
+            return e1 == cudaSuccess ? run_rebuild(d) : e1;
+        });
+        body = d.launches - l1;
+        d.launches = l1;
+    }
+    if (e == cudaSuccess) e = capture_into(d, g, graph, &node, 1, [&] { return run_end_step(d); });
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&g->sort_exec, graph, 0);
+    cudaGraphDestroy(graph);
+    if (e == cudaSuccess) {
+        g->body_launches = body;
+        g->sort_launches = d.launches - l0;
+    } else {
+        g->sort_exec = nullptr;
+    }
+    d.launches = l0;
+    return e;
+}
+
+// The step loop of list mode: a graph that takes ctrl->left steps by itself.
+//   while (steps left and no error) {
+//       while (steps left and no sort due) { LOOP_STEPS x (force pass, decision, bookkeeping) }
+//       the sort and the new lists (they do nothing when no sort is due), its bookkeeping
+//   }
+// A step that finds a sort due (or no step left) idles, so the sort needs no conditional
+// node of its own after every step: an untaken IF node costs 8 us on GB300, as much as ten
+// kernel nodes (0.8 us each), a turn of a WHILE node 3.2 us.
+constexpr int LOOP_STEPS = 8;
+
+cudaError_t capture_loop(Domain& d, StepGraph* g) {
+    cudaError_t e;
+    if ((e = side_stream(g)) != cudaSuccess) return e;
+    const int64_t l0 = d.launches;
+    cudaGraph_t graph = nullptr, outer = nullptr, inner = nullptr;
+    cudaGraphNode_t n_outer, n_inner;
+    int64_t steps = 0, body = 0;
+    if ((e = cudaGraphCreate(&graph, 0)) != cudaSuccess) return e;
+    d.in_loop = 1;
+    e = cudaGraphConditionalHandleCreate(&d.loop_outer, graph, 1, cudaGraphCondAssignDefault);
+    if (e == cudaSuccess)
+        e = add_conditional(&n_outer, graph, nullptr, 0, d.loop_outer, cudaGraphCondTypeWhile, &outer);
+    if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&d.loop_inner, outer, 1, cudaGraphCondAssignDefault);
+    if (e == cudaSuccess)
+        e = add_conditional(&n_inner, outer, nullptr, 0, d.loop_inner, cudaGraphCondTypeWhile, &inner);
+    if (e == cudaSuccess)
+        e = capture_into(d, g, inner, nullptr, 0, [&] {
+            cudaError_t e1 = cudaSuccess;
+            for (int k = 0; k < LOOP_STEPS && e1 == cudaSuccess; ++k) {
+                e1 = run_force(d, false, nullptr, nullptr);
+                if (e1 == cudaSuccess) e1 = run_loop_end(d);
+            }
+            return e1;
+        });
+    steps = d.launches - l0;
+    if (e == cudaSuccess)
+        e = capture_into(d, g, outer, &n_inner, 1, [&] {
+            const cudaError_t e1 = run_hash(d);
+            return e1 == cudaSuccess ? run_rebuild(d) : e1;
+        });
+    body = d.launches - l0 - steps;
+    d.in_loop = 0;
+    d.launches = l0;
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&g->exec, graph, 0);
+    cudaGraphDestroy(graph);
+    if (e != cudaSuccess) {
+        g->exec = nullptr;
         return e;
     }
-    const int64_t l0 = d.launches;
-    const int hc0 = d.h_cur;
-    if ((e = cudaStreamBeginCapture(d.stream, cudaStreamCaptureModeThreadLocal)) != cudaSuccess) return e;
-    int64_t b1 = 0, b2 = 0;
-    cudaError_t e1 = capture_step_cond(d, g, b1);
-    cudaError_t e2 = e1 == cudaSuccess ? capture_step_cond(d, g, b2) : e1;
-    cudaGraph_t graph = nullptr;
-    e = cudaStreamEndCapture(d.stream, &graph);
-    if (e1 == cudaSuccess && e2 == cudaSuccess && e == cudaSuccess) e = cudaGraphInstantiate(&g->exec, graph, 0);
-    if (graph) cudaGraphDestroy(graph);
-    const cudaError_t bad = e1 != cudaSuccess ? e1 : (e2 != cudaSuccess ? e2 : e);
-    if (bad != cudaSuccess) {
-        g->exec = nullptr;
-        d.launches = l0;
-        d.h_cur = hc0;
-        return bad;
-    }
-    g->launches = d.launches - l0;
-    g->body_launches = b1;
-    d.launches = l0;
+    g->loop = true;
+    g->launches = steps / LOOP_STEPS;
+    g->body_launches = body;
     return cudaSuccess;
 }
 
+// nsteps steps enqueued: the step loop (list mode) or a graph of two steps replayed; plain
+// launches on the legacy default stream and for an odd last step.
 cudaError_t run_steps(Domain& d, StepGraph* g, int64_t nsteps) {
     cudaError_t e;
     if (!g || !d.stream || d.n == 0) {
@@ -717,22 +728,37 @@ cudaError_t run_steps(Domain& d, StepGraph* g, int64_t nsteps) {
             if ((e = enqueue_step(d)) != cudaSuccess) return e;
         return cudaSuccess;
     }
-    if (d.h_cur == 1 && nsteps > 0) {
+    if (!d.list_mode && d.h_cur == 1 && nsteps > 0) {
         if ((e = enqueue_step(d)) != cudaSuccess) return e;
         --nsteps;
     }
-    if (nsteps >= 2 && !g->exec && d.list_mode) {
-        const cudaError_t ce = capture_cond_graph(d, g);
+    if (nsteps >= 2 && !g->exec && d.list_mode && !g->no_loop) {
+        const cudaError_t ce = capture_loop(d, g);
         if (ce != cudaSuccess) {
-            cudaGetLastError();   // conditional nodes unavailable: fall back to the plain graph
-            g->reset();
+            cudaGetLastError();   // conditional nodes unavailable: the plain graph of two steps
+            g->no_loop = true;
             static bool said = false;
             if (!said) {
                 said = true;
-                fprintf(stderr, "dem: step graph with a conditional sort node unavailable (%s); using the plain graph\n",
+                fprintf(stderr, "dem: step loop as a graph unavailable (%s); using the plain graph\n",
                         cudaGetErrorString(ce));
             }
         }
+    }
+    if (nsteps >= 2 && g->loop) {
+        for (int64_t k = nsteps & ~(int64_t)1; k > 0;) {
+            const int64_t chunk = std::min<int64_t>(k, 1 << 30);
+            CtrlDev* from = d.ctrl_host + 1;   // pinned; read by the copy before the loop starts
+            if (k != (nsteps & ~(int64_t)1) && (e = cudaStreamSynchronize(d.stream)) != cudaSuccess) return e;
+            from->left = (uint32_t)chunk;
+            from->stop = LOOP_GO;
+            if ((e = cudaMemcpyAsync(&d.ctrl->left, &from->left, 8, cudaMemcpyHostToDevice, d.stream)) != cudaSuccess ||
+                (e = cudaGraphLaunch(g->exec, d.stream)) != cudaSuccess)
+                return e;
+            d.launches += g->launches * chunk;
+            k -= chunk;   // (an even number of steps: the history buffers keep their roles)
+        }
+        nsteps &= 1;
     }
     if (nsteps >= 2 && !g->exec) {
         const int64_t l0 = d.launches;
@@ -798,7 +824,7 @@ dem_status dem_create(const dem_config* cfg, int device, void* cuda_stream, dem_
     if (cudaMalloc(&d.st, sizeof(StatusDev)) != cudaSuccess ||
         cudaMallocHost(&d.st_host, sizeof(StatusDev)) != cudaSuccess ||
         cudaMalloc(&d.ctrl, sizeof(CtrlDev)) != cudaSuccess ||
-        cudaMallocHost(&d.ctrl_host, sizeof(CtrlDev)) != cudaSuccess ||
+        cudaMallocHost(&d.ctrl_host, 2 * sizeof(CtrlDev)) != cudaSuccess ||
         cudaMemset(d.ctrl, 0, sizeof(CtrlDev)) != cudaSuccess ||
         cudaMalloc(&d.diag_out, 16 * sizeof(double)) != cudaSuccess ||
         cudaMalloc(&h->chk_dev, 2 * sizeof(uint32_t)) != cudaSuccess ||
@@ -878,15 +904,15 @@ dem_status dem_step(dem_handle* h, int64_t nsteps) {
         if (timed) {
             // list mode on a capturable stream: the sort tail runs as a small graph whose sort
             // node executes only when the device decided to sort
-            if (d.list_mode && d.stream && !h->graph.sort_exec[0] && capture_sort_graphs(d, &h->graph) != cudaSuccess)
+            if (d.list_mode && d.stream && !h->graph.sort_exec && capture_sort_graph(d, &h->graph) != cudaSuccess)
                 cudaGetLastError();
             for (int64_t s = 0; s < left; ++s) {
                 CK(h, cudaEventRecord(h->events[3 * s], d.stream));
                 CK(h, run_force(d, false, nullptr, nullptr));
                 CK(h, cudaEventRecord(h->events[3 * s + 1], d.stream));
                 d.h_cur = 1 - d.h_cur;
-                if (h->graph.sort_exec[d.h_cur]) {
-                    CK(h, cudaGraphLaunch(h->graph.sort_exec[d.h_cur], d.stream));
+                if (h->graph.sort_exec) {
+                    CK(h, cudaGraphLaunch(h->graph.sort_exec, d.stream));
                     d.launches += h->graph.sort_launches;
                 } else {
                     if (d.list_mode) CK(h, run_hash(d));   // (sort steps only; fused into the force pass otherwise)
@@ -1553,7 +1579,7 @@ dem_status repack(dem_batch* b) {
     nd.h_cur = 0;
     BCK(b, run_hash(nd));
     BCK(b, run_rebuild(nd));
-    BCK(b, run_end_step(nd));
+    BCK(b, run_end_step(nd, false));
     BCK(b, cudaStreamSynchronize(nd.stream));
     // swap in
     b->graph.reset();
@@ -1608,7 +1634,7 @@ dem_status dem_batch_create(int precision, int model, int stiffness, int max_con
     d.sort_blocks = sort_blocks_of(device);
     d.stream = (cudaStream_t)cuda_stream;
     if (cudaMalloc(&d.st, sizeof(StatusDev)) != cudaSuccess || cudaMallocHost(&d.st_host, sizeof(StatusDev)) != cudaSuccess ||
-        cudaMalloc(&d.ctrl, sizeof(CtrlDev)) != cudaSuccess || cudaMallocHost(&d.ctrl_host, sizeof(CtrlDev)) != cudaSuccess ||
+        cudaMalloc(&d.ctrl, sizeof(CtrlDev)) != cudaSuccess || cudaMallocHost(&d.ctrl_host, 2 * sizeof(CtrlDev)) != cudaSuccess ||
         cudaMalloc(&d.diag_out, 16 * sizeof(double)) != cudaSuccess || cudaMemset(d.st, 0, sizeof(StatusDev)) != cudaSuccess ||
         cudaMemset(d.ctrl, 0, sizeof(CtrlDev)) != cudaSuccess) {
         cudaGetLastError();

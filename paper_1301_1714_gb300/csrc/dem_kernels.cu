@@ -433,14 +433,17 @@ __global__ void k_reorder(uint32_t n, typename PR::State S0, typename PR::State 
 // the step just finished (descending; ties keep the (cell, id) order). The lanes of a warp run
 // their candidate lists in lockstep, so grouping similar counts shortens the longest
 // lane's loop; a particle's own sums keep their order, so results do not change.
-// Three passes replace k_reorder: the (cell, id) position of every particle, its final
-// position in its window, and the gather to the final position.
+// Two passes replace k_reorder: the (cell, id) position of every particle, then its final
+// position in its window and the gather to it.
 template <class PR>
 __global__ void k_rank_cell(uint32_t n, typename PR::State S0, typename PR::State S1, const CtrlDev* ctrl,
                             const uint32_t* __restrict__ key, const uint32_t* __restrict__ cs,
-                            const uint32_t* __restrict__ tmp, const uint32_t* __restrict__ hcnt_last,
-                            uint32_t* __restrict__ canon, uint32_t* __restrict__ wkey) {
+                            const uint32_t* __restrict__ tmp, const uint32_t* __restrict__ hcnt0,
+                            const uint32_t* __restrict__ hcnt1, uint32_t* __restrict__ canon,
+                            uint32_t* __restrict__ wkey) {
     if (ctrl->rebuild != 1) return;   // no sort this step (or a void step)
+    // contact counts of the step just finished (pre-sort order)
+    const uint32_t* __restrict__ hcnt_last = ctrl->hlast ? hcnt1 : hcnt0;
     const typename PR::State B = ctrl->cur ? S0 : S1;
     for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
         const uint32_t p = tmp[s];
@@ -455,17 +458,26 @@ __global__ void k_rank_cell(uint32_t n, typename PR::State S0, typename PR::Stat
 }
 
 // One block per window of wsize (cell, id) positions (blockDim.x: the power of two at or
-// above wsize, at most 1,024): fin[q] = final position, the window's particles in descending order of their last
-// contact count (ties in (cell, id) order), so the lanes of a force-pass warp carry similar
-// numbers of contacts. A window is split where one scene ends and the next begins (scenes
-// are contiguous in the (cell, id) order), so every particle stays inside its scene's range
-// of positions. The order is a bitonic sort in shared memory of one 32-bit word per
-// position: scene run within the window (10 bits), 63 - count (6 bits), position (10 bits).
+// above wsize, at most 1,024): fin[q] = final position, the window's particles in descending
+// order of their last contact count (ties in (cell, id) order), so the lanes of a force-pass
+// warp carry similar numbers of contacts. A window is split where one scene ends and the next
+// begins (scenes are contiguous in the (cell, id) order), so every particle stays inside its
+// scene's range of positions. The order is a bitonic sort in shared memory of one 32-bit word
+// per position: scene run within the window (10 bits), 63 - count (6 bits), position (10 bits).
+// The block then gathers its window's state to the final positions: the order it has just
+// found is still in shared memory, so a separate gather pass (one launch, and fin and canon
+// read once more) is not needed.
+template <class PR>
 __global__ void __launch_bounds__(1024) k_window(uint32_t n, uint32_t wsize, const SceneDev* scenes, int nscenes,
-                                                 const CtrlDev* ctrl, const uint32_t* __restrict__ wkey,
-                                                 uint32_t* __restrict__ fin) {
+                                                 typename PR::State S0, typename PR::State S1, const CtrlDev* ctrl,
+                                                 const uint32_t* __restrict__ wkey, const uint32_t* __restrict__ key,
+                                                 const uint32_t* __restrict__ canon, uint32_t* __restrict__ fin,
+                                                 uint32_t* __restrict__ perm, uint32_t* __restrict__ skey,
+                                                 float4* __restrict__ ref) {
     if (ctrl->rebuild != 1) return;   // no sort this step (or a void step)
     __shared__ uint32_t s_w[1024];
+    const typename PR::State A = ctrl->cur ? S1 : S0;
+    const typename PR::State B = ctrl->cur ? S0 : S1;
     const uint32_t w = blockDim.x, t = threadIdx.x;
     for (uint32_t base = blockIdx.x * wsize; base < n; base += gridDim.x * wsize) {
         const uint32_t q = base + t;
@@ -492,45 +504,101 @@ __global__ void __launch_bounds__(1024) k_window(uint32_t n, uint32_t wsize, con
                 __syncthreads();
             }
         const uint32_t sw = s_w[t];
-        if (sw != 0xFFFFFFFFu) fin[base + (sw & 1023u)] = base + t;
-    }
-}
-
-template <class PR>
-__global__ void k_gather(uint32_t n, typename PR::State S0, typename PR::State S1, const CtrlDev* ctrl,
-                         const uint32_t* __restrict__ key, const uint32_t* __restrict__ canon,
-                         const uint32_t* __restrict__ fin, uint32_t* __restrict__ perm, uint32_t* __restrict__ skey,
-                         float4* __restrict__ ref) {
-    if (ctrl->rebuild != 1) return;   // no sort this step (or a void step)
-    const typename PR::State A = ctrl->cur ? S1 : S0;
-    const typename PR::State B = ctrl->cur ? S0 : S1;
-    for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
-        const uint32_t p = canon[q], f = fin[q];
+        if (sw == 0xFFFFFFFFu) continue;
+        const uint32_t from = base + (sw & 1023u);   // (cell, id) position of the particle stored at q
+        fin[from] = q;
+        const uint32_t p = canon[from];
         const typename PR::Self m = PR::load(B, p);
-        PR::store(A, f, m);
-        perm[f] = p;
-        skey[f] = key[p];
-        ref[f] = PR::pos_f(m);
+        PR::store(A, q, m);
+        perm[q] = p;
+        skey[q] = key[p];
+        ref[q] = PR::pos_f(m);
     }
 }
 
-// Step bookkeeping (one thread): after a sort the current set stays and springs are read
-// through the permutation next step; otherwise the next set becomes current.
-__global__ void k_end_step(CtrlDev* ctrl, StatusDev* st, int walk_mode) {
-    if (ctrl->rebuild & DEM_HALT) return;   // a void step changes nothing
-    ctrl->steps_done += 1;
-    if (ctrl->rebuild) {
+// Counters of the finished pass become the last ones.
+__device__ __forceinline__ void rotate(StatusDev* st) {
+    st->last = st->live;
+    st->live = CountersDev{};
+}
+
+// End of a list-mode sort (one thread): the current set stays and springs are read through
+// the permutation next step. In the step loop (loop = 1) it also finishes the step whose
+// bookkeeping waited for the sort, and says whether the loop goes on.
+__global__ void k_sort_end(CtrlDev* ctrl, StatusDev* st, int loop, cudaGraphConditionalHandle inner,
+                           cudaGraphConditionalHandle outer) {
+    if (ctrl->rebuild == 1) {
         ctrl->perm_valid = 1;
         ctrl->since = 0;
         ctrl->nsorts += 1;
-    } else {
+        ctrl->sorted = 1;
+        ctrl->rebuild = 0;
+    }
+    if (!loop) return;
+    if (ctrl->stop == LOOP_SORT) {
+        ctrl->sorted = 0;
+        rotate(st);
+        ctrl->stop = ctrl->left ? LOOP_GO : LOOP_DONE;
+    }
+    unsigned int go = ctrl->stop == LOOP_GO ? 1u : 0u;
+    // every turn takes at least one step; a loop that does not is ended and reported
+    ctrl->idle = ctrl->left == ctrl->seen ? ctrl->idle + 1 : 0;
+    ctrl->seen = ctrl->left;
+    if (go && ctrl->idle > 4) {
+        raise_status(st, ST_STUCK, (int32_t)ctrl->left);
+        go = 0;
+    }
+    cudaGraphSetConditional(inner, go);
+    cudaGraphSetConditional(outer, go);
+}
+
+// Step bookkeeping outside the loop (one thread): after a sort the current set stays;
+// otherwise the next set becomes current. step = 0: the sort that follows an import.
+__global__ void k_end_step(CtrlDev* ctrl, StatusDev* st, int walk_mode, int step) {
+    if (ctrl->rebuild & DEM_HALT) return;   // a void step changes nothing
+    ctrl->steps_done += step;
+    ctrl->hcur ^= step;
+    if (walk_mode) {
+        ctrl->perm_valid = 1;
+        ctrl->since = 0;
+        ctrl->nsorts += 1;
+    } else if (!ctrl->sorted) {
         ctrl->cur ^= 1;
         ctrl->perm_valid = 0;
         ctrl->since += 1;
     }
+    ctrl->sorted = 0;
     ctrl->rebuild = walk_mode;
-    st->last = st->live;
-    st->live = CountersDev{};
+    rotate(st);
+}
+
+// The two one-thread kernels after a force pass of the step loop: what the pass decided,
+// then the bookkeeping of a step that does not sort (a step that sorts is finished by
+// k_sort_end). The loop's inner body goes on while steps are left and no sort is due.
+__global__ void k_loop_decide(CtrlDev* ctrl) {
+    if (ctrl->stop != LOOP_GO) return;
+    const int r = ctrl->rebuild;
+    ctrl->stop = (r & DEM_HALT) ? LOOP_VOID : (r == 1 ? LOOP_TOSORT : LOOP_KEEP);
+}
+__global__ void k_loop_end(CtrlDev* ctrl, StatusDev* st, cudaGraphConditionalHandle inner) {
+    const int s = ctrl->stop;
+    if (s == LOOP_KEEP || s == LOOP_TOSORT) {
+        ctrl->steps_done += 1;
+        ctrl->hcur ^= 1;
+        const uint32_t left = ctrl->left - 1;
+        ctrl->left = left;
+        if (s == LOOP_TOSORT) {
+            ctrl->cond_sorts += 1;
+            ctrl->stop = LOOP_SORT;
+        } else {
+            ctrl->cur ^= 1;
+            ctrl->perm_valid = 0;
+            ctrl->since += 1;
+            rotate(st);
+            ctrl->stop = left ? LOOP_GO : LOOP_DONE;
+        }
+    }
+    cudaGraphSetConditional(inner, ctrl->stop == LOOP_GO ? 1u : 0u);
 }
 
 // ======================================================================= set-up / read-out
@@ -829,34 +897,33 @@ cudaError_t run_rebuild(Domain& d) {
         DEM_LAUNCH_CHECK();
     } else {
         // (cell, id) positions, the window order by last contact count, the gather
-        const uint32_t* hc = d.hcnt[d.h_cur];   // contact counts of the step just finished (pre-sort order)
         const uint32_t wsz = std::min(1024u, (uint32_t)d.block * DEM_WINDOW_MULT);
         uint32_t wb = 32;
         while (wb < wsz) wb <<= 1;
         const uint32_t wg = std::max(1u, std::min(nblk(d.n, wsz), (uint32_t)std::max(d.sort_blocks, 1)));
         if (d.precision == 0)
-            k_rank_cell<PF64><<<sgrid(d, d.n), 256, 0, d.stream>>>(d.n, d.S64[0], d.S64[1], d.ctrl, d.key, d.cs,
-                                                                     d.tmp, hc, d.canon, d.rank);
+            k_rank_cell<PF64><<<sgrid(d, d.n), 256, 0, d.stream>>>(d.n, d.S64[0], d.S64[1], d.ctrl, d.key, d.cs, d.tmp,
+                                                                   d.hcnt[0], d.hcnt[1], d.canon, d.rank);
         else
-            k_rank_cell<PF32><<<sgrid(d, d.n), 256, 0, d.stream>>>(d.n, d.S32[0], d.S32[1], d.ctrl, d.key, d.cs,
-                                                                     d.tmp, hc, d.canon, d.rank);
-        DEM_LAUNCH_CHECK();
-        k_window<<<wg, wb, 0, d.stream>>>(d.n, wsz, d.d_scenes, d.nscenes, d.ctrl, d.rank, d.fin);
+            k_rank_cell<PF32><<<sgrid(d, d.n), 256, 0, d.stream>>>(d.n, d.S32[0], d.S32[1], d.ctrl, d.key, d.cs, d.tmp,
+                                                                   d.hcnt[0], d.hcnt[1], d.canon, d.rank);
         DEM_LAUNCH_CHECK();
         if (d.precision == 0)
-            k_gather<PF64><<<sgrid(d, d.n), 256, 0, d.stream>>>(d.n, d.S64[0], d.S64[1], d.ctrl, d.key, d.canon,
-                                                                  d.fin, d.perm, d.skey, d.ref);
+            k_window<PF64><<<wg, wb, 0, d.stream>>>(d.n, wsz, d.d_scenes, d.nscenes, d.S64[0], d.S64[1], d.ctrl, d.rank,
+                                                    d.key, d.canon, d.fin, d.perm, d.skey, d.ref);
         else
-            k_gather<PF32><<<sgrid(d, d.n), 256, 0, d.stream>>>(d.n, d.S32[0], d.S32[1], d.ctrl, d.key, d.canon,
-                                                                  d.fin, d.perm, d.skey, d.ref);
+            k_window<PF32><<<wg, wb, 0, d.stream>>>(d.n, wsz, d.d_scenes, d.nscenes, d.S32[0], d.S32[1], d.ctrl, d.rank,
+                                                    d.key, d.canon, d.fin, d.perm, d.skey, d.ref);
         DEM_LAUNCH_CHECK();
         cudaError_t e = run_lists(d);
         if (e != cudaSuccess) return e;
+        k_sort_end<<<1, 1, 0, d.stream>>>(d.ctrl, d.st, d.in_loop, d.loop_inner, d.loop_outer);
+        DEM_LAUNCH_CHECK();
     }
     return cudaSuccess;
 }
 
-// Sets the condition of the step graph's sort node from the device-side decision, and
+// Sets the condition of the timed step's sort node from the device-side decision, and
 // counts the sorts that run that way (one thread).
 __global__ void k_sort_cond(cudaGraphConditionalHandle h, CtrlDev* ctrl) {
     const unsigned int go = ctrl->rebuild == 1 ? 1u : 0u;
@@ -870,8 +937,16 @@ cudaError_t run_sort_cond(Domain& d, cudaGraphConditionalHandle h) {
     return cudaSuccess;
 }
 
-cudaError_t run_end_step(Domain& d) {
-    k_end_step<<<1, 1, 0, d.stream>>>(d.ctrl, d.st, d.list_mode ? 0 : 1);
+cudaError_t run_end_step(Domain& d, bool step) {
+    k_end_step<<<1, 1, 0, d.stream>>>(d.ctrl, d.st, d.list_mode ? 0 : 1, step ? 1 : 0);
+    DEM_LAUNCH_CHECK();
+    return cudaSuccess;
+}
+
+cudaError_t run_loop_end(Domain& d) {
+    k_loop_decide<<<1, 1, 0, d.stream>>>(d.ctrl);
+    DEM_LAUNCH_CHECK();
+    k_loop_end<<<1, 1, 0, d.stream>>>(d.ctrl, d.st, d.loop_inner);
     DEM_LAUNCH_CHECK();
     return cudaSuccess;
 }

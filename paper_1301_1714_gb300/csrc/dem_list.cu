@@ -46,16 +46,14 @@ struct ListArgs {
     int interval;                // sort at least every `interval` steps (0: never forced)
     const uint32_t* perm;
     const uint32_t* wmask;       // walls each particle can reach until the next sort
-    const uint32_t* hin_cnt;     // springs read
-    const uint32_t* hin_pid;
-    const T* hin_d;
-    uint32_t* hout_cnt;          // springs written
-    uint32_t* hout_pid;
-    T* hout_d;
+    uint32_t* hcnt[2];           // springs: ctrl->hcur names the buffer read, the other is written
+    uint32_t* hpid[2];
+    T* hd[2];
     StatusDev* st;
     double* dbgF;
     double* dbgT;
     int halt;                    // 1: a capacity overflow makes the step void (DEM_HALT)
+    int loop;                    // 1: a pass of the step loop, idle unless ctrl->stop says go
 };
 
 // ------------------------------------------------------------------- force pass
@@ -69,14 +67,24 @@ __global__ void __launch_bounds__(256, DEM_LIST_MIN_BLOCKS) k_list(ListArgs<PR> 
     constexpr bool TERMS = MODEL == 2;
     const unsigned full = 0xffffffffu;
     extern __shared__ uint32_t smem[];
+    if (!EVAL && a.loop && a.ctrl->stop != LOOP_GO) return;   // (written between passes only)
     // a void step (an earlier launch overflowed): nothing to do; one decision per warp
     if (!EVAL && __any_sync(full, (a.ctrl->rebuild & DEM_HALT) != 0)) return;
     const int cur = a.ctrl->cur;
     const typename PR::State A = cur ? a.S1 : a.S0;
     const typename PR::State B = cur ? a.S0 : a.S1;
     const bool pv = a.ctrl->perm_valid != 0;
-    if (!EVAL && blockIdx.x == 0 && threadIdx.x == 0 && a.interval > 0 && a.ctrl->since + 1 >= a.interval)
-        atomicOr(&a.ctrl->rebuild, 1);
+    const int hi = a.ctrl->hcur, ho = 1 - hi;
+    if (!EVAL && blockIdx.x == 0 && threadIdx.x == 0) {
+        a.ctrl->hlast = ho;
+        if (a.interval > 0 && a.ctrl->since + 1 >= a.interval) atomicOr(&a.ctrl->rebuild, 1);
+    }
+    const uint32_t* __restrict__ hin_cnt = hi ? a.hcnt[1] : a.hcnt[0];
+    const uint32_t* __restrict__ hin_pid = hi ? a.hpid[1] : a.hpid[0];
+    const T* __restrict__ hin_d = hi ? a.hd[1] : a.hd[0];
+    uint32_t* __restrict__ hout_cnt = ho ? a.hcnt[1] : a.hcnt[0];
+    uint32_t* __restrict__ hout_pid = ho ? a.hpid[1] : a.hpid[0];
+    T* __restrict__ hout_d = ho ? a.hd[1] : a.hd[0];
     const uint32_t tid = threadIdx.x, bd = blockDim.x, lane = tid & 31u;
     const uint32_t maxc = (uint32_t)a.maxc;
     uint32_t* s_oid = smem;   // [maxc][bd] partner ids of each particle's stored springs
@@ -92,31 +100,31 @@ __global__ void __launch_bounds__(256, DEM_LIST_MIN_BLOCKS) k_list(ListArgs<PR> 
     if (valid) {
         src = pv ? __ldg(&a.perm[q]) : q;
         if (live) m = min(__ldg(&a.ncnt[q]), (uint32_t)DEM_LIST_CAP);
-        if (PRACT || !S.active) cnt_old = min(__ldg(&a.hin_cnt[src]), maxc);
+        if (PRACT || !S.active) cnt_old = min(__ldg(&hin_cnt[src]), maxc);
         // the list and the stored springs stream from DRAM: start every line fill now, so
         // that the loads below do not wait for them one after another
         for (uint32_t k = 0; k < m; ++k) prefetch_l1(&a.nl[k * cap + q]);
-        for (uint32_t k = 0; k < cnt_old; ++k) prefetch_l1(&a.hin_pid[k * cap + src]);
+        for (uint32_t k = 0; k < cnt_old; ++k) prefetch_l1(&hin_pid[k * cap + src]);
         for (uint32_t k = 0; k < cnt_old; ++k)
-            for (int c = 0; c < 3; ++c) prefetch_l1(&a.hin_d[(c * (size_t)maxc + k) * cap + src]);
+            for (int c = 0; c < 3; ++c) prefetch_l1(&hin_d[(c * (size_t)maxc + k) * cap + src]);
     }
     // ---- phase 1: list entries that pass the prefilter
     uint64_t near_mask = 0;
     if (live) near_mask = PR::scan_list(A, PR::load(A, q), S, a.nl, m, cap, q);
-    for (uint32_t k = 0; k < cnt_old; ++k) s_oid[k * bd + tid] = __ldg(&a.hin_pid[k * cap + src]);
+    for (uint32_t k = 0; k < cnt_old; ++k) s_oid[k * bd + tid] = __ldg(&hin_pid[k * cap + src]);
     __syncwarp();
     if (valid && !live) {
         // frozen scene: carry state and springs unchanged
         if (!EVAL) {
             PR::store(B, q, PR::load(A, q));
             for (uint32_t k = 0; k < cnt_old; ++k) {
-                a.hout_pid[k * cap + q] = s_oid[k * bd + tid];
+                hout_pid[k * cap + q] = s_oid[k * bd + tid];
                 for (int c = 0; c < 3; ++c)
-                    a.hout_d[(c * (size_t)maxc + k) * cap + q] = a.hin_d[(c * (size_t)maxc + k) * cap + src];
+                    hout_d[(c * (size_t)maxc + k) * cap + q] = hin_d[(c * (size_t)maxc + k) * cap + src];
             }
-            a.hout_cnt[q] = cnt_old;
+            hout_cnt[q] = cnt_old;
         } else {
-            a.hout_cnt[q] = 0;
+            hout_cnt[q] = 0;
         }
     }
     // ---- phase 2: the lanes of a warp in lockstep over their near candidates
@@ -155,21 +163,21 @@ __global__ void __launch_bounds__(256, DEM_LIST_MIN_BLOCKS) k_list(ListArgs<PR> 
                 const T mj = PR::mass(S, rj);
                 const T meff = law_div(mi * mj, mi + mj);
                 const T Reff = law_div(ri * rjT, ri + rjT);
-                const V3<T> dold = find_spring(s_oid, bd, tid, cnt_old, gid, a.hin_d, (size_t)maxc, cap, src);
+                const V3<T> dold = find_spring(s_oid, bd, tid, cnt_old, gid, hin_d, (size_t)maxc, cap, src);
                 V3<T> Fc, Ftc, dnew, Mr;
                 law_practical<TERMS>(L, n, delta, v, rw, Reff, meff, dold, Fc, Ftc, dnew, me.w - wj, Mr);
                 F = F + Fc;
                 Tq = Tq + cross(n, Ftc) * ri;
                 if (TERMS) Tq = Tq + Mr;
                 if (nnew < maxc) {
-                    a.hout_pid[nnew * cap + q] = gid;
-                    a.hout_d[(0 * (size_t)maxc + nnew) * cap + q] = dnew.x;
-                    a.hout_d[(1 * (size_t)maxc + nnew) * cap + q] = dnew.y;
-                    a.hout_d[(2 * (size_t)maxc + nnew) * cap + q] = dnew.z;
+                    hout_pid[nnew * cap + q] = gid;
+                    hout_d[(0 * (size_t)maxc + nnew) * cap + q] = dnew.x;
+                    hout_d[(1 * (size_t)maxc + nnew) * cap + q] = dnew.y;
+                    hout_d[(2 * (size_t)maxc + nnew) * cap + q] = dnew.z;
                 }
             } else {
                 F = F + law_simple(L, n, delta, v);
-                if (EVAL && nnew < maxc) a.hout_pid[nnew * cap + q] = gid;
+                if (EVAL && nnew < maxc) hout_pid[nnew * cap + q] = gid;
             }
             ++nnew;
             ++c_pp;
@@ -191,21 +199,21 @@ __global__ void __launch_bounds__(256, DEM_LIST_MIN_BLOCKS) k_list(ListArgs<PR> 
             const uint32_t gid = DEM_WALL_BASE + (uint32_t)w;
             if (PRACT) {
                 const V3<T> rw = me.w * ri;
-                const V3<T> dold = find_spring(s_oid, bd, tid, cnt_old, gid, a.hin_d, (size_t)maxc, cap, src);
+                const V3<T> dold = find_spring(s_oid, bd, tid, cnt_old, gid, hin_d, (size_t)maxc, cap, src);
                 V3<T> Fc, Ftc, dnew, Mr;
                 law_practical<TERMS>(L, n, delta, v, rw, ri, mi, dold, Fc, Ftc, dnew, me.w - PR::wall_omega(W), Mr);
                 F = F + Fc;
                 Tq = Tq + cross(n, Ftc) * ri;
                 if (TERMS) Tq = Tq + Mr;
                 if (nnew < maxc) {
-                    a.hout_pid[nnew * cap + q] = gid;
-                    a.hout_d[(0 * (size_t)maxc + nnew) * cap + q] = dnew.x;
-                    a.hout_d[(1 * (size_t)maxc + nnew) * cap + q] = dnew.y;
-                    a.hout_d[(2 * (size_t)maxc + nnew) * cap + q] = dnew.z;
+                    hout_pid[nnew * cap + q] = gid;
+                    hout_d[(0 * (size_t)maxc + nnew) * cap + q] = dnew.x;
+                    hout_d[(1 * (size_t)maxc + nnew) * cap + q] = dnew.y;
+                    hout_d[(2 * (size_t)maxc + nnew) * cap + q] = dnew.z;
                 }
             } else {
                 F = F + law_simple(L, n, delta, v);
-                if (EVAL && nnew < maxc) a.hout_pid[nnew * cap + q] = gid;
+                if (EVAL && nnew < maxc) hout_pid[nnew * cap + q] = gid;
             }
             ++nnew;
             ++c_wc;
@@ -216,7 +224,7 @@ __global__ void __launch_bounds__(256, DEM_LIST_MIN_BLOCKS) k_list(ListArgs<PR> 
             if (!EVAL && a.halt) atomicOr(&a.ctrl->rebuild, DEM_HALT);
         }
         c_nnew = nnew;
-        if (PRACT || EVAL) a.hout_cnt[q] = min(nnew, maxc);
+        if (PRACT || EVAL) hout_cnt[q] = min(nnew, maxc);
         // gravity, once per particle
         {
             const T gx = sizeof(T) == 8 ? (T)S.g[0] : (T)S.g_f[0];
@@ -289,17 +297,16 @@ static cudaError_t force_list_impl(Domain& d, const typename PR::State& S0, cons
     a.interval = d.interval;
     a.perm = d.perm;
     a.wmask = d.wmask;
-    const int hi = d.h_cur, ho = 1 - d.h_cur;
-    a.hin_cnt = d.hcnt[hi];
-    a.hin_pid = d.hpid[hi];
-    a.hin_d = (const T*)d.hd[hi];
-    a.hout_cnt = d.hcnt[ho];
-    a.hout_pid = d.hpid[ho];
-    a.hout_d = (T*)d.hd[ho];
+    for (int k = 0; k < 2; ++k) {
+        a.hcnt[k] = d.hcnt[k];
+        a.hpid[k] = d.hpid[k];
+        a.hd[k] = (T*)d.hd[k];
+    }
     a.st = d.st;
     a.dbgF = dbgF;
     a.dbgT = dbgT;
     a.halt = d.regrow;
+    a.loop = d.in_loop;
     const uint32_t b = (uint32_t)d.block;
     const size_t smem = (size_t)d.maxc * b * sizeof(uint32_t);
     const int model = d.model != 0 ? 1 : (d.terms != 0 ? 2 : 0);
