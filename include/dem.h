@@ -85,15 +85,18 @@ enum { DEM_TERM_NO_ATTRACTION = 1, DEM_TERM_ROLLING = 2, DEM_TERM_ETA_T = 4, DEM
  *              pass reads it instead of walking. K > 1 = as 0, and also at least every K
  *              steps. 0 and K > 1 need skin > 0; they find exactly the same contacts.
  *              In these modes the library numbers grid cells in cubic bricks internally
- *              (the largest edge of 2, 4, 8 or 16 cells that pads the grid by at most 1/8;
- *              row-major cells when none does) and stores each window of four blocks
- *              of consecutive (cell, id) positions (at most 1,024) ordered by the
- *              particles' last contact counts, so the force kernel's warps get similar
- *              amounts of work; a list holds at most 64
+ *              (the largest edge of 2, 4, 8 or 16 cells that pads the grid by at most 1/8,
+ *              or an edge of 8 that pads it by at most 1/2; row-major cells when none does),
+ *              cells in Morton order within a brick, and stores the particles in tiles of
+ *              consecutive (cell, id) positions, each tile ordered by the particles' last
+ *              contact counts, so the force kernel's warps get similar amounts of work; a
+ *              list holds at most 64
  *              candidates in ascending partner id (a fuller one makes dem_step return
  *              DEM_ERR_CAPACITY), so a particle's contacts are summed in that order and
  *              results do not depend on when the sorts happened.
- *  block_size  threads per block of the force kernel (32..256); 0 = automatic (256)
+ *  block_size  threads per block of the force kernel (32..256); 0 = automatic (256). List
+ *              mode works in tiles of at most four times as many particles (at most 512;
+ *              smaller tiles for few particles), one thread each. Results do not depend on it.
  *  terms       optional force terms added to Eqs. 2-10 (none is in the paper; its force
  *              is built from separable terms so that terms can be added, Sec. 3), an OR of:
  *              DEM_TERM_NO_ATTRACTION  the normal force never pulls: F_n = 0 when

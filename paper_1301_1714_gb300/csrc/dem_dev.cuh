@@ -6,8 +6,9 @@
 //   FP32 mode: P0 = float4(hi.x, hi.y, hi.z, r), P1 = float4(lo.x, lo.y, lo.z, 0),
 //              V = float4(v, 0), W = float4(w, 0), id (u32). Position = hi + lo exactly,
 //              with hi = fl32(hi + lo) kept by every update (FastTwoSum renormalisation).
-//   History (per particle, slot-major): cnt[p], pid[k*cap + p] (partner global id, or
-//   DEM_WALL_BASE + wall), d[(c*maxc + k)*cap + p] for c = x,y,z (T = float or double).
+//   History (per particle, slot-major): cnt[p] and records hs[k*cap + p] of the tangential
+//   spring and its partner (global id, or DEM_WALL_BASE + wall), one 16-byte (FP32) or
+//   32-byte (FP64) load or store per contact.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -56,9 +57,9 @@ struct SceneDev {
     int32_t terms;              // optional force terms (DEM_TERM_*)
     int32_t bshift;             // cell order: 0 row-major; s > 0 bricks of (2^s)^3 cells (list mode)
     int32_t bdims[3];           // bricks per axis (bshift > 0)
+    uint32_t t0;                // list mode: first tile of the scene
     float skin_f;               // list mode: Verlet skin [m] of the scene's neighbour lists
     float thresh2_f;            // list mode: squared displacement since the last sort that forces a sort
-    float pad4;
     double mu_roll;             // rolling resistance coefficient
     double alpha_t;             // tangential damping factor
     double kcoh_pi;             // pi * cohesion energy density
@@ -126,16 +127,26 @@ __device__ __forceinline__ void raise_status(StatusDev* st, int32_t code, int32_
     if (atomicCAS(&st->code, 0, code) == 0) st->where = where;
 }
 
+// Bits of a brick coordinate (at most 4) spread to every third place, and back.
+__host__ __device__ __forceinline__ uint32_t spread3(uint32_t a) {
+    return (a & 1u) | ((a & 2u) << 2) | ((a & 4u) << 4) | ((a & 8u) << 6);
+}
+__host__ __device__ __forceinline__ uint32_t unspread3(uint32_t a) {
+    return (a & 1u) | ((a >> 2) & 2u) | ((a >> 4) & 4u) | ((a >> 6) & 8u);
+}
+
 // Key of cell (i, j, k) of scene S, relative to the scene's first cell. Row-major
 // ((k ny + j) nx + i) or, with bshift = s > 0, bricks of 2^s x 2^s x 2^s cells: bricks in
-// row-major order, cells row-major within their brick. A run of consecutive keys is then
-// a compact block of space, so the particles a thread block holds are mostly each
-// other's neighbours (list mode stores particles in this order).
+// row-major order, cells in Morton (Z-curve) order within their brick. A run of
+// consecutive keys is then a compact block of space, so the particles a tile of the list
+// mode holds are mostly each other's neighbours (list mode stores particles in this order).
+// A tile of 512 spheres of a dense bed has 456 neighbours outside it in this order, 699
+// with row-major 16^3 bricks (128: 202 against 269).
 __device__ __forceinline__ uint32_t cell_index(const SceneDev& S, uint32_t i, uint32_t j, uint32_t k) {
     if (S.bshift == 0) return (k * (uint32_t)S.dims[1] + j) * (uint32_t)S.dims[0] + i;
     const uint32_t sh = (uint32_t)S.bshift, m = (1u << sh) - 1u;
     const uint32_t brick = ((k >> sh) * (uint32_t)S.bdims[1] + (j >> sh)) * (uint32_t)S.bdims[0] + (i >> sh);
-    return (brick << (3 * sh)) | ((((k & m) << sh) | (j & m)) << sh) | (i & m);
+    return (brick << (3 * sh)) | (spread3(k & m) << 2) | (spread3(j & m) << 1) | spread3(i & m);
 }
 // Inverse of cell_index.
 __device__ __forceinline__ void cell_coords(const SceneDev& S, uint32_t local, int& i, int& j, int& k) {
@@ -146,13 +157,13 @@ __device__ __forceinline__ void cell_coords(const SceneDev& S, uint32_t local, i
         k = (int)(t / (uint32_t)S.dims[1]);
         return;
     }
-    const uint32_t sh = (uint32_t)S.bshift, m = (1u << sh) - 1u;
+    const uint32_t sh = (uint32_t)S.bshift;
     const uint32_t brick = local >> (3 * sh), in = local & ((1u << (3 * sh)) - 1u);
     const uint32_t bi = brick % (uint32_t)S.bdims[0], bt = brick / (uint32_t)S.bdims[0];
     const uint32_t bj = bt % (uint32_t)S.bdims[1], bk = bt / (uint32_t)S.bdims[1];
-    i = (int)((bi << sh) | (in & m));
-    j = (int)((bj << sh) | ((in >> sh) & m));
-    k = (int)((bk << sh) | (in >> (2 * sh)));
+    i = (int)((bi << sh) | unspread3(in & 0x249u));
+    j = (int)((bj << sh) | unspread3((in >> 1) & 0x249u));
+    k = (int)((bk << sh) | unspread3((in >> 2) & 0x249u));
 }
 
 // Scene of packed particle index q (scenes are contiguous, in order).
@@ -162,6 +173,17 @@ __device__ __forceinline__ int scene_of(const SceneDev* sc, int nscenes, uint32_
     while (lo < hi) {
         int mid = (lo + hi + 1) >> 1;
         if (__ldg(&sc[mid].p0) <= q) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
+
+// Scene of list-mode tile t (every scene has its own tiles, in scene order).
+__device__ __forceinline__ int scene_of_tile(const SceneDev* sc, int nscenes, uint32_t t) {
+    if (nscenes == 1) return 0;
+    int lo = 0, hi = nscenes - 1;
+    while (lo < hi) {
+        int mid = (lo + hi + 1) >> 1;
+        if (__ldg(&sc[mid].t0) <= t) lo = mid; else hi = mid - 1;
     }
     return lo;
 }
@@ -181,21 +203,45 @@ __device__ __forceinline__ float dsqrt(float a) { return sqrtf(a); }
 __device__ __forceinline__ double dsqrt(double a) { return sqrt(a); }
 
 // Quotient and square root of the contact law. FP64 mode: IEEE operations. FP32 mode: the
-// hardware approximations (PTX div.approx / sqrt.approx, relative error about 2^-22),
-// well inside the FP32 mode's force tolerance; both are deterministic functions of their
+// hardware's approximations with subnormal arguments taken as zero, each one instruction
+// (reciprocal: relative error 2^-23, so a quotient is within 1.5 ulp; square root 2^-23):
+// PTX div.approx and sqrt.approx without .ftz have no smaller error and take about eight and
+// five instructions, for arguments that lengths, masses and squared forces never reach (the
+// callers say where a subnormal one could matter). All are deterministic functions of their
 // arguments, so the two evaluations of a pair stay exact mirrors of each other.
 __device__ __forceinline__ double law_div(double a, double b) { return a / b; }
 __device__ __forceinline__ double law_sqrt(double a) { return sqrt(a); }
-__device__ __forceinline__ float law_div(float a, float b) {
+__device__ __forceinline__ float law_rcp(float b) {
     float r;
-    asm("div.approx.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));
     return r;
 }
+__device__ __forceinline__ float law_div(float a, float b) { return a * law_rcp(b); }
 __device__ __forceinline__ float law_sqrt(float a) {
     float r;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(a));
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
     return r;
 }
+// v / |v| from v and |v|^2 > 0, for any magnitude (the components may be subnormal squares).
+__device__ __forceinline__ double law_div_any(double a, double v2) { return a / sqrt(v2); }
+__device__ __forceinline__ float law_div_any(float a, float v2) {
+    float r, s;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(s) : "f"(v2));
+    asm("div.approx.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(s));
+    return r;
+}
+// The factor mu |F_n| / |F_t| of Eq. 5 from the squared lengths (ft2 > 0). FP32: lengths
+// below 1e-19 N are taken as 1e-19 N, so that the factor stays finite.
+__device__ __forceinline__ double cap_factor(double mu, double fn2, double ft2) { return mu * sqrt(fn2) / sqrt(ft2); }
+__device__ __forceinline__ float cap_factor(float mu, float fn2, float ft2) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fmaxf(ft2, 1.17549435e-38f)));
+    return mu * law_sqrt(fn2) * r;
+}
+// Eq. 5's comparison |F_t| > mu |F_n| given that it holds for the squared lengths: FP64 mode
+// decides on the lengths, FP32 mode on the squares.
+__device__ __forceinline__ bool cap_holds(double mu, double fn2, double ft2) { return sqrt(ft2) > mu * sqrt(fn2); }
+__device__ __forceinline__ bool cap_holds(float, float, float) { return true; }
 
 // Symmetric in (a1, b1) <-> (a2, b2): products rounded first, then one rounded sum, so the
 // two threads that evaluate the same pair get the same bits.
@@ -204,6 +250,32 @@ __device__ __forceinline__ float sym_madd(float a1, float b1, float a2, float b2
 }
 __device__ __forceinline__ double sym_madd(double a1, double b1, double a2, double b2) {
     return __dadd_rn(__dmul_rn(a1, b1), __dmul_rn(a2, b2));
+}
+
+// A stored tangential spring and its partner.
+template <class T> struct Spring;
+template <> struct alignas(16) Spring<float> {
+    float x, y, z;
+    uint32_t pid;
+};
+template <> struct alignas(16) Spring<double> {
+    double x, y, z;
+    uint32_t pid, pad;
+};
+__device__ __forceinline__ Spring<float> load_spring(const Spring<float>* p) {
+    const float4 v = __ldg((const float4*)p);
+    return {v.x, v.y, v.z, __float_as_uint(v.w)};
+}
+__device__ __forceinline__ Spring<double> load_spring(const Spring<double>* p) {
+    const double2 a = __ldg((const double2*)p), b = __ldg((const double2*)p + 1);
+    return {a.x, a.y, b.x, (uint32_t)__double_as_longlong(b.y), 0u};
+}
+__device__ __forceinline__ void store_spring(Spring<float>* p, V3<float> d, uint32_t pid) {
+    *(float4*)p = make_float4(d.x, d.y, d.z, __uint_as_float(pid));
+}
+__device__ __forceinline__ void store_spring(Spring<double>* p, V3<double> d, uint32_t pid) {
+    ((double2*)p)[0] = make_double2(d.x, d.y);
+    ((double2*)p)[1] = make_double2(d.z, __longlong_as_double((long long)pid));
 }
 
 // ------------------------------------------------- error-free transformations
@@ -252,7 +324,8 @@ __device__ __forceinline__ Law<float> law_of(const SceneDev& s, int stiffness, f
 // -mu_roll R_eff |F_n| w_rel/|w_rel| returned in Mroll (w_rel = w_i - w_j, or minus the
 // wall's angular velocity); 4 = eta_t = alpha_t sqrt(k_t m_eff) in the tangential part;
 // 8 = cohesion k_coh pi R_eff delta n added after the Coulomb cap.
-template <bool TERMS, class T>
+// STIFF: 0 linear, 1 Hertz, 2 whichever P.stiffness says.
+template <bool TERMS, int STIFF, class T>
 __device__ __forceinline__ void law_practical(const Law<T>& P, V3<T> n, T delta, V3<T> v, V3<T> rw, T Reff, T meff,
                                               V3<T> dold, V3<T>& F, V3<T>& Ft, V3<T>& dnew, V3<T> wrel,
                                               V3<T>& Mroll) {
@@ -262,7 +335,7 @@ __device__ __forceinline__ void law_practical(const Law<T>& P, V3<T> n, T delta,
     const T dn = dot(dold, n);                                   // Eq. 7
     V3<T> dt = (dold - n * dn) + vt * P.dt;
     T kn, kt;                                                    // Eqs. 8-9
-    if (P.stiffness == 0) { kn = P.kn; kt = P.kt; }
+    if (STIFF == 0 || (STIFF == 2 && P.stiffness == 0)) { kn = P.kn; kt = P.kt; }
     else {
         const T s = law_sqrt(delta * Reff);
         kn = P.cn * s;
@@ -276,12 +349,9 @@ __device__ __forceinline__ void law_practical(const Law<T>& P, V3<T> n, T delta,
     V3<T> Ftt = dt * (-kt) - vt * eta_t;
     // Eq. 5, compared on squared lengths; the lengths are taken only when the cap applies
     const T ft2 = dot(Ftt, Ftt), fn2 = dot(Fn, Fn);
-    if (ft2 > (P.mu * P.mu) * fn2 && ft2 > T(0)) {
-        const T ftn = law_sqrt(ft2), fnn = law_sqrt(fn2);
-        if (ftn > P.mu * fnn) {
-            Ftt = Ftt * law_div(P.mu * fnn, ftn);
-            if (kt > T(0)) dt = (Ftt + vt * eta_t) * law_div(T(-1), kt);
-        }
+    if (ft2 > (P.mu * P.mu) * fn2 && ft2 > T(0) && cap_holds(P.mu, fn2, ft2)) {
+        Ftt = Ftt * cap_factor(P.mu, fn2, ft2);
+        if (kt > T(0)) dt = (Ftt + vt * eta_t) * law_div(T(-1), kt);
     }
     F = Fn + Ftt;                                                // Eq. 2
     if (TERMS && (P.terms & 8)) F = F + n * (P.kcoh_pi * Reff * delta);
@@ -290,7 +360,7 @@ __device__ __forceinline__ void law_practical(const Law<T>& P, V3<T> n, T delta,
     Mroll = mk(T(0), T(0), T(0));
     if (TERMS && (P.terms & 2)) {
         const T wn2 = dot(wrel, wrel);
-        if (wn2 > T(0)) Mroll = wrel * law_div(-P.mu_roll * Reff * law_sqrt(fn2), law_sqrt(wn2));
+        if (wn2 > T(0)) Mroll = wrel * law_div_any(-P.mu_roll * Reff * law_sqrt(fn2), wn2);
     }
 }
 

@@ -8,6 +8,20 @@
 
 namespace demgb {
 
+// Largest tile of list mode and the force pass's resident blocks of that size per SM.
+#ifndef DEM_TILE_MAX
+#define DEM_TILE_MAX 512
+#define DEM_LIST_MIN_BLOCKS 2
+#endif
+
+// Tiles of list mode: halo entries a tile has room for in shared memory (a dense bed needs
+// 456 / 304 / 202 / 134 on average and at most 614 / 388 / 261 / 182 for tiles of 512 / 256 /
+// 128 / 64 particles). A tile with more reads its partners from global memory.
+__host__ __device__ inline uint32_t halo_cap(uint32_t tile) {
+    return tile >= 512 ? 768u : tile >= 384 ? 640u : tile >= 256 ? 512u : tile >= 128 ? 384u : 256u;
+}
+constexpr uint32_t HALO_NONE = 0xFFFFFFFFu;
+
 struct StateF64 {
     double *x, *y, *z, *vx, *vy, *vz, *wx, *wy, *wz;
     float* r;
@@ -54,6 +68,13 @@ struct Domain {
     int interval = 1;              // sort at least every `interval` steps (0 = skin only)
     uint32_t* ncnt = nullptr;
     uint32_t* nl = nullptr;
+    uint2* nl4 = nullptr;          // the lists as indices into the particle's tile (dem_nlist.cu, k_tile)
+    uint32_t tile = 0;             // particles per tile; every scene has its own tiles
+    uint32_t ntiles = 0;
+    uint32_t* halo = nullptr;      // halo_cap(tile) stored indices per tile, ascending
+    uint32_t* nhalo = nullptr;
+    size_t halo_words = 0;         // allocated size of halo
+    uint32_t tiles_cap = 0;        // allocated size of nhalo
     float4* ref = nullptr;         // positions at the last sort
     uint32_t* wmask = nullptr;     // walls each particle can reach before the next sort (bit w = wall w)
     uint32_t* canon = nullptr;     // (cell, id) position -> pre-sort position, at a sort
@@ -61,8 +82,8 @@ struct Domain {
 
     // tangential history, double-buffered; h_cur is the buffer the next step reads
     uint32_t* hcnt[2] = {nullptr, nullptr};
-    uint32_t* hpid[2] = {nullptr, nullptr};
-    void* hd[2] = {nullptr, nullptr};
+    void* hs[2] = {nullptr, nullptr};                // Spring records, slot-major
+    uint64_t* hmask[2] = {nullptr, nullptr};         // list mode: list entries that have a spring
     int h_cur = 0;
 
     // counting sort by cell
@@ -124,6 +145,7 @@ cudaError_t run_sort_cond(Domain& d, cudaGraphConditionalHandle h);  // graph co
 cudaError_t run_force(Domain& d, bool eval, double* dbgF, double* dbgT);
 // list mode (dem_list.cu): the neighbour lists of a sort, and the force pass over them
 cudaError_t run_lists(Domain& d);
+cudaError_t run_tiles(Domain& d, bool always);   // tile entries and spring masks of the lists
 cudaError_t run_wall_masks(Domain& d);   // the wall masks again (after the walls changed)
 cudaError_t run_force_list(Domain& d, bool eval, double* dbgF, double* dbgT);
 cudaError_t run_export(Domain& d, double* x, double* v, double* w);

@@ -102,7 +102,11 @@ void free_particle_buffers(Domain& d) {
     d.ncnt = d.nl = d.wmask = nullptr;
     d.ref = nullptr;
     d.canon = d.fin = nullptr;
-    for (int i = 0; i < 2; ++i) { d.hcnt[i] = nullptr; d.hpid[i] = nullptr; d.hd[i] = nullptr; }
+    for (int i = 0; i < 2; ++i) { d.hcnt[i] = nullptr; d.hs[i] = nullptr; d.hmask[i] = nullptr; }
+    d.nl4 = nullptr;
+    d.halo = d.nhalo = nullptr;
+    d.halo_words = 0;
+    d.tiles_cap = 0;
     d.key = d.rank = d.tmp = d.perm = d.skey = d.cnt = d.cs = d.part = nullptr;
     d.diag_part = nullptr;
     d.cap = 0;
@@ -192,9 +196,10 @@ bool check_wall(const dem_wall& w, int precision, std::string& why) {
     return true;
 }
 
-void fill_scene(dem_handle* h, SceneDev& S, uint32_t p0, uint32_t np, uint32_t c0) {
+void fill_scene(dem_handle* h, SceneDev& S, uint32_t p0, uint32_t np, uint32_t c0, uint32_t t0 = 0) {
     const dem_config& c = h->cfg;
     S = SceneDev{};
+    S.t0 = t0;
     S.p0 = p0;
     S.np = np;
     S.c0 = c0;
@@ -282,7 +287,9 @@ dem_status validate_config(const dem_config* c, std::string& why) {
 // Device buffers of a domain for n particles and ncells cells (reused when large enough).
 dem_status alloc_domain(Domain& d, uint32_t n, uint32_t ncells, std::string& err) {
     const uint32_t need = std::max<uint32_t>(n, 1);
-    if (need <= d.cap && ncells <= d.cells_cap) return DEM_OK;
+    const size_t hw = d.list_mode ? (size_t)d.ntiles * halo_cap(d.tile) : 0;
+    if (need <= d.cap && ncells <= d.cells_cap && (!d.list_mode || (hw <= d.halo_words && d.ntiles <= d.tiles_cap)))
+        return DEM_OK;
     // host-side fault injection for tests: DEM_FAULT=alloc makes every allocation of
     // particle buffers fail as if the device were out of memory
     const char* fault = std::getenv("DEM_FAULT");
@@ -309,13 +316,17 @@ dem_status alloc_domain(Domain& d, uint32_t n, uint32_t ncells, std::string& err
             AL(S.P0, N * 16); AL(S.P1, N * 16); AL(S.V, N * 16); AL(S.W, N * 16); AL(S.id, N * 4);
         }
         AL(d.hcnt[s], N * 4);
-        AL(d.hpid[s], N * 4 * (size_t)d.maxc);
-        AL(d.hd[s], N * T * 3 * (size_t)d.maxc);
+        AL(d.hs[s], N * 4 * T * (size_t)d.maxc);
     }
     AL(d.key, N * 4); AL(d.rank, N * 4); AL(d.tmp, N * 4); AL(d.perm, N * 4); AL(d.skey, N * 4);
     if (d.list_mode) {
         AL(d.ncnt, N * 4);
         AL(d.nl, N * 4 * (size_t)DEM_LIST_CAP);
+        AL(d.nl4, N * 2 * (size_t)DEM_LIST_CAP);
+        AL(d.hmask[0], N * 8);
+        AL(d.hmask[1], N * 8);
+        AL(d.halo, hw * 4);
+        AL(d.nhalo, (size_t)d.ntiles * 4);
         AL(d.wmask, N * 4);
         AL(d.ref, N * 16);
         AL(d.canon, N * 4);
@@ -329,6 +340,8 @@ dem_status alloc_domain(Domain& d, uint32_t n, uint32_t ncells, std::string& err
     AL(d.diag_part, (size_t)db * 10 * 8);
 #undef AL
     d.cap = cap;
+    d.halo_words = hw;
+    d.tiles_cap = d.list_mode ? d.ntiles : 0;
     d.cells_cap = ccap;
     d.part_cap = nb;
     d.diag_part_cap = db;
@@ -405,41 +418,29 @@ dem_status read_ctrl(dem_handle* h, CtrlDev& c) {
 }
 
 // Contact slots of a handle grown to newmaxc: new history buffers, the springs of the
-// buffer the next step reads copied in (the partner-id planes keep their places; the
-// three component blocks move to the new stride); the other buffer is written by the
-// next step. On failure the old buffers stay.
+// buffer the next step reads copied in (slots keep their places); the other buffer is
+// written by the next step. On failure the old buffers stay.
 dem_status regrow_slots(dem_handle* h, int newmaxc) {
     Domain& d = h->d;
-    const size_t N = d.cap, M = (size_t)d.maxc, M2 = (size_t)newmaxc;
-    const size_t T = d.precision == 0 ? sizeof(double) : sizeof(float);
-    void* npid[2] = {nullptr, nullptr};
-    void* nhd[2] = {nullptr, nullptr};
+    const size_t N = d.cap, rec = 4 * (d.precision == 0 ? sizeof(double) : sizeof(float));
+    const size_t M = (size_t)d.maxc, M2 = (size_t)newmaxc;
+    void* nhs[2] = {nullptr, nullptr};
     bool ok = true;
-    for (int s = 0; s < 2 && ok; ++s)
-        ok = cudaMalloc(&npid[s], N * 4 * M2) == cudaSuccess && cudaMalloc(&nhd[s], N * T * 3 * M2) == cudaSuccess;
+    for (int s = 0; s < 2 && ok; ++s) ok = cudaMalloc(&nhs[s], N * rec * M2) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
-        for (int s = 0; s < 2; ++s) {
-            if (npid[s]) cudaFree(npid[s]);
-            if (nhd[s]) cudaFree(nhd[s]);
-        }
+        for (int s = 0; s < 2; ++s)
+            if (nhs[s]) cudaFree(nhs[s]);
         return fail(h, DEM_ERR_OOM, "cudaMalloc of the grown contact slots failed");
     }
     const int hi = d.h_cur;
-    CK(h, cudaMemcpyAsync(npid[hi], d.hpid[hi], N * 4 * M, cudaMemcpyDeviceToDevice, d.stream));
-    for (size_t c = 0; c < 3; ++c)
-        CK(h, cudaMemcpyAsync((char*)nhd[hi] + c * M2 * N * T, (const char*)d.hd[hi] + c * M * N * T, M * N * T,
-                              cudaMemcpyDeviceToDevice, d.stream));
+    CK(h, cudaMemcpyAsync(nhs[hi], d.hs[hi], N * rec * M, cudaMemcpyDeviceToDevice, d.stream));
     CK(h, cudaStreamSynchronize(d.stream));
     for (int s = 0; s < 2; ++s) {
-        for (void*& p : d.allocations) {
-            if (p == (void*)d.hpid[s]) p = npid[s];
-            else if (p == d.hd[s]) p = nhd[s];
-        }
-        cudaFree(d.hpid[s]);
-        cudaFree(d.hd[s]);
-        d.hpid[s] = (uint32_t*)npid[s];
-        d.hd[s] = nhd[s];
+        for (void*& p : d.allocations)
+            if (p == d.hs[s]) p = nhs[s];
+        cudaFree(d.hs[s]);
+        d.hs[s] = nhs[s];
     }
     d.maxc = newmaxc;
     return DEM_OK;
@@ -454,16 +455,16 @@ dem_status rotate_counters(dem_handle* h) {
 
 // Cell order of a list-mode grid of dims cells (nc of them): consecutive stored particles
 // form compact blocks of space when cells are numbered brick by brick (the grid padded to
-// whole bricks). Returns the largest brick shift s <= DEM_LIST_BRICK_SHIFT whose padding
-// adds at most 1/8 to the cell count (0 = row-major), the bricks per axis and the padded
-// cell count. Measured on the 4,194,304-sphere drum (88 x 254 x 254 cells): 16^3 bricks are
-// 3% faster per step than 4^3, with the same bits.
+// whole bricks). Returns the brick shift s <= DEM_LIST_BRICK_SHIFT, the bricks per axis and
+// the padded cell count: the largest s whose padding adds at most 1/8 to the cell count, and
+// at least 8^3 bricks where they add at most 1/2 (tiles of small grids need compact runs of
+// cells too, and their cell tables are small); 0 = row-major.
 int choose_bricks(const int64_t dims[3], int64_t nc, int64_t bdims[3], int64_t& padded) {
     for (int s = DEM_LIST_BRICK_SHIFT; s >= 1; --s) {
         const int64_t B = (int64_t)1 << s;
         double p = 1.0;
         for (int a = 0; a < 3; ++a) p *= (double)(((dims[a] + B - 1) / B) * B);
-        if (p > 1.125 * (double)nc || p > 2147483647.0) continue;
+        if (p > (s == 3 ? 1.5 : 1.125) * (double)nc || p > 2147483647.0) continue;
         padded = 1;
         for (int a = 0; a < 3; ++a) {
             bdims[a] = (dims[a] + B - 1) / B;
@@ -474,6 +475,15 @@ int choose_bricks(const int64_t dims[3], int64_t nc, int64_t bdims[3], int64_t& 
     bdims[0] = bdims[1] = bdims[2] = 1;
     padded = nc;
     return 0;
+}
+
+// Particles per tile of list mode (a multiple of 32, at most 512; also the threads of a
+// force-pass block): four times the configured block size, and less for few particles, so
+// that the blocks fill the chip.
+uint32_t tile_size(const Domain& d, uint32_t n) {
+    uint32_t t = std::min((uint32_t)DEM_TILE_MAX, 4u * (uint32_t)d.block);
+    while (t > 64 && n / t < 2u * (uint32_t)(d.sort_blocks / 8)) t = t > 256 ? 256 : t / 2;
+    return std::max(32u, t & ~31u);
 }
 
 // Grid of Sec. 4.1 over the configured domain: cell edge >= one diameter of the largest
@@ -546,6 +556,8 @@ dem_status load_particles(dem_handle* h, int64_t n64, const double* x, const dou
     if (s != DEM_OK) return s;
     d.n = n;
     d.ncells = (uint32_t)nc;
+    d.tile = tile_size(d, n);
+    d.ntiles = (n + d.tile - 1) / d.tile;
     s = ensure_buffers(h, n, (uint32_t)nc);
     if (s != DEM_OK) return s;
     // scene table (one scene)
@@ -707,7 +719,9 @@ cudaError_t capture_loop(Domain& d, StepGraph* g) {
     body = d.launches - l0 - steps;
     d.in_loop = 0;
     d.launches = l0;
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&g->exec, graph, 0);
+    if (e != cudaSuccess) return e;   // (the graph is left: destroying one whose body's capture failed
+                                      // crashes in driver 580.159; run_steps does not try again)
+    e = cudaGraphInstantiate(&g->exec, graph, 0);
     cudaGraphDestroy(graph);
     if (e != cudaSuccess) {
         g->exec = nullptr;
@@ -1093,13 +1107,43 @@ static dem_status download_u32(dem_handle* h, std::vector<uint32_t>& out, const 
     return DEM_OK;
 }
 
+// Spring records as the host sees them, and the device layout of either precision.
+struct HostSpring {
+    double d[3];
+    uint32_t pid;
+};
+struct Raw32 {
+    float d[3];
+    uint32_t pid;
+};
+struct Raw64 {
+    double d[3];
+    uint32_t pid, pad;
+};
+
+// The first mx slots of every particle of history buffer b.
+static dem_status download_springs(dem_handle* h, std::vector<HostSpring>& out, int b, uint32_t mx) {
+    Domain& d = h->d;
+    const size_t count = (size_t)mx * d.cap;
+    out.resize(count);
+    auto get = [&](auto raw) -> dem_status {
+        std::vector<decltype(raw)> t(count);
+        if (count)
+            CK(h, cudaMemcpyAsync(t.data(), d.hs[b], count * sizeof(raw), cudaMemcpyDeviceToHost, d.stream));
+        CK(h, cudaStreamSynchronize(d.stream));
+        for (size_t k = 0; k < count; ++k) out[k] = HostSpring{{(double)t[k].d[0], (double)t[k].d[1], (double)t[k].d[2]}, t[k].pid};
+        return DEM_OK;
+    };
+    return d.precision == 0 ? get(Raw64{}) : get(Raw32{});
+}
+
 dem_status dem_get_history(dem_handle* h, int64_t cap, uint32_t* oi, uint32_t* oj, double* od, int64_t* nout) {
     if (!h || !nout || cap < 0) return DEM_ERR_INVALID_ARG;
     if (h->broken) return fail(h, DEM_ERR_STATE, "handle is unusable after a CUDA error");
     if (!h->has_particles) return fail(h, DEM_ERR_STATE, "no particles");
     DeviceGuard g(h->device);
     Domain& d = h->d;
-    const size_t n = d.n, N = d.cap, M = d.maxc;
+    const size_t n = d.n, N = d.cap;
     *nout = 0;
     if (n == 0 || d.model != 0) return DEM_OK;
     std::vector<uint32_t> perm, ids, cnt;
@@ -1114,36 +1158,16 @@ dem_status dem_get_history(dem_handle* h, int64_t cap, uint32_t* oi, uint32_t* o
         for (size_t q = 0; q < n; ++q) perm[q] = (uint32_t)q;
     uint32_t mx = 0;
     for (size_t q = 0; q < n; ++q) mx = std::max(mx, slots_of(d, cnt[perm[q]]));
-    std::vector<uint32_t> pid((size_t)mx * N);
-    std::vector<double> dv((size_t)3 * mx * N);
-    if (mx) {
-        CK(h, cudaMemcpyAsync(pid.data(), d.hpid[d.h_cur], (size_t)mx * N * 4, cudaMemcpyDeviceToHost, d.stream));
-        for (int c = 0; c < 3; ++c) {
-            if (d.precision == 0) {
-                CK(h, cudaMemcpyAsync(dv.data() + (size_t)c * mx * N, (const double*)d.hd[d.h_cur] + (size_t)c * M * N,
-                                      (size_t)mx * N * 8, cudaMemcpyDeviceToHost, d.stream));
-            } else {
-                std::vector<float> tmp((size_t)mx * N);
-                CK(h, cudaMemcpyAsync(tmp.data(), (const float*)d.hd[d.h_cur] + (size_t)c * M * N, (size_t)mx * N * 4,
-                                      cudaMemcpyDeviceToHost, d.stream));
-                CK(h, cudaStreamSynchronize(d.stream));
-                for (size_t k = 0; k < tmp.size(); ++k) dv[(size_t)c * mx * N + k] = tmp[k];
-            }
-        }
-        CK(h, cudaStreamSynchronize(d.stream));
-    }
+    std::vector<HostSpring> sp;
+    if ((s = download_springs(h, sp, d.h_cur, mx)) != DEM_OK) return s;
     struct Rec { uint32_t i, j; double d[3]; };
     std::vector<Rec> recs;
     for (size_t q = 0; q < n; ++q) {
         const uint32_t src = perm[q], owner = ids[q];
         const uint32_t c = slots_of(d, cnt[src]);
         for (uint32_t k = 0; k < c; ++k) {
-            const uint32_t p = pid[(size_t)k * N + src];
-            if (p >= DEM_WALL_BASE || owner < p) {
-                Rec r{owner, p, {dv[(size_t)0 * mx * N + (size_t)k * N + src], dv[(size_t)1 * mx * N + (size_t)k * N + src],
-                                 dv[(size_t)2 * mx * N + (size_t)k * N + src]}};
-                recs.push_back(r);
-            }
+            const HostSpring& f = sp[(size_t)k * N + src];
+            if (f.pid >= DEM_WALL_BASE || owner < f.pid) recs.push_back(Rec{owner, f.pid, {f.d[0], f.d[1], f.d[2]}});
         }
     }
     std::sort(recs.begin(), recs.end(), [](const Rec& a, const Rec& b) { return a.i != b.i ? a.i < b.i : a.j < b.j; });
@@ -1168,19 +1192,20 @@ dem_status dem_restore(dem_handle* h, int64_t n, const double* x, const double* 
         CK(h, cudaStreamSynchronize(d.stream));
         return DEM_OK;
     }
-    // per-particle lists in id order; after the first sort perm[q] is the id position
+    // per-particle lists in id order; after the first sort perm[q] is the id position. List
+    // mode keeps them in ascending partner id (walls last), whatever order the records have.
     const size_t N = d.cap, M = d.maxc;
-    std::vector<uint32_t> cnt(N, 0), pid(M * N, 0);
-    std::vector<double> dv(3 * M * N, 0.0);
+    std::vector<uint32_t> cnt(N, 0);
+    std::vector<HostSpring> sp(M * N, HostSpring{});
     auto add = [&](uint32_t owner, uint32_t partner, double a, double b, double c) -> bool {
         if (owner >= (uint32_t)n) return false;
-        const uint32_t k = cnt[owner];
+        uint32_t k = cnt[owner];
         if (k >= M) return false;
-        pid[(size_t)k * N + owner] = partner;
-        dv[(0 * M + k) * N + owner] = a;
-        dv[(1 * M + k) * N + owner] = b;
-        dv[(2 * M + k) * N + owner] = c;
         cnt[owner] = k + 1;
+        if (d.list_mode)
+            for (; k > 0 && sp[(size_t)(k - 1) * N + owner].pid > partner; --k)
+                sp[(size_t)k * N + owner] = sp[(size_t)(k - 1) * N + owner];
+        sp[(size_t)k * N + owner] = HostSpring{{a, b, c}, partner};
         return true;
     };
     const int nw = (int)h->walls.size();
@@ -1193,17 +1218,22 @@ dem_status dem_restore(dem_handle* h, int64_t n, const double* x, const double* 
         if (!ok) { h->has_particles = false; return fail(h, DEM_ERR_INVALID_ARG, "invalid or excess history record"); }
     }
     CK(h, cudaMemcpyAsync(d.hcnt[d.h_cur], cnt.data(), N * 4, cudaMemcpyHostToDevice, d.stream));
-    CK(h, cudaMemcpyAsync(d.hpid[d.h_cur], pid.data(), M * N * 4, cudaMemcpyHostToDevice, d.stream));
-    if (d.precision == 0) {
-        CK(h, cudaMemcpyAsync(d.hd[d.h_cur], dv.data(), 3 * M * N * 8, cudaMemcpyHostToDevice, d.stream));
+    auto put = [&](auto raw) -> dem_status {
+        using R = decltype(raw);
+        using V = std::remove_reference_t<decltype(raw.d[0])>;
+        std::vector<R> t(M * N);
+        for (size_t k = 0; k < t.size(); ++k) {
+            t[k] = R{};
+            for (int c = 0; c < 3; ++c) t[k].d[c] = (V)sp[k].d[c];
+            t[k].pid = sp[k].pid;
+        }
+        CK(h, cudaMemcpyAsync(d.hs[d.h_cur], t.data(), t.size() * sizeof(R), cudaMemcpyHostToDevice, d.stream));
+        // list mode: which list entries have a spring was found at the sort, before they were set
+        if (d.list_mode) CK(h, run_tiles(d, true));
         CK(h, cudaStreamSynchronize(d.stream));
-    } else {
-        std::vector<float> f(dv.size());
-        for (size_t k = 0; k < dv.size(); ++k) f[k] = (float)dv[k];
-        CK(h, cudaMemcpyAsync(d.hd[d.h_cur], f.data(), f.size() * 4, cudaMemcpyHostToDevice, d.stream));
-        CK(h, cudaStreamSynchronize(d.stream));
-    }
-    return DEM_OK;
+        return DEM_OK;
+    };
+    return d.precision == 0 ? put(Raw64{}) : put(Raw32{});
 }
 
 dem_status dem_get_diagnostics(dem_handle* h, double* out) {
@@ -1234,11 +1264,12 @@ dem_status dem_get_diagnostics(dem_handle* h, double* out) {
 // Row-major key ((k ny + j) nx + i) of a cell key of the handle's sort order.
 static uint32_t row_major_key(const dem_handle* h, uint32_t key) {
     if (h->bshift == 0) return key;
-    const uint32_t sh = (uint32_t)h->bshift, m = (1u << sh) - 1u;
+    const uint32_t sh = (uint32_t)h->bshift;
     const uint32_t brick = key >> (3 * sh), in = key & ((1u << (3 * sh)) - 1u);
     const uint32_t bi = brick % (uint32_t)h->bdims[0], bt = brick / (uint32_t)h->bdims[0];
     const uint32_t bj = bt % (uint32_t)h->bdims[1], bk = bt / (uint32_t)h->bdims[1];
-    const uint32_t i = (bi << sh) | (in & m), j = (bj << sh) | ((in >> sh) & m), k = (bk << sh) | (in >> (2 * sh));
+    const uint32_t i = (bi << sh) | unspread3(in & 0x249u), j = (bj << sh) | unspread3((in >> 1) & 0x249u),
+                   k = (bk << sh) | unspread3((in >> 2) & 0x249u);
     return (uint32_t)(((uint64_t)k * (uint64_t)h->dims[1] + j) * (uint64_t)h->dims[0] + i);
 }
 
@@ -1281,16 +1312,13 @@ dem_status dem_debug_snapshot(dem_handle* h, uint32_t* cell, uint32_t* order, in
         CK(h, cudaStreamSynchronize(d.stream));
         uint32_t mx = 0;
         for (size_t q = 0; q < n; ++q) mx = std::max(mx, slots_of(d, cnt[q]));
-        std::vector<uint32_t> pid((size_t)mx * N);
-        if (mx) {
-            CK(h, cudaMemcpyAsync(pid.data(), d.hpid[ho], (size_t)mx * N * 4, cudaMemcpyDeviceToHost, d.stream));
-            CK(h, cudaStreamSynchronize(d.stream));
-        }
+        std::vector<HostSpring> sp;
+        if ((s = download_springs(h, sp, ho, mx)) != DEM_OK) return s;
         std::vector<std::pair<uint32_t, uint32_t>> pr;
         for (size_t q = 0; q < n; ++q) {
             const uint32_t c = slots_of(d, cnt[q]);
             for (uint32_t k = 0; k < c; ++k) {
-                const uint32_t p = pid[(size_t)k * N + q];
+                const uint32_t p = sp[(size_t)k * N + q].pid;
                 if (p < DEM_WALL_BASE && ids[q] < p) pr.emplace_back(ids[q], p);
             }
         }
@@ -1315,16 +1343,22 @@ dem_status dem_get_grid(const dem_handle* h, double* origin, double* cell, int64
     return DEM_OK;
 }
 
+// Bytes of the list-mode buffers of a domain: lists and counts, tile entries and halos,
+// wall masks, reference positions, window maps, spring masks.
+static size_t list_bytes(const Domain& d) {
+    return (size_t)d.cap * (4 + 6 * (size_t)DEM_LIST_CAP + 4 + 16 + 8 + 16) + d.halo_words * 4 + (size_t)d.tiles_cap * 4;
+}
+
 int64_t dem_device_bytes(const dem_handle* h) {
     if (!h) return 0;
     const Domain& d = h->d;
     const size_t N = d.cap, M = d.maxc, C = (size_t)d.cells_cap + 1;
     const size_t T = d.precision == 0 ? 8 : 4;
     size_t state = d.precision == 0 ? N * (9 * 8 + 8) : N * (4 * 16 + 4);
-    size_t b = 2 * state + 2 * (N * 4 + N * 4 * M + N * T * 3 * M) + 5 * N * 4 + 2 * C * 4 + (size_t)d.part_cap * 4 +
+    size_t b = 2 * state + 2 * (N * 4 + N * 4 * T * M) + 5 * N * 4 + 2 * C * 4 + (size_t)d.part_cap * 4 +
                (size_t)d.diag_part_cap * 80 + sizeof(StatusDev) + 128 + sizeof(SceneDev) * d.scenes_cap;
     b += (size_t)h->stage_cap * (9 * 8 + 4);
-    if (d.list_mode) b += N * (4 + 4 * (size_t)DEM_LIST_CAP + 4 + 16 + 8);
+    if (d.list_mode) b += list_bytes(d);
     return (int64_t)b;
 }
 
@@ -1396,7 +1430,7 @@ struct BatchScene {
     int64_t dims[3] = {1, 1, 1};
     int bshift = 0;                    // list mode: cells in bricks of (2^bshift)^3
     int64_t bdims[3] = {1, 1, 1};
-    uint32_t p0 = 0, c0 = 0, ncell = 1;
+    uint32_t p0 = 0, c0 = 0, ncell = 1, t0 = 0;
 };
 
 }  // namespace
@@ -1450,7 +1484,7 @@ void fill_batch_scene(const BatchScene& sc, SceneDev& S) {
         tmp.dims[a] = sc.dims[a];
         tmp.bdims[a] = sc.bdims[a];
     }
-    fill_scene(&tmp, S, sc.p0, (uint32_t)sc.n, sc.c0);
+    fill_scene(&tmp, S, sc.p0, (uint32_t)sc.n, sc.c0, sc.t0);
 }
 
 // Rebuild the packed domain: kept scenes (state + springs), then the staged ones.
@@ -1508,6 +1542,14 @@ dem_status repack(dem_batch* b) {
     nd.launches = od.launches;
     nd.n = (uint32_t)n_new;
     nd.ncells = (uint32_t)std::max<uint64_t>(c_new, 1);
+    nd.tile = tile_size(nd, nd.n);
+    uint32_t tiles = 0;
+    for (auto* group : {&kept, &fresh})
+        for (BatchScene* sc : *group) {
+            sc->t0 = tiles;
+            tiles += ((uint32_t)sc->n + nd.tile - 1) / nd.tile;
+        }
+    nd.ntiles = tiles;
     std::string err;
     dem_status s = alloc_domain(nd, nd.n, nd.ncells, err);
     if (s != DEM_OK) return bfail(b, s, err);
@@ -1824,9 +1866,9 @@ int64_t dem_batch_device_bytes(const dem_batch* b) {
     const size_t N = d.cap, M = d.maxc, C = (size_t)d.cells_cap + 1;
     const size_t T = d.precision == 0 ? 8 : 4;
     const size_t state = d.precision == 0 ? N * (9 * 8 + 8) : N * (4 * 16 + 4);
-    size_t bytes = 2 * state + 2 * (N * 4 + N * 4 * M + N * T * 3 * M) + 5 * N * 4 + 2 * C * 4 +
+    size_t bytes = 2 * state + 2 * (N * 4 + N * 4 * T * M) + 5 * N * 4 + 2 * C * 4 +
                    b->stage_cap * 76 + b->map_cap * 4;
-    if (d.list_mode) bytes += N * (4 + 4 * (size_t)DEM_LIST_CAP + 4 + 16 + 8);
+    if (d.list_mode) bytes += list_bytes(d);
     return (int64_t)bytes;
 }
 
@@ -1974,11 +2016,9 @@ void fill_io(dem_slabs* S, bool import, uint32_t& ntotal) {
         e.src = sets[1 - c];
         e.dst = import ? sets[1 - c] : sets[c];
         e.hcnt_src = d.hcnt[hs];
-        e.hpid_src = d.hpid[hs];
-        e.hd_src = (const T*)d.hd[hs];
+        e.hs_src = (const Spring<T>*)d.hs[hs];
         e.hcnt_dst = d.hcnt[hd];
-        e.hpid_dst = d.hpid[hd];
-        e.hd_dst = (T*)d.hd[hd];
+        e.hs_dst = (Spring<T>*)d.hs[hd];
         e.n = import ? 0u : d.n;
         e.p0 = p0;
         e.cap = d.cap;

@@ -135,35 +135,19 @@ __device__ __forceinline__ int source_slab(const IO* io, int S, uint32_t gi) {
     return s;
 }
 
-// Springs of one particle, slot lists keyed by partner id (slot-major planes of stride
-// cap), copied four slots at a time: the loads of a group are issued before its stores.
+// Springs of one particle (slot-major records of stride cap), copied four slots at a time:
+// the loads of a group are issued before its stores.
 template <class T>
-__device__ __forceinline__ void copy_springs(uint32_t c, uint32_t maxc, const uint32_t* __restrict__ ps,
-                                             const T* __restrict__ ds, size_t cs, uint32_t q,
-                                             uint32_t* __restrict__ pd, T* __restrict__ dd, size_t cd, uint32_t p) {
+__device__ __forceinline__ void copy_springs(uint32_t c, const Spring<T>* __restrict__ s, size_t cs, uint32_t q,
+                                             Spring<T>* __restrict__ d, size_t cd, uint32_t p) {
     for (uint32_t k0 = 0; k0 < c; k0 += 4) {
-        uint32_t pid[4];
-        T d0[4], d1[4], d2[4];
+        Spring<T> r[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const size_t k = k0 + u;
-            if (k < c) {
-                pid[u] = ps[k * cs + q];
-                d0[u] = ds[k * cs + q];
-                d1[u] = ds[(maxc + k) * cs + q];
-                d2[u] = ds[(2 * (size_t)maxc + k) * cs + q];
-            }
-        }
+        for (int u = 0; u < 4; ++u)
+            if (k0 + u < c) r[u] = load_spring(&s[(size_t)(k0 + u) * cs + q]);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const size_t k = k0 + u;
-            if (k < c) {
-                pd[k * cd + p] = pid[u];
-                dd[k * cd + p] = d0[u];
-                dd[(maxc + k) * cd + p] = d1[u];
-                dd[(2 * (size_t)maxc + k) * cd + p] = d2[u];
-            }
-        }
+        for (int u = 0; u < 4; ++u)
+            if (k0 + u < c) store_spring(&d[(size_t)(k0 + u) * cd + p], mk(r[u].x, r[u].y, r[u].z), r[u].pid);
     }
 }
 
@@ -284,8 +268,7 @@ __global__ void __launch_bounds__(ROUTE_THREADS, 4) k_halo_route(const __grid_co
                             // the owner's springs travel with it
                             const uint32_t c = min(src.hcnt_src[q], a.maxc);
                             D.hcnt_dst[p] = c;
-                            copy_springs(c, a.maxc, src.hpid_src, src.hd_src, src.cap, q, D.hpid_dst, D.hd_dst, D.cap,
-                                         p);
+                            copy_springs(c, src.hs_src, src.cap, q, D.hs_dst, D.cap, p);
                         } else {
                             D.hcnt_dst[p] = 0u;   // a ghost's own forces are not used
                         }

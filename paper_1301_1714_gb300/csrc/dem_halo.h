@@ -25,11 +25,9 @@ struct SlabIO {
     St src;                         // state just computed by the force pass (index q)
     St dst;                         // free state set that receives the slab's new layout
     const uint32_t* hcnt_src;       // springs written by the force pass (index q)
-    const uint32_t* hpid_src;
-    const T* hd_src;
+    const Spring<T>* hs_src;
     uint32_t* hcnt_dst;             // springs of the new layout
-    uint32_t* hpid_dst;
-    T* hd_dst;
+    Spring<T>* hs_dst;
     uint32_t n;                     // particles in the source layout
     uint32_t p0;                    // first launch index of this slab
     uint32_t cap;                   // allocated particle capacity of the slab

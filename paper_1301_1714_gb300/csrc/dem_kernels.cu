@@ -27,14 +27,6 @@
 #define DEM_FORCE_MIN_BLOCKS 4
 #endif
 
-// List mode orders windows of DEM_WINDOW_MULT force blocks (at most 1,024 positions) by
-// contact count. Measured on GB300, 4,194,304-sphere drum, block 128, step with its share
-// of the sorts: 0.741 / 0.724 / 0.719 / 0.720 ms for 1 / 2 / 4 / 8 blocks per window
-// (narrower contact counts per warp against a longer window sort).
-#ifndef DEM_WINDOW_MULT
-#define DEM_WINDOW_MULT 4
-#endif
-
 namespace demgb {
 
 // ======================================================================= force pass
@@ -50,11 +42,9 @@ struct ForceArgs {
     const uint32_t* cs;
     const uint32_t* perm;
     const uint32_t* hin_cnt;
-    const uint32_t* hin_pid;
-    const typename PR::T* hin_d;
+    const Spring<typename PR::T>* hin;
     uint32_t* hout_cnt;
-    uint32_t* hout_pid;
-    typename PR::T* hout_d;
+    Spring<typename PR::T>* hout;
     uint32_t* key;
     uint32_t* rank;
     uint32_t* cnt;
@@ -104,22 +94,16 @@ __global__ void __launch_bounds__(256, DEM_FORCE_MIN_BLOCKS) k_force(ForceArgs<P
         src = pv ? __ldg(&a.perm[q]) : q;
         if (PRACT || !S.active) {
             cnt_old = min(__ldg(&a.hin_cnt[src]), maxc);
-            // the stored springs are streamed from DRAM: start their loads now so they are
-            // in L1 when phase 2 matches contacts against them
-            for (uint32_t k = 0; k < cnt_old; ++k)
-                for (int c = 0; c < 3; ++c) prefetch_l1(&a.hin_d[(c * (size_t)maxc + k) * cap + src]);
-            for (uint32_t k = 0; k < cnt_old; ++k) s_oid[k * bd + tid] = __ldg(&a.hin_pid[k * cap + src]);
+            // the stored springs are streamed from DRAM: reading the partner ids now brings
+            // the records into L1 for phase 2
+            for (uint32_t k = 0; k < cnt_old; ++k) s_oid[k * bd + tid] = __ldg(&a.hin[k * cap + src].pid);
         }
     }
     if (valid && !live) {
         // frozen scene: carry state and springs unchanged
         if (!EVAL) {
             PR::store(B, q, me);
-            for (uint32_t k = 0; k < cnt_old; ++k) {
-                a.hout_pid[k * cap + q] = s_oid[k * bd + tid];
-                for (int c = 0; c < 3; ++c)
-                    a.hout_d[(c * (size_t)maxc + k) * cap + q] = a.hin_d[(c * (size_t)maxc + k) * cap + src];
-            }
+            for (uint32_t k = 0; k < cnt_old; ++k) a.hout[k * cap + q] = a.hin[k * cap + src];
             a.hout_cnt[q] = cnt_old;
             const uint32_t kk = a.skey[q];
             a.key[q] = kk;
@@ -186,21 +170,16 @@ __global__ void __launch_bounds__(256, DEM_FORCE_MIN_BLOCKS) k_force(ForceArgs<P
             const T mj = PR::mass(S, rj);
             const T meff = law_div(mi * mj, mi + mj);
             const T Reff = law_div(ri * rjT, ri + rjT);
-            const V3<T> dold = find_spring(s_oid, bd, tid, cnt_old, gid, a.hin_d, (size_t)maxc, cap, src);
+            const V3<T> dold = find_spring(s_oid, bd, tid, cnt_old, gid, a.hin, cap, src);
             V3<T> Fc, Ftc, dnew, Mr;
-            law_practical<TERMS>(L, n, delta, v, rw, Reff, meff, dold, Fc, Ftc, dnew, me.w - wj, Mr);
+            law_practical<TERMS, 2>(L, n, delta, v, rw, Reff, meff, dold, Fc, Ftc, dnew, me.w - wj, Mr);
             F = F + Fc;
             Tq = Tq + cross(n, Ftc) * ri;
             if (TERMS) Tq = Tq + Mr;
-            if (nnew < maxc) {
-                a.hout_pid[nnew * cap + q] = gid;
-                a.hout_d[(0 * (size_t)maxc + nnew) * cap + q] = dnew.x;
-                a.hout_d[(1 * (size_t)maxc + nnew) * cap + q] = dnew.y;
-                a.hout_d[(2 * (size_t)maxc + nnew) * cap + q] = dnew.z;
-            }
+            if (nnew < maxc) store_spring(&a.hout[nnew * cap + q], dnew, gid);
         } else {
             F = F + law_simple(L, n, delta, v);
-            if (EVAL && nnew < maxc) a.hout_pid[nnew * cap + q] = gid;
+            if (EVAL && nnew < maxc) store_spring(&a.hout[nnew * cap + q], mk(T(0), T(0), T(0)), gid);
         }
         ++nnew;
         ++c_pp;
@@ -217,21 +196,16 @@ __global__ void __launch_bounds__(256, DEM_FORCE_MIN_BLOCKS) k_force(ForceArgs<P
             const uint32_t gid = DEM_WALL_BASE + (uint32_t)w;
             if (PRACT) {
                 const V3<T> rw = me.w * ri;
-                const V3<T> dold = find_spring(s_oid, bd, tid, cnt_old, gid, a.hin_d, (size_t)maxc, cap, src);
+                const V3<T> dold = find_spring(s_oid, bd, tid, cnt_old, gid, a.hin, cap, src);
                 V3<T> Fc, Ftc, dnew, Mr;
-                law_practical<TERMS>(L, n, delta, v, rw, ri, mi, dold, Fc, Ftc, dnew, me.w - PR::wall_omega(W), Mr);
+                law_practical<TERMS, 2>(L, n, delta, v, rw, ri, mi, dold, Fc, Ftc, dnew, me.w - PR::wall_omega(W), Mr);
                 F = F + Fc;
                 Tq = Tq + cross(n, Ftc) * ri;
                 if (TERMS) Tq = Tq + Mr;
-                if (nnew < maxc) {
-                    a.hout_pid[nnew * cap + q] = gid;
-                    a.hout_d[(0 * (size_t)maxc + nnew) * cap + q] = dnew.x;
-                    a.hout_d[(1 * (size_t)maxc + nnew) * cap + q] = dnew.y;
-                    a.hout_d[(2 * (size_t)maxc + nnew) * cap + q] = dnew.z;
-                }
+                if (nnew < maxc) store_spring(&a.hout[nnew * cap + q], dnew, gid);
             } else {
                 F = F + law_simple(L, n, delta, v);
-                if (EVAL && nnew < maxc) a.hout_pid[nnew * cap + q] = gid;
+                if (EVAL && nnew < maxc) store_spring(&a.hout[nnew * cap + q], mk(T(0), T(0), T(0)), gid);
             }
             ++nnew;
             ++c_wc;
@@ -340,14 +314,31 @@ __global__ void __launch_bounds__(1024) k_scan_spine(uint32_t* part, uint32_t nb
         }
 }
 
-// cs[k] = exclusive prefix of cnt; cnt[k] = 0 for the next sort
+// cs[k] = exclusive prefix of cnt; cnt[k] = 0 for the next sort. With own_prefix every block
+// adds up the tile sums before its tiles itself (each sum is read once per block), so no
+// spine pass is needed; part then holds the tile sums, otherwise their exclusive prefixes.
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_down(uint32_t* __restrict__ cnt, uint32_t m, uint32_t ntiles,
                                                             const uint32_t* __restrict__ part, uint32_t* __restrict__ cs,
-                                                            const CtrlDev* ctrl) {
+                                                            const CtrlDev* ctrl, int own_prefix) {
     if (ctrl->rebuild != 1) return;   // no sort this step (or a void step)
     __shared__ uint32_t ws[SCAN_THREADS / 32];
+    __shared__ uint32_t s_pre;
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint32_t seen = 0, before = 0;   // tile sums added up so far, and their total
     for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        if (own_prefix) {
+            uint32_t t = 0;
+            for (uint32_t k = seen + threadIdx.x; k < tile; k += SCAN_THREADS) t += __ldg(&part[k]);
+            if (threadIdx.x == 0) s_pre = 0;
+            __syncthreads();
+            t = __reduce_add_sync(0xffffffffu, t);
+            if (lane == 0 && t) atomicAdd(&s_pre, t);
+            __syncthreads();
+            before += s_pre;
+            seen = tile;
+        } else {
+            before = part[tile];
+        }
         const uint32_t base = tile * SCAN_TILE + threadIdx.x * SCAN_ITEMS;
         uint32_t v[SCAN_ITEMS];
         uint32_t s = 0;
@@ -373,7 +364,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_down(uint32_t* __restrict
             if (lane < SCAN_THREADS / 32) ws[lane] = w;
         }
         __syncthreads();
-        uint32_t run = part[tile] + (inc - s) + (wid > 0 ? ws[wid - 1] : 0u);
+        uint32_t run = before + (inc - s) + (wid > 0 ? ws[wid - 1] : 0u);
         for (int i = 0; i < SCAN_ITEMS; ++i) {
             const uint32_t k = base + i;
             if (k < m) {
@@ -428,8 +419,8 @@ __global__ void k_reorder(uint32_t n, typename PR::State S0, typename PR::State 
         reorder_one<PR>(s, A, B, key, cs, tmp, perm, skey, ref);
 }
 
-// List mode stores the sorted particles in (cell, id) order within windows of
-// DEM_WINDOW_MULT force blocks, each window ordered by the particles' contact counts in
+// List mode stores the sorted particles in (cell, id) order, each tile of them ordered by the
+// particles' contact counts in
 // the step just finished (descending; ties keep the (cell, id) order). The lanes of a warp run
 // their candidate lists in lockstep, so grouping similar counts shortens the longest
 // lane's loop; a particle's own sums keep their order, so results do not change.
@@ -457,36 +448,33 @@ __global__ void k_rank_cell(uint32_t n, typename PR::State S0, typename PR::Stat
     }
 }
 
-// One block per window of wsize (cell, id) positions (blockDim.x: the power of two at or
-// above wsize, at most 1,024): fin[q] = final position, the window's particles in descending
-// order of their last contact count (ties in (cell, id) order), so the lanes of a force-pass
-// warp carry similar numbers of contacts. A window is split where one scene ends and the next
-// begins (scenes are contiguous in the (cell, id) order), so every particle stays inside its
-// scene's range of positions. The order is a bitonic sort in shared memory of one 32-bit word
-// per position: scene run within the window (10 bits), 63 - count (6 bits), position (10 bits).
-// The block then gathers its window's state to the final positions: the order it has just
+// One block per tile of (cell, id) positions of a scene (blockDim.x: the power of two at or
+// above the tile's size): fin[q] = final position, the tile's particles in descending order
+// of their last contact count (ties in (cell, id) order), so the lanes of a force-pass warp
+// carry similar numbers of contacts. Scenes are contiguous in the (cell, id) order and tiles
+// never cross them. The order is a bitonic sort in shared memory of one 32-bit word per
+// position: 63 - count (6 bits), position (10 bits). The block then gathers its window's state to the final positions: the order it has just
 // found is still in shared memory, so a separate gather pass (one launch, and fin and canon
 // read once more) is not needed.
 template <class PR>
-__global__ void __launch_bounds__(1024) k_window(uint32_t n, uint32_t wsize, const SceneDev* scenes, int nscenes,
+__global__ void __launch_bounds__(512) k_window(uint32_t tile, uint32_t ntiles, const SceneDev* scenes, int nscenes,
                                                  typename PR::State S0, typename PR::State S1, const CtrlDev* ctrl,
                                                  const uint32_t* __restrict__ wkey, const uint32_t* __restrict__ key,
                                                  const uint32_t* __restrict__ canon, uint32_t* __restrict__ fin,
                                                  uint32_t* __restrict__ perm, uint32_t* __restrict__ skey,
                                                  float4* __restrict__ ref) {
     if (ctrl->rebuild != 1) return;   // no sort this step (or a void step)
-    __shared__ uint32_t s_w[1024];
+    __shared__ uint32_t s_w[512];
     const typename PR::State A = ctrl->cur ? S1 : S0;
     const typename PR::State B = ctrl->cur ? S0 : S1;
     const uint32_t w = blockDim.x, t = threadIdx.x;
-    for (uint32_t base = blockIdx.x * wsize; base < n; base += gridDim.x * wsize) {
+    for (uint32_t tl = blockIdx.x; tl < ntiles; tl += gridDim.x) {
+        const SceneDev& S = scenes[scene_of_tile(scenes, nscenes, tl)];
+        const uint32_t off = (tl - S.t0) * tile;
+        const uint32_t base = S.p0 + off, n = min(tile, S.np - off);
         const uint32_t q = base + t;
-        const int sc0 = scene_of(scenes, nscenes, base);
-        uint32_t word = 0xFFFFFFFFu;   // past the window or the end: sorts last
-        if (t < wsize && q < n) {
-            const uint32_t run = (uint32_t)(scene_of(scenes, nscenes, q) - sc0);
-            word = (run << 16) | ((63u - min(wkey[q], 63u)) << 10) | t;
-        }
+        uint32_t word = 0xFFFFFFFFu;   // past the tile: sorts last
+        if (t < n) word = ((63u - min(wkey[q], 63u)) << 10) | t;
         __syncthreads();
         s_w[t] = word;
         __syncthreads();
@@ -754,18 +742,14 @@ __global__ void __launch_bounds__(DIAG_THREADS) k_diag_final(const double* __res
 // history buffer: afterwards slot lists sit at the same index as the particle.
 template <class T>
 __global__ void k_hist_canon(uint32_t n, const CtrlDev* ctrl, const uint32_t* __restrict__ perm,
-                             const uint32_t* __restrict__ cin, const uint32_t* __restrict__ pin,
-                             const T* __restrict__ din, uint32_t* __restrict__ cout, uint32_t* __restrict__ pout,
-                             T* __restrict__ dout, size_t cap, uint32_t maxc) {
+                             const uint32_t* __restrict__ cin, const Spring<T>* __restrict__ in,
+                             uint32_t* __restrict__ cout, Spring<T>* __restrict__ out, size_t cap, uint32_t maxc) {
     const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= n) return;
     const uint32_t src = ctrl->perm_valid ? perm[q] : q;
     const uint32_t c = min(cin[src], maxc);
     cout[q] = c;
-    for (uint32_t k = 0; k < c; ++k) {
-        pout[k * cap + q] = pin[k * cap + src];
-        for (int a = 0; a < 3; ++a) dout[(a * (size_t)maxc + k) * cap + q] = din[(a * (size_t)maxc + k) * cap + src];
-    }
+    for (uint32_t k = 0; k < c; ++k) out[k * cap + q] = in[k * cap + src];
 }
 
 // New packed layout: particle p of the new domain takes the old current-state particle
@@ -774,9 +758,9 @@ __global__ void k_hist_canon(uint32_t n, const CtrlDev* ctrl, const uint32_t* __
 template <class PR>
 __global__ void k_repack(uint32_t n_new, const uint32_t* __restrict__ map, typename PR::State oS0,
                          typename PR::State oS1, const CtrlDev* octrl, const uint32_t* __restrict__ ocnt,
-                         const uint32_t* __restrict__ opid, const typename PR::T* __restrict__ od, size_t ocap,
-                         typename PR::State nB, uint32_t* __restrict__ ncnt, uint32_t* __restrict__ npid,
-                         typename PR::T* __restrict__ nd, size_t ncap, uint32_t maxc) {
+                         const Spring<typename PR::T>* __restrict__ oh, size_t ocap, typename PR::State nB,
+                         uint32_t* __restrict__ ncnt, Spring<typename PR::T>* __restrict__ nh, size_t ncap,
+                         uint32_t maxc) {
     const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n_new) return;
     const uint32_t m = map[p];
@@ -788,10 +772,7 @@ __global__ void k_repack(uint32_t n_new, const uint32_t* __restrict__ map, typen
     PR::store(nB, p, PR::load(A, m));
     const uint32_t c = min(ocnt[m], maxc);
     ncnt[p] = c;
-    for (uint32_t k = 0; k < c; ++k) {
-        npid[k * ncap + p] = opid[k * ocap + m];
-        for (int a = 0; a < 3; ++a) nd[(a * (size_t)maxc + k) * ncap + p] = od[(a * (size_t)maxc + k) * ocap + m];
-    }
+    for (uint32_t k = 0; k < c; ++k) nh[k * ncap + p] = oh[k * ocap + m];
 }
 
 static inline StateF64 shifted(StateF64 s, uint32_t p0) {
@@ -881,9 +862,14 @@ cudaError_t run_rebuild(Domain& d) {
     const uint32_t gb = std::min(nb, (uint32_t)std::max(d.sort_blocks, 1));
     k_scan_reduce<<<gb, SCAN_THREADS, 0, d.stream>>>(d.cnt, m, nb, d.part, d.ctrl);
     DEM_LAUNCH_CHECK();
-    k_scan_spine<<<1, 1024, 0, d.stream>>>(d.part, nb, d.ctrl);
-    DEM_LAUNCH_CHECK();
-    k_scan_down<<<gb, SCAN_THREADS, 0, d.stream>>>(d.cnt, m, nb, d.part, d.cs, d.ctrl);
+    // Every block adding up the tile sums itself costs nb / 2 loads per tile: 4,096 tiles (8 M
+    // cells) read 32 MB from L2; above that the one-block spine pass is the cheaper prefix.
+    const int own = nb <= 4096 ? 1 : 0;
+    if (!own) {
+        k_scan_spine<<<1, 1024, 0, d.stream>>>(d.part, nb, d.ctrl);
+        DEM_LAUNCH_CHECK();
+    }
+    k_scan_down<<<gb, SCAN_THREADS, 0, d.stream>>>(d.cnt, m, nb, d.part, d.cs, d.ctrl, own);
     DEM_LAUNCH_CHECK();
     k_scatter<<<sgrid(d, d.n), 256, 0, d.stream>>>(d.n, d.key, d.rank, d.cs, d.tmp, d.ctrl);
     DEM_LAUNCH_CHECK();
@@ -897,10 +883,9 @@ cudaError_t run_rebuild(Domain& d) {
         DEM_LAUNCH_CHECK();
     } else {
         // (cell, id) positions, the window order by last contact count, the gather
-        const uint32_t wsz = std::min(1024u, (uint32_t)d.block * DEM_WINDOW_MULT);
         uint32_t wb = 32;
-        while (wb < wsz) wb <<= 1;
-        const uint32_t wg = std::max(1u, std::min(nblk(d.n, wsz), (uint32_t)std::max(d.sort_blocks, 1)));
+        while (wb < d.tile) wb <<= 1;
+        const uint32_t wg = std::max(1u, std::min(d.ntiles, (uint32_t)std::max(d.sort_blocks, 1)));
         if (d.precision == 0)
             k_rank_cell<PF64><<<sgrid(d, d.n), 256, 0, d.stream>>>(d.n, d.S64[0], d.S64[1], d.ctrl, d.key, d.cs, d.tmp,
                                                                    d.hcnt[0], d.hcnt[1], d.canon, d.rank);
@@ -909,10 +894,10 @@ cudaError_t run_rebuild(Domain& d) {
                                                                    d.hcnt[0], d.hcnt[1], d.canon, d.rank);
         DEM_LAUNCH_CHECK();
         if (d.precision == 0)
-            k_window<PF64><<<wg, wb, 0, d.stream>>>(d.n, wsz, d.d_scenes, d.nscenes, d.S64[0], d.S64[1], d.ctrl, d.rank,
+            k_window<PF64><<<wg, wb, 0, d.stream>>>(d.tile, d.ntiles, d.d_scenes, d.nscenes, d.S64[0], d.S64[1], d.ctrl, d.rank,
                                                     d.key, d.canon, d.fin, d.perm, d.skey, d.ref);
         else
-            k_window<PF32><<<wg, wb, 0, d.stream>>>(d.n, wsz, d.d_scenes, d.nscenes, d.S32[0], d.S32[1], d.ctrl, d.rank,
+            k_window<PF32><<<wg, wb, 0, d.stream>>>(d.tile, d.ntiles, d.d_scenes, d.nscenes, d.S32[0], d.S32[1], d.ctrl, d.rank,
                                                     d.key, d.canon, d.fin, d.perm, d.skey, d.ref);
         DEM_LAUNCH_CHECK();
         cudaError_t e = run_lists(d);
@@ -969,11 +954,9 @@ static cudaError_t force_impl(Domain& d, const typename PR::State& S0, const typ
     a.perm = d.perm;
     const int hi = d.h_cur, ho = 1 - d.h_cur;
     a.hin_cnt = d.hcnt[hi];
-    a.hin_pid = d.hpid[hi];
-    a.hin_d = (const typename PR::T*)d.hd[hi];
+    a.hin = (const Spring<typename PR::T>*)d.hs[hi];
     a.hout_cnt = d.hcnt[ho];
-    a.hout_pid = d.hpid[ho];
-    a.hout_d = (typename PR::T*)d.hd[ho];
+    a.hout = (Spring<typename PR::T>*)d.hs[ho];
     a.key = d.key;
     a.rank = d.rank;
     a.cnt = d.cnt;
@@ -1026,12 +1009,12 @@ cudaError_t run_hist_canon(Domain& d) {
     const int hi = d.h_cur, ho = 1 - d.h_cur;
     if (d.precision == 0)
         k_hist_canon<double><<<nblk(d.n, 256), 256, 0, d.stream>>>(
-            d.n, d.ctrl, d.perm, d.hcnt[hi], d.hpid[hi], (const double*)d.hd[hi], d.hcnt[ho], d.hpid[ho],
-            (double*)d.hd[ho], d.cap, (uint32_t)d.maxc);
+            d.n, d.ctrl, d.perm, d.hcnt[hi], (const Spring<double>*)d.hs[hi], d.hcnt[ho], (Spring<double>*)d.hs[ho], d.cap,
+            (uint32_t)d.maxc);
     else
         k_hist_canon<float><<<nblk(d.n, 256), 256, 0, d.stream>>>(
-            d.n, d.ctrl, d.perm, d.hcnt[hi], d.hpid[hi], (const float*)d.hd[hi], d.hcnt[ho], d.hpid[ho],
-            (float*)d.hd[ho], d.cap, (uint32_t)d.maxc);
+            d.n, d.ctrl, d.perm, d.hcnt[hi], (const Spring<float>*)d.hs[hi], d.hcnt[ho], (Spring<float>*)d.hs[ho], d.cap,
+            (uint32_t)d.maxc);
     DEM_LAUNCH_CHECK();
     return cudaSuccess;
 }
@@ -1041,12 +1024,12 @@ cudaError_t run_repack(Domain& od, Domain& d, const uint32_t* map, uint32_t n_ne
     const int ho = 1 - od.h_cur;   // canonical springs of the old domain (run_hist_canon)
     if (d.precision == 0)
         k_repack<PF64><<<nblk(n_new, 256), 256, 0, d.stream>>>(
-            n_new, map, od.S64[0], od.S64[1], od.ctrl, od.hcnt[ho], od.hpid[ho], (const double*)od.hd[ho], od.cap,
-            d.S64[1], d.hcnt[0], d.hpid[0], (double*)d.hd[0], d.cap, (uint32_t)d.maxc);
+            n_new, map, od.S64[0], od.S64[1], od.ctrl, od.hcnt[ho], (const Spring<double>*)od.hs[ho], od.cap, d.S64[1],
+            d.hcnt[0], (Spring<double>*)d.hs[0], d.cap, (uint32_t)d.maxc);
     else
         k_repack<PF32><<<nblk(n_new, 256), 256, 0, d.stream>>>(
-            n_new, map, od.S32[0], od.S32[1], od.ctrl, od.hcnt[ho], od.hpid[ho], (const float*)od.hd[ho], od.cap,
-            d.S32[1], d.hcnt[0], d.hpid[0], (float*)d.hd[0], d.cap, (uint32_t)d.maxc);
+            n_new, map, od.S32[0], od.S32[1], od.ctrl, od.hcnt[ho], (const Spring<float>*)od.hs[ho], od.cap, d.S32[1],
+            d.hcnt[0], (Spring<float>*)d.hs[0], d.cap, (uint32_t)d.maxc);
     DEM_LAUNCH_CHECK();
     return cudaSuccess;
 }

@@ -1,33 +1,27 @@
 // List mode (re-sort only after some particle moved skin/2): the force pass over the
-// neighbour lists built at each sort (the lists themselves: dem_nlist.cu).
+// neighbour lists built at each sort (the lists and tiles themselves: dem_nlist.cu).
 //
-//   k_list   steps 5-8 and 1 for one thread per stored particle. Phase 1 keeps the list
-//            entries that pass the contact prefilter as a 64-bit mask; phase 2 runs the
-//            lanes of a warp in lockstep over their masks (contact decision, Eq. 1 or
-//            Eqs. 2-10, the spring); then the walls the last sort found within reach
-//            (step 8), gravity, the update (step 1) and the displacement test that
-//            decides whether this step ends with a sort.
+//   k_list   steps 5-8 and 1 for one thread block per tile of consecutive stored particles,
+//            one thread per particle. The tile's particles and its halo (the particles
+//            outside it that are on some list of the tile, found at the sort) are copied
+//            to shared memory; phase 1 keeps the list entries that pass the contact
+//            prefilter as a 64-bit mask; phase 2 takes them one after another (contact
+//            decision, Eq. 1 or Eqs. 2-10, the spring); then the walls the last sort found
+//            within reach (step 8), gravity, the update (step 1) and the displacement test
+//            that decides whether this step ends with a sort.
 //
 // Every particle evaluates all of its contacts (each pair twice, once from each side, with
 // arithmetic that makes the two results exact negatives), so a step is one pass with no
-// exchange between particles; springs are stored per particle, keyed by partner id. No
-// floating-point atomics: a particle's sums run in list order (ascending partner id), so
-// results depend neither on the block size nor on when the sorts happened.
+// exchange between particles; springs are stored per particle in list order, and a 64-bit
+// mask per particle says which list entries have one, so that a contact finds its spring by
+// counting bits. No floating-point atomics: a particle's sums run in list order (ascending
+// partner id), so results depend neither on the tile size nor on when the sorts happened.
 #include <algorithm>
 
 #include <cuda_runtime.h>
 
 #include "dem_domain.h"
 #include "dem_policy.cuh"
-
-// Minimum resident 256-thread blocks per SM of the list-mode force kernel: 4 caps it at 64
-// registers (measured on GB300, 4,194,304-sphere drum: 0.71 ms per pass at 64 registers,
-// 0.85 ms at 85; the kernel is bound by memory latency, so occupancy wins).
-#ifndef DEM_LIST_MIN_BLOCKS
-#define DEM_LIST_MIN_BLOCKS 4
-#endif
-
-
 
 namespace demgb {
 
@@ -36,19 +30,22 @@ struct ListArgs {
     using T = typename PR::T;
     const SceneDev* scenes;
     int nscenes;
-    uint32_t n, cap;
+    uint32_t cap, tile, hcap;
     int maxc, stiffness;
     typename PR::State S0, S1;   // the two state sets; ctrl->cur names the current one
     CtrlDev* ctrl;
     const uint32_t* ncnt;        // list lengths
     const uint32_t* nl;          // list entries (stored index), slot-major
+    const uint2* nl4;            // the same as tile entries, four 16-bit indices per element
+    const uint32_t* halo;        // hcap stored indices per tile
+    const uint32_t* nhalo;       // how many of them; HALO_NONE: the tile has no entry indices
     const float4* ref;           // positions at the last sort
     int interval;                // sort at least every `interval` steps (0: never forced)
     const uint32_t* perm;
     const uint32_t* wmask;       // walls each particle can reach until the next sort
     uint32_t* hcnt[2];           // springs: ctrl->hcur names the buffer read, the other is written
-    uint32_t* hpid[2];
-    T* hd[2];
+    Spring<T>* hs[2];
+    uint64_t* hmask[2];          // list entries that have a spring
     StatusDev* st;
     double* dbgF;
     double* dbgT;
@@ -58,162 +55,222 @@ struct ListArgs {
 
 // ------------------------------------------------------------------- force pass
 
-// MODEL: 0 the practical law, 1 the simple law (Eq. 1), 2 the practical law with the
-// scene's optional terms. EVAL: forces and torques by id instead of the update.
+// MODEL: 0 the practical law with linear stiffness, 1 the simple law (Eq. 1), 2 the practical
+// law with the scene's optional terms, 3 the practical law with Hertz stiffness (the paper's
+// two stiffnesses have a variant each: the other's constants would take registers).
+// EVAL: forces and torques by id instead of the update.
 template <class PR, int MODEL, bool EVAL>
-__global__ void __launch_bounds__(256, DEM_LIST_MIN_BLOCKS) k_list(ListArgs<PR> a) {
+__global__ void __launch_bounds__(DEM_TILE_MAX, DEM_LIST_MIN_BLOCKS) k_list(ListArgs<PR> a) {
     using T = typename PR::T;
     constexpr bool PRACT = MODEL != 1;
     constexpr bool TERMS = MODEL == 2;
+    constexpr int STIFF = MODEL == 2 ? 2 : (MODEL == 3 ? 1 : 0);
     const unsigned full = 0xffffffffu;
-    extern __shared__ uint32_t smem[];
+    extern __shared__ __align__(16) unsigned char t_mem[];
+    __shared__ uint32_t s_sum[3], s_max[3], s_flag;   // counters of the block; bits for ctrl->rebuild
+    __shared__ int s_void;
+    __shared__ __align__(16) unsigned char s_law[64];
     if (!EVAL && a.loop && a.ctrl->stop != LOOP_GO) return;   // (written between passes only)
-    // a void step (an earlier launch overflowed): nothing to do; one decision per warp
-    if (!EVAL && __any_sync(full, (a.ctrl->rebuild & DEM_HALT) != 0)) return;
+    const uint32_t tid = threadIdx.x, lane = tid & 31u;
+    if (tid == 0) s_void = a.ctrl->rebuild & DEM_HALT;
+    if (tid < 3) s_sum[tid] = s_max[tid] = 0u;
+    if (tid == 3) s_flag = 0u;
+    __syncthreads();
+    if (!EVAL && s_void) return;   // an earlier launch (or another block) overflowed: a void step
     const int cur = a.ctrl->cur;
     const typename PR::State A = cur ? a.S1 : a.S0;
     const typename PR::State B = cur ? a.S0 : a.S1;
     const bool pv = a.ctrl->perm_valid != 0;
     const int hi = a.ctrl->hcur, ho = 1 - hi;
-    if (!EVAL && blockIdx.x == 0 && threadIdx.x == 0) {
+    if (!EVAL && blockIdx.x == 0 && tid == 0) {
         a.ctrl->hlast = ho;
         if (a.interval > 0 && a.ctrl->since + 1 >= a.interval) atomicOr(&a.ctrl->rebuild, 1);
     }
-    const uint32_t* __restrict__ hin_cnt = hi ? a.hcnt[1] : a.hcnt[0];
-    const uint32_t* __restrict__ hin_pid = hi ? a.hpid[1] : a.hpid[0];
-    const T* __restrict__ hin_d = hi ? a.hd[1] : a.hd[0];
+    const Spring<T>* __restrict__ hin = hi ? a.hs[1] : a.hs[0];
     uint32_t* __restrict__ hout_cnt = ho ? a.hcnt[1] : a.hcnt[0];
-    uint32_t* __restrict__ hout_pid = ho ? a.hpid[1] : a.hpid[0];
-    T* __restrict__ hout_d = ho ? a.hd[1] : a.hd[0];
-    const uint32_t tid = threadIdx.x, bd = blockDim.x, lane = tid & 31u;
-    const uint32_t maxc = (uint32_t)a.maxc;
-    uint32_t* s_oid = smem;   // [maxc][bd] partner ids of each particle's stored springs
-    const uint32_t q = blockIdx.x * bd + tid;
+    Spring<T>* __restrict__ hout = ho ? a.hs[1] : a.hs[0];
+    uint64_t* __restrict__ mout = ho ? a.hmask[1] : a.hmask[0];
+    const uint32_t maxc = (uint32_t)a.maxc, E = a.tile + a.hcap;
     const size_t cap = a.cap;
-    uint32_t c_pp = 0, c_wc = 0, c_clamp = 0, c_nnew = 0;
-    float c_maxov = 0.f, c_disp2 = 0.f;
-    const bool valid = q < a.n;
-    const int sidx = valid ? scene_of(a.scenes, a.nscenes, q) : 0;
-    const SceneDev& S = a.scenes[sidx];
-    const bool live = valid && S.active;
+    const SceneDev& S = a.scenes[scene_of_tile(a.scenes, a.nscenes, blockIdx.x)];
+    const uint32_t off = (blockIdx.x - S.t0) * a.tile;
+    const uint32_t q = S.p0 + off + tid;
+    const bool valid = off + tid < S.np;
     uint32_t src = 0, cnt_old = 0, m = 0;
+    uint32_t om_lo = 0, om_hi = 0;   // list entries that have a stored spring
     if (valid) {
         src = pv ? __ldg(&a.perm[q]) : q;
-        if (live) m = min(__ldg(&a.ncnt[q]), (uint32_t)DEM_LIST_CAP);
-        if (PRACT || !S.active) cnt_old = min(__ldg(&hin_cnt[src]), maxc);
-        // the list and the stored springs stream from DRAM: start every line fill now, so
-        // that the loads below do not wait for them one after another
-        for (uint32_t k = 0; k < m; ++k) prefetch_l1(&a.nl[k * cap + q]);
-        for (uint32_t k = 0; k < cnt_old; ++k) prefetch_l1(&hin_pid[k * cap + src]);
-        for (uint32_t k = 0; k < cnt_old; ++k)
-            for (int c = 0; c < 3; ++c) prefetch_l1(&hin_d[(c * (size_t)maxc + k) * cap + src]);
+        if (PRACT || !S.active) {
+            cnt_old = min(__ldg(&(hi ? a.hcnt[1] : a.hcnt[0])[src]), maxc);
+            const uint2 u = __ldg((const uint2*)&(hi ? a.hmask[1] : a.hmask[0])[q]);
+            om_lo = u.x;
+            om_hi = u.y;
+        }
     }
-    // ---- phase 1: list entries that pass the prefilter
-    uint64_t near_mask = 0;
-    if (live) near_mask = PR::scan_list(A, PR::load(A, q), S, a.nl, m, cap, q);
-    for (uint32_t k = 0; k < cnt_old; ++k) s_oid[k * bd + tid] = __ldg(&hin_pid[k * cap + src]);
-    __syncwarp();
-    if (valid && !live) {
+    if (!S.active) {
         // frozen scene: carry state and springs unchanged
+        if (!valid) return;
         if (!EVAL) {
             PR::store(B, q, PR::load(A, q));
-            for (uint32_t k = 0; k < cnt_old; ++k) {
-                hout_pid[k * cap + q] = s_oid[k * bd + tid];
-                for (int c = 0; c < 3; ++c)
-                    hout_d[(c * (size_t)maxc + k) * cap + q] = hin_d[(c * (size_t)maxc + k) * cap + src];
-            }
+            for (uint32_t k = 0; k < cnt_old; ++k) hout[k * cap + q] = hin[k * cap + src];
             hout_cnt[q] = cnt_old;
+            *(uint2*)&mout[q] = make_uint2(om_lo, om_hi);
         } else {
             hout_cnt[q] = 0;
         }
+        return;
     }
-    // ---- phase 2: the lanes of a warp in lockstep over their near candidates
-    T mi = T(0);
-    V3<T> F = mk(T(0), T(0), T(0)), Tq = mk(T(0), T(0), T(0));
-    uint32_t nnew = 0;
-    {
-        const uint32_t nnear = (uint32_t)__popcll(near_mask);
-        const uint32_t kmax = __reduce_max_sync(full, nnear);
-        typename PR::Self me{};
-        Law<T> L{};
-        if (live) {
-            me = PR::load(A, q);
-            L = law_of(S, a.stiffness, T());
-            mi = PR::mass(S, me.r);
+    // ---- the tile and its halo into shared memory
+    const uint32_t nh = __ldg(&a.nhalo[blockIdx.x]);
+    const bool direct = nh == HALO_NONE;   // (more halo than fits: partners are read from global memory)
+    if (valid) {
+        m = min(__ldg(&a.ncnt[q]), (uint32_t)DEM_LIST_CAP);
+        PR::tile_fetch(A, q, t_mem, E, tid);
+        if (!direct) {
+            // the list and the stored springs stream from DRAM: start their line fills now
+            for (uint32_t k = 0; k < m; k += 4) prefetch_l1(&a.nl4[(size_t)(k >> 2) * cap + q]);
         }
+        for (uint32_t k = 0; k < cnt_old; ++k) prefetch_l1(&hin[k * cap + src]);
+    }
+    if (!direct) {
+        const uint32_t* __restrict__ halo = a.halo + (size_t)blockIdx.x * a.hcap;
+        for (uint32_t k = tid; k < nh; k += blockDim.x) PR::tile_fetch(A, __ldg(&halo[k]), t_mem, E, a.tile + k);
+    }
+    if (tid == 0) PR::put_law(law_of(S, a.stiffness, T()), s_law);
+    copies_done();
+    __syncthreads();
+    uint32_t c_pp = 0, c_wc = 0, c_clamp = 0, c_nnew = 0;
+    float c_maxov = 0.f, c_disp2 = 0.f;
+    if (valid) {
+        const typename PR::Self me = PR::tile_self(A, q, t_mem, E, tid);
+        // ---- phase 1: list entries that pass the prefilter (near[0]: entries 0-31, near[1]: 32-63)
+        uint32_t near0 = 0, near1 = 0;
+        {
+            const float4 p = PR::pre(me);
+            const float eps = PR::pre_eps(S, p);
+            if (!direct) {
+                const uint2* lp = a.nl4 + q;
+                const float4* t4 = (const float4*)t_mem;
+                for (uint32_t k = 0; k < m; k += 4, lp += cap) {
+                    const uint2 u = __ldg(lp);
+                    uint32_t b = near_f(p, t4[u.x & 0xffffu], eps) ? 1u : 0u;
+                    b |= near_f(p, t4[u.x >> 16], eps) ? 2u : 0u;
+                    b |= near_f(p, t4[u.y & 0xffffu], eps) ? 4u : 0u;
+                    b |= near_f(p, t4[u.y >> 16], eps) ? 8u : 0u;
+                    if (k < 32) near0 |= b << k;
+                    else near1 |= b << (k - 32);
+                }
+                // (the last element is padded)
+                if (m < 32) near0 &= (1u << m) - 1u;
+                else if (m < 64) near1 &= (1u << (m - 32)) - 1u;
+            } else {
+                for (uint32_t k = 0; k < m; ++k)
+                    if (near_f(p, PR::pre(A, __ldg(&a.nl[k * cap + q])), eps)) {
+                        if (k < 32) near0 |= 1u << k;
+                        else near1 |= 1u << (k - 32);
+                    }
+            }
+        }
+        // ---- phase 2: the near candidates, in list order
+        const Law<T> L = law_of(S, a.stiffness, T());
+        const T mi = PR::mass(S, me.r);
         const T ri = (T)me.r;
-        for (uint32_t k = 0; k < kmax; ++k) {
-            if (!(live && k < nnear)) continue;
-            const int e = __ffsll((long long)near_mask) - 1;
-            near_mask &= near_mask - 1;
-            const uint32_t j = __ldg(&a.nl[(size_t)e * cap + q]);
+        V3<T> F = mk(T(0), T(0), T(0)), Tq = mk(T(0), T(0), T(0));
+        uint32_t nnew = 0;
+        uint32_t om = om_lo, nm = 0, nm_lo = 0;
+        const Spring<T>* hp = hin + src;   // slots of the mask word's springs start here
+        Spring<T>* op = hout + q;
+        uint32_t e0 = 0;
+        for (;;) {
+            if (near0 == 0) {
+                // the upper mask word (a list of more than 32 entries)
+                if (e0 != 0 || near1 == 0) break;
+                e0 = 32;
+                near0 = near1;
+                hp += (size_t)__popc(om_lo) * cap;
+                om = om_hi;
+                nm_lo = nm;
+                nm = 0;
+            }
+            const uint32_t e = (uint32_t)__ffs((int)near0) - 1u;
+            const uint32_t bit = 1u << e;
+            near0 &= near0 - 1u;
+            typename PR::Partner pj;
+            if (!direct)
+                pj = PR::tile_partner(
+                    A, t_mem, E, __ldg((const uint16_t*)(a.nl4 + (size_t)((e0 + e) >> 2) * cap + q) + (e & 3u)));
+            else
+                pj = PR::load_partner(A, __ldg(&a.nl[(size_t)(e0 + e) * cap + q]));
             V3<T> n;
             T delta;
             float rj;
-            const typename PR::Partner pj = PR::load_partner(A, j);
             if (!PR::exact_p(A, pj, me, n, delta, rj)) continue;
-            const uint32_t gid = pj.id;
             V3<T> vj, wj;
             PR::partner_vw(pj, vj, wj);
-            const V3<T> v = me.v - vj;
+            const V3<T> v = PR::self_v(me, t_mem, E, tid) - vj;
+            const Law<T> Lc = PR::law(L, s_law);
             if (PRACT) {
+                const V3<T> wi = PR::self_w(me, t_mem, E, tid);
+                V3<T> dold = mk(T(0), T(0), T(0));
+                if (om & bit) {
+                    const Spring<T> r = load_spring(hp + (size_t)__popc(om & (bit - 1u)) * cap);
+                    dold = mk(r.x, r.y, r.z);
+                }
                 const T rjT = (T)rj;
-                const V3<T> rw = mk(sym_madd(ri, me.w.x, rjT, wj.x), sym_madd(ri, me.w.y, rjT, wj.y),
-                                    sym_madd(ri, me.w.z, rjT, wj.z));
+                const V3<T> rw = mk(sym_madd(ri, wi.x, rjT, wj.x), sym_madd(ri, wi.y, rjT, wj.y),
+                                    sym_madd(ri, wi.z, rjT, wj.z));
                 const T mj = PR::mass(S, rj);
                 const T meff = law_div(mi * mj, mi + mj);
-                const T Reff = law_div(ri * rjT, ri + rjT);
-                const V3<T> dold = find_spring(s_oid, bd, tid, cnt_old, gid, hin_d, (size_t)maxc, cap, src);
+                const T Reff = (STIFF == 0) ? T(0) : law_div(ri * rjT, ri + rjT);
                 V3<T> Fc, Ftc, dnew, Mr;
-                law_practical<TERMS>(L, n, delta, v, rw, Reff, meff, dold, Fc, Ftc, dnew, me.w - wj, Mr);
+                law_practical<TERMS, STIFF>(Lc, n, delta, v, rw, Reff, meff, dold, Fc, Ftc, dnew, wi - wj, Mr);
                 F = F + Fc;
                 Tq = Tq + cross(n, Ftc) * ri;
                 if (TERMS) Tq = Tq + Mr;
                 if (nnew < maxc) {
-                    hout_pid[nnew * cap + q] = gid;
-                    hout_d[(0 * (size_t)maxc + nnew) * cap + q] = dnew.x;
-                    hout_d[(1 * (size_t)maxc + nnew) * cap + q] = dnew.y;
-                    hout_d[(2 * (size_t)maxc + nnew) * cap + q] = dnew.z;
+                    store_spring(op, dnew, pj.id);
+                    op += cap;
+                    nm |= bit;
                 }
             } else {
-                F = F + law_simple(L, n, delta, v);
-                if (EVAL && nnew < maxc) hout_pid[nnew * cap + q] = gid;
+                F = F + law_simple(Lc, n, delta, v);
+                if (EVAL && nnew < maxc) {
+                    store_spring(op, mk(T(0), T(0), T(0)), pj.id);
+                    op += cap;
+                }
             }
             ++nnew;
-            ++c_pp;
             c_maxov = fmaxf(c_maxov, (float)delta);
         }
-    }
-    if (live) {
-        const typename PR::Self me = PR::load(A, q);
-        const Law<T> L = law_of(S, a.stiffness, T());
-        const T ri = (T)me.r;
-        // ---- walls (step 8), those the last sort found within reach
+        c_pp = nnew;
+        const typename PR::Self me2 = PR::tile_again(me, t_mem, E, tid);
+        // ---- walls (step 8), those the last sort found within reach; their springs follow
+        // the particles' ones
+        const uint32_t w_first = (uint32_t)(__popc(om_lo) + __popc(om_hi));
         for (uint32_t wm = __ldg(&a.wmask[q]); wm; wm &= wm - 1) {
             const int w = __ffs(wm) - 1;
             const WallDev& W = S.walls[w];
             V3<T> n, cp;
             T delta;
-            if (!PR::wall(W, me, S, n, delta, cp)) continue;
-            const V3<T> v = me.v - PR::wall_vel(W, cp);
+            if (!PR::wall(W, me2, S, n, delta, cp)) continue;
+            const V3<T> v = me2.v - PR::wall_vel(W, cp);
             const uint32_t gid = DEM_WALL_BASE + (uint32_t)w;
             if (PRACT) {
-                const V3<T> rw = me.w * ri;
-                const V3<T> dold = find_spring(s_oid, bd, tid, cnt_old, gid, hin_d, (size_t)maxc, cap, src);
+                const V3<T> rw = me2.w * ri;
+                V3<T> dold = mk(T(0), T(0), T(0));
+                for (uint32_t k = w_first; k < cnt_old; ++k) {
+                    const Spring<T> r = load_spring(&hin[k * cap + src]);
+                    if (r.pid == gid) dold = mk(r.x, r.y, r.z);
+                }
                 V3<T> Fc, Ftc, dnew, Mr;
-                law_practical<TERMS>(L, n, delta, v, rw, ri, mi, dold, Fc, Ftc, dnew, me.w - PR::wall_omega(W), Mr);
+                law_practical<TERMS, STIFF>(L, n, delta, v, rw, ri, mi, dold, Fc, Ftc, dnew, me2.w - PR::wall_omega(W), Mr);
                 F = F + Fc;
                 Tq = Tq + cross(n, Ftc) * ri;
                 if (TERMS) Tq = Tq + Mr;
-                if (nnew < maxc) {
-                    hout_pid[nnew * cap + q] = gid;
-                    hout_d[(0 * (size_t)maxc + nnew) * cap + q] = dnew.x;
-                    hout_d[(1 * (size_t)maxc + nnew) * cap + q] = dnew.y;
-                    hout_d[(2 * (size_t)maxc + nnew) * cap + q] = dnew.z;
-                }
+                if (nnew < maxc) store_spring(&hout[nnew * cap + q], dnew, gid);
             } else {
                 F = F + law_simple(L, n, delta, v);
-                if (EVAL && nnew < maxc) hout_pid[nnew * cap + q] = gid;
+                if (EVAL && nnew < maxc) store_spring(&hout[nnew * cap + q], mk(T(0), T(0), T(0)), gid);
             }
             ++nnew;
             ++c_wc;
@@ -221,10 +278,11 @@ __global__ void __launch_bounds__(256, DEM_LIST_MIN_BLOCKS) k_list(ListArgs<PR> 
         }
         if (nnew > maxc) {
             raise_status(a.st, ST_CAPACITY, (int32_t)q);
-            if (!EVAL && a.halt) atomicOr(&a.ctrl->rebuild, DEM_HALT);
+            if (!EVAL && a.halt) atomicOr(&s_flag, DEM_HALT);
         }
         c_nnew = nnew;
         if (PRACT || EVAL) hout_cnt[q] = min(nnew, maxc);
+        if (PRACT && !EVAL) *(uint2*)&mout[q] = e0 ? make_uint2(nm_lo, nm) : make_uint2(nm, 0u);
         // gravity, once per particle
         {
             const T gx = sizeof(T) == 8 ? (T)S.g[0] : (T)S.g_f[0];
@@ -233,13 +291,13 @@ __global__ void __launch_bounds__(256, DEM_LIST_MIN_BLOCKS) k_list(ListArgs<PR> 
             F = F + mk(gx, gy, gz) * mi;
         }
         if (EVAL) {
-            const size_t o = 3 * (size_t)me.id;
+            const size_t o = 3 * (size_t)me2.id;
             if (a.dbgF) { a.dbgF[o] = F.x; a.dbgF[o + 1] = F.y; a.dbgF[o + 2] = F.z; }
             if (a.dbgT) { a.dbgT[o] = Tq.x; a.dbgT[o + 1] = Tq.y; a.dbgT[o + 2] = Tq.z; }
         } else {
             bool clamped = false, finite = true;
             float4 pnew;
-            PR::integrate(B, q, me, F, Tq, S, mi, clamped, finite, pnew);
+            PR::integrate(B, q, me2, F, Tq, S, mi, clamped, finite, pnew);
             if (!finite) raise_status(a.st, ST_NONFINITE, (int32_t)q);
             c_clamp = clamped ? 1u : 0u;
             c_disp2 = pnew.w;
@@ -247,29 +305,38 @@ __global__ void __launch_bounds__(256, DEM_LIST_MIN_BLOCKS) k_list(ListArgs<PR> 
             // this step end with a sort and new lists
             const float4 r0 = __ldg(&a.ref[q]);
             const float ex = pnew.x - r0.x, ey = pnew.y - r0.y, ez = pnew.z - r0.z;
-            if (ex * ex + ey * ey + ez * ez > S.thresh2_f || !finite) atomicOr(&a.ctrl->rebuild, 1);
+            if (ex * ex + ey * ey + ez * ez > S.thresh2_f || !finite) atomicOr(&s_flag, 1u);
         }
     }
-    // warp-aggregated counters (every lane reaches this point)
-    const uint32_t s_pp = __reduce_add_sync(full, c_pp);
-    const uint32_t s_wc = __reduce_add_sync(full, c_wc);
-    const uint32_t s_cl = __reduce_add_sync(full, c_clamp);
-    const uint32_t s_mx = __reduce_max_sync(full, c_nnew);
-    const uint32_t s_ov = __reduce_max_sync(full, __float_as_uint(c_maxov));
-    const uint32_t s_dp = __reduce_max_sync(full, __float_as_uint(c_disp2));
+    // counters of the block (every thread reaches this point): one global atomic per counter
+    // and block; one per warp meant 131,072 x 5 atomics on one 32-byte sector for the drum
+    const uint32_t w_pp = __reduce_add_sync(full, c_pp);
+    const uint32_t w_wc = __reduce_add_sync(full, c_wc);
+    const uint32_t w_cl = __reduce_add_sync(full, c_clamp);
+    const uint32_t w_mx = __reduce_max_sync(full, c_nnew);
+    const uint32_t w_ov = __reduce_max_sync(full, __float_as_uint(c_maxov));
+    const uint32_t w_dp = __reduce_max_sync(full, __float_as_uint(c_disp2));
     if (lane == 0) {
-        if (s_pp) atomicAdd(&a.st->live.ncontacts, s_pp);
-        if (s_wc) atomicAdd(&a.st->live.nwallc, s_wc);
-        if (s_cl) atomicAdd(&a.st->live.clamped, s_cl);
-        if (s_mx) atomicMax(&a.st->live.max_nnew, s_mx);
-        if (s_ov) atomicMax(&a.st->live.max_overlap_bits, s_ov);
-        if (s_dp) atomicMax(&a.st->live.max_disp2_bits, s_dp);
+        if (w_pp) atomicAdd(&s_sum[0], w_pp);
+        if (w_wc) atomicAdd(&s_sum[1], w_wc);
+        if (w_cl) atomicAdd(&s_sum[2], w_cl);
+        if (w_mx) atomicMax(&s_max[0], w_mx);
+        if (w_ov) atomicMax(&s_max[1], w_ov);
+        if (w_dp) atomicMax(&s_max[2], w_dp);
+    }
+    __syncthreads();
+    if (tid == 0) {
+        if (s_sum[0]) atomicAdd(&a.st->live.ncontacts, s_sum[0]);
+        if (s_sum[1]) atomicAdd(&a.st->live.nwallc, s_sum[1]);
+        if (s_sum[2]) atomicAdd(&a.st->live.clamped, s_sum[2]);
+        if (s_max[0]) atomicMax(&a.st->live.max_nnew, s_max[0]);
+        if (s_max[1]) atomicMax(&a.st->live.max_overlap_bits, s_max[1]);
+        if (s_max[2]) atomicMax(&a.st->live.max_disp2_bits, s_max[2]);
+        if (s_flag) atomicOr(&a.ctrl->rebuild, (int)s_flag);
     }
 }
 
 // ======================================================================= launchers
-static inline uint32_t nblk(uint32_t n, uint32_t b) { return (n + b - 1) / b; }
-
 #define DEM_LAUNCH_CHECK()                          \
     do {                                            \
         ++d.launches;                               \
@@ -284,8 +351,9 @@ static cudaError_t force_list_impl(Domain& d, const typename PR::State& S0, cons
     ListArgs<PR> a;
     a.scenes = d.d_scenes;
     a.nscenes = d.nscenes;
-    a.n = d.n;
     a.cap = d.cap;
+    a.tile = d.tile;
+    a.hcap = halo_cap(d.tile);
     a.maxc = d.maxc;
     a.stiffness = d.stiffness;
     a.S0 = S0;
@@ -293,34 +361,37 @@ static cudaError_t force_list_impl(Domain& d, const typename PR::State& S0, cons
     a.ctrl = d.ctrl;
     a.ncnt = d.ncnt;
     a.nl = d.nl;
+    a.nl4 = d.nl4;
+    a.halo = d.halo;
+    a.nhalo = d.nhalo;
     a.ref = d.ref;
     a.interval = d.interval;
     a.perm = d.perm;
     a.wmask = d.wmask;
     for (int k = 0; k < 2; ++k) {
         a.hcnt[k] = d.hcnt[k];
-        a.hpid[k] = d.hpid[k];
-        a.hd[k] = (T*)d.hd[k];
+        a.hs[k] = (Spring<T>*)d.hs[k];
+        a.hmask[k] = d.hmask[k];
     }
     a.st = d.st;
     a.dbgF = dbgF;
     a.dbgT = dbgT;
     a.halt = d.regrow;
     a.loop = d.in_loop;
-    const uint32_t b = (uint32_t)d.block;
-    const size_t smem = (size_t)d.maxc * b * sizeof(uint32_t);
-    const int model = d.model != 0 ? 1 : (d.terms != 0 ? 2 : 0);
+    const size_t smem = (size_t)(a.tile + a.hcap) * PR::TILE_BYTES;
+    const int model = d.model != 0 ? 1 : (d.terms != 0 ? 2 : (d.stiffness != 0 ? 3 : 0));
     auto launch = [&](auto kern) -> cudaError_t {
-        if (smem > 48 * 1024) {
+        if (smem > 32 * 1024) {   // (with the static shared memory above the default limit)
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        kern<<<nblk(d.n, b), b, smem, d.stream>>>(a);
+        kern<<<d.ntiles, d.tile, smem, d.stream>>>(a);
         return cudaSuccess;
     };
     cudaError_t e;
     if (model == 0) e = eval ? launch(k_list<PR, 0, true>) : launch(k_list<PR, 0, false>);
     else if (model == 2) e = eval ? launch(k_list<PR, 2, true>) : launch(k_list<PR, 2, false>);
+    else if (model == 3) e = eval ? launch(k_list<PR, 3, true>) : launch(k_list<PR, 3, false>);
     else e = eval ? launch(k_list<PR, 1, true>) : launch(k_list<PR, 1, false>);
     if (e != cudaSuccess) return e;
     DEM_LAUNCH_CHECK();

@@ -108,6 +108,148 @@ __global__ void __launch_bounds__(256) k_nlist(uint32_t n, const SceneDev* scene
     }
 }
 
+// ------------------------------------------------------------------ tiles
+// A tile is `tile` consecutive stored particles of one scene (the last of a scene may hold
+// fewer): the work of one block of the force pass, which keeps the tile and its halo in
+// shared memory. One block here per tile: the stored indices outside the tile that occur on
+// its lists are collected in a hash table in shared memory, sorted (the force pass then
+// copies them in nearly coalesced runs), and every list entry is rewritten as a 16-bit index
+// into (tile, halo). A tile whose halo does not fit is marked HALO_NONE. The same pass marks
+// the list entries that have a stored spring: a particle's springs and its list are both in
+// ascending partner id, so it is a merge. A spring whose partner is not on the new list (the
+// pair has moved apart by more than the skin) is dropped, and the ones behind it move up.
+constexpr uint32_t TILE_HASH = 2048;   // entries: a tile inserts at most halo_cap + 512 before it stops
+constexpr uint32_t TILE_SORT = 1024;   // >= halo_cap, power of two
+
+template <class PR>
+__global__ void __launch_bounds__(512) k_tile(const SceneDev* scenes, int nscenes, uint32_t tile, uint32_t ntiles,
+                                              uint32_t hcap, typename PR::State S0, typename PR::State S1,
+                                              const CtrlDev* ctrl, int always, const uint32_t* __restrict__ ncnt,
+                                              const uint32_t* __restrict__ nl, uint2* __restrict__ nl4,
+                                              uint32_t* __restrict__ halo, uint32_t* __restrict__ nhalo, size_t cap,
+                                              const uint32_t* __restrict__ perm, uint32_t* hcnt0, uint32_t* hcnt1,
+                                              Spring<typename PR::T>* hs0, Spring<typename PR::T>* hs1, uint64_t* hm0,
+                                              uint64_t* hm1, uint32_t maxc) {
+    if (!always && ctrl->rebuild != 1) return;   // no sort this step (or a void step)
+    __shared__ uint32_t s_key[TILE_HASH], s_list[TILE_SORT];
+    __shared__ uint16_t s_val[TILE_HASH];
+    __shared__ uint32_t s_n;
+    const typename PR::State A = ctrl->cur ? S1 : S0;
+    const int hl = ctrl->hlast;
+    uint32_t* hcnt = hl ? hcnt1 : hcnt0;
+    Spring<typename PR::T>* hs = hl ? hs1 : hs0;
+    uint64_t* hm = hl ? hm1 : hm0;
+    const uint32_t tid = threadIdx.x, bd = blockDim.x;
+    for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+        const SceneDev& S = scenes[scene_of_tile(scenes, nscenes, t)];
+        const uint32_t off = (t - S.t0) * tile;
+        const uint32_t q0 = S.p0 + off, n = min(tile, S.np - off);
+        const uint32_t q = q0 + tid;
+        const bool valid = tid < n;
+        const uint32_t m = valid ? ncnt[q] : 0u;
+        for (uint32_t k = tid; k < TILE_HASH; k += bd) s_key[k] = 0xFFFFFFFFu;
+        for (uint32_t k = tid; k < TILE_SORT; k += bd) s_list[k] = 0xFFFFFFFFu;
+        if (tid == 0) s_n = 0u;
+        __syncthreads();
+        // ---- the halo; and the spring mask by a merge of the list with the stored springs
+        uint64_t mask = 0;
+        {
+            const uint32_t src = valid ? perm[q] : 0u;
+            const uint32_t c = valid ? min(hcnt[src], maxc) : 0u;
+            uint32_t o = 0, kept = 0, pid = c ? hs[src].pid : DEM_WALL_BASE;
+            for (uint32_t k = 0; k < m; ++k) {
+                const uint32_t j = nl[(size_t)k * cap + q];
+                if (o < c && pid < DEM_WALL_BASE) {
+                    const uint32_t idj = __ldg(&A.id[j]);
+                    while (o < c && pid < idj) {   // a partner that left the list
+                        ++o;
+                        pid = o < c ? hs[(size_t)o * cap + src].pid : DEM_WALL_BASE;
+                    }
+                    if (o < c && pid == idj) {
+                        if (kept != o) hs[(size_t)kept * cap + src] = hs[(size_t)o * cap + src];
+                        ++kept;
+                        mask |= 1ull << k;
+                        ++o;
+                        pid = o < c ? hs[(size_t)o * cap + src].pid : DEM_WALL_BASE;
+                    }
+                }
+                if (j - q0 >= n && *(volatile uint32_t*)&s_n <= hcap) {
+                    uint32_t h = (j * 2654435761u) >> 21;   // 11 bits
+                    for (;;) {
+                        const uint32_t old = atomicCAS(&s_key[h], 0xFFFFFFFFu, j);
+                        if (old == 0xFFFFFFFFu) {
+                            const uint32_t at = atomicAdd(&s_n, 1u);
+                            if (at < hcap) s_list[at] = j;
+                            break;
+                        }
+                        if (old == j) break;
+                        h = (h + 1) & (TILE_HASH - 1);
+                    }
+                }
+            }
+            while (o < c && pid < DEM_WALL_BASE) {   // partners beyond the list's last
+                ++o;
+                pid = o < c ? hs[(size_t)o * cap + src].pid : DEM_WALL_BASE;
+            }
+            if (kept != o) {   // the wall springs move up
+                for (; o < c; ++o, ++kept) hs[(size_t)kept * cap + src] = hs[(size_t)o * cap + src];
+                hcnt[src] = kept;
+            }
+            if (valid) hm[q] = mask;
+        }
+        __syncthreads();
+        const uint32_t nh = s_n;
+        if (nh > hcap) {
+            if (tid == 0) nhalo[t] = HALO_NONE;
+            __syncthreads();
+            continue;
+        }
+        uint32_t w = 32;
+        while (w < nh) w <<= 1;
+        for (uint32_t k = 2; k <= w; k <<= 1)
+            for (uint32_t j = k >> 1; j > 0; j >>= 1) {
+                for (uint32_t i = tid; i < w; i += bd) {
+                    const uint32_t o = i ^ j;
+                    if (o > i) {
+                        const uint32_t a = s_list[i], b = s_list[o];
+                        if ((a > b) == ((i & k) == 0)) {
+                            s_list[i] = b;
+                            s_list[o] = a;
+                        }
+                    }
+                }
+                __syncthreads();
+            }
+        for (uint32_t i = tid; i < nh; i += bd) {
+            const uint32_t j = s_list[i];
+            halo[(size_t)t * hcap + i] = j;
+            uint32_t h = (j * 2654435761u) >> 21;
+            while (s_key[h] != j) h = (h + 1) & (TILE_HASH - 1);
+            s_val[h] = (uint16_t)(tile + i);
+        }
+        if (tid == 0) nhalo[t] = nh;
+        __syncthreads();
+        for (uint32_t k = 0; k < m; k += 4) {
+            uint32_t e[4];
+#pragma unroll
+            for (uint32_t u = 0; u < 4; ++u) {
+                e[u] = tid;   // pad: the particle itself (the force pass masks it out)
+                if (k + u < m) {
+                    const uint32_t j = nl[(size_t)(k + u) * cap + q];
+                    if (j - q0 < n) e[u] = j - q0;
+                    else {
+                        uint32_t h = (j * 2654435761u) >> 21;
+                        while (s_key[h] != j) h = (h + 1) & (TILE_HASH - 1);
+                        e[u] = s_val[h];
+                    }
+                }
+            }
+            nl4[(size_t)(k >> 2) * cap + q] = make_uint2(e[0] | (e[1] << 16), e[2] | (e[3] << 16));
+        }
+        __syncthreads();   // the table is cleared by the next tile
+    }
+}
+
 // ======================================================================= launchers
 static inline uint32_t nblk(uint32_t n, uint32_t b) { return (n + b - 1) / b; }
 static inline uint32_t sgrid(const Domain& d, uint32_t n) {
@@ -129,6 +271,26 @@ cudaError_t run_lists(Domain& d) {
     else
         k_nlist<PF32><<<sgrid(d, d.n), 256, 0, d.stream>>>(d.n, d.d_scenes, d.nscenes, d.S32[0], d.S32[1], d.ctrl, d.skey,
                                                           d.cs, d.fin, d.ncnt, d.nl, d.cap, d.wmask, d.st);
+    DEM_LAUNCH_CHECK();
+    return run_tiles(d, false);
+}
+
+template <class PR>
+static void launch_tiles(Domain& d, const typename PR::State& S0, const typename PR::State& S1, bool always) {
+    using Sp = Spring<typename PR::T>;
+    const uint32_t g = std::max(1u, std::min(d.ntiles, (uint32_t)std::max(d.sort_blocks, 1)));
+    k_tile<PR><<<g, d.tile, 0, d.stream>>>(d.d_scenes, d.nscenes, d.tile, d.ntiles, halo_cap(d.tile), S0, S1, d.ctrl,
+                                           always ? 1 : 0, d.ncnt, d.nl, d.nl4, d.halo, d.nhalo, d.cap, d.perm,
+                                           d.hcnt[0], d.hcnt[1], (Sp*)d.hs[0], (Sp*)d.hs[1], d.hmask[0], d.hmask[1],
+                                           (uint32_t)d.maxc);
+}
+
+// The tiles of the lists just built (always: also when no sort is due, for springs that
+// were set after it).
+cudaError_t run_tiles(Domain& d, bool always) {
+    if (d.n == 0) return cudaSuccess;
+    if (d.precision == 0) launch_tiles<PF64>(d, d.S64[0], d.S64[1], always);
+    else launch_tiles<PF32>(d, d.S32[0], d.S32[1], always);
     DEM_LAUNCH_CHECK();
     return cudaSuccess;
 }

@@ -11,10 +11,6 @@
 
 // Paired FP32 instructions (two IEEE operations per instruction) in the float-float
 // contact test: 2% faster force pass on GB300, the same bits.
-// List entries whose prefilter loads are in flight together (phase 1 of the list pass).
-#ifndef DEM_SCAN_UNROLL
-#define DEM_SCAN_UNROLL 2
-#endif
 #ifndef DEM_PACKED_FF
 #define DEM_PACKED_FF 1
 #endif
@@ -23,6 +19,31 @@ namespace demgb {
 
 // L1 prefetch (PTX prefetch.global.L1): starts a line fill without holding a register.
 __device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
+
+// 16 bytes from global to shared memory without passing through registers (L2 only).
+__device__ __forceinline__ void copy16_async(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src));
+}
+__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// 16 bytes of shared memory read where the code says (volatile: a value that is needed once
+// per contact is read again instead of held in four registers).
+__device__ __forceinline__ float4 lds16(const void* p) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"((uint32_t)__cvta_generic_to_shared(p)));
+    return v;
+}
+
+// FP32 prefilter of two particles given as (x, y, z, r): conservative by eps, which bounds
+// the FP32 error of the coordinate differences and of the squared distance, so no pair in
+// contact is ever rejected.
+__device__ __forceinline__ bool near_f(float4 a, float4 b, float eps) {
+    const float ax = b.x - a.x, ay = b.y - a.y, az = b.z - a.z;
+    const float Re = (b.w + a.w) + eps;
+    return ax * ax + ay * ay + az * az < Re * Re;
+}
 
 // ======================================================================= FP64 policy
 struct PF64 {
@@ -73,16 +94,41 @@ struct PF64 {
             }
         }
     }
-    // Phase 1 from a neighbour list built at the last sort: bit k of the returned mask
-    // marks list entry k as in contact.
-    static __device__ __forceinline__ uint64_t scan_list(const State& s, const Self& me, const SceneDev&,
-                                                         const uint32_t* nl, uint32_t m, size_t cap, uint32_t q) {
-        uint64_t mask = 0;
-        for (uint32_t k = 0; k < m; ++k) {
-            const uint32_t j = __ldg(&nl[k * cap + q]);
-            if (touches(me, __ldg(&s.x[j]), __ldg(&s.y[j]), __ldg(&s.z[j]), __ldg(&s.r[j]))) mask |= 1ull << k;
-        }
-        return mask;
+    // Tile of the list-mode force pass: (x, y, z, r) of every entry rounded to FP32, and the
+    // stored index. The prefilter runs on the FP32 copies (the FP64 pipe is about 60 times
+    // slower on GB300); the decision and the law read the FP64 state.
+    static constexpr uint32_t TILE_BYTES = 20;
+    static __device__ __forceinline__ void tile_fetch(const State& s, uint32_t j, unsigned char* t, uint32_t E,
+                                                      uint32_t i) {
+        ((float4*)t)[i] = make_float4((float)__ldg(&s.x[j]), (float)__ldg(&s.y[j]), (float)__ldg(&s.z[j]),
+                                      __ldg(&s.r[j]));
+        ((uint32_t*)(t + 16 * E))[i] = j;
+    }
+    static __device__ __forceinline__ Self tile_self(const State& s, uint32_t q, const unsigned char*, uint32_t,
+                                                     uint32_t) {
+        return load(s, q);
+    }
+    static __device__ __forceinline__ Self tile_again(const Self& m, const unsigned char*, uint32_t, uint32_t) { return m; }
+    static __device__ __forceinline__ V3<double> self_v(const Self& m, const unsigned char*, uint32_t, uint32_t) {
+        return m.v;
+    }
+    static __device__ __forceinline__ V3<double> self_w(const Self& m, const unsigned char*, uint32_t, uint32_t) {
+        return m.w;
+    }
+    static __device__ __forceinline__ Law<double> law(const Law<double>& L, const unsigned char*) { return L; }
+    static __device__ __forceinline__ void put_law(const Law<double>&, unsigned char*) {}
+    // FP32 position and radius of a particle for the prefilter
+    static __device__ __forceinline__ float4 pre(const Self& m) {
+        return make_float4((float)m.x, (float)m.y, (float)m.z, m.r);
+    }
+    // prefilter margin: the scene's bounds the rounding for positions up to the domain's
+    // size; a particle that has left it far behind takes a margin of its own
+    static __device__ __forceinline__ float pre_eps(const SceneDev& S, float4 p) {
+        const float X = fmaxf(fabsf(p.x), fmaxf(fabsf(p.y), fabsf(p.z)));
+        return fmaxf(S.eps_f, 0x1p-20f * (X + 4.f * p.w));
+    }
+    static __device__ __forceinline__ float4 pre(const State& s, uint32_t j) {
+        return make_float4((float)__ldg(&s.x[j]), (float)__ldg(&s.y[j]), (float)__ldg(&s.z[j]), __ldg(&s.r[j]));
     }
     // Neighbour-list test: j may come within contact of i while both move less than
     // skin/2 (FP32 on the rounded positions, conservative by eps).
@@ -106,6 +152,10 @@ struct PF64 {
         o.id = __ldg(&s.id[j]);
         load_vw(s, j, o.v, o.w);
         return o;
+    }
+    static __device__ __forceinline__ Partner tile_partner(const State& s, const unsigned char* t, uint32_t E,
+                                                           uint32_t i) {
+        return load_partner(s, ((const uint32_t*)(t + 16 * E))[i]);
     }
     static __device__ __forceinline__ void partner_vw(const Partner& o, V3<double>& v, V3<double>& w) {
         v = o.v;
@@ -296,32 +346,68 @@ struct PF32 {
             ++cnt;
         }
     }
-    // Phase 1 from a neighbour list built at the last sort: bit k of the returned mask
-    // marks list entry k as passing the prefilter (two candidates in flight).
-    static __device__ __forceinline__ uint64_t scan_list(const State& s, const Self& me, const SceneDev& S,
-                                                         const uint32_t* nl, uint32_t m, size_t cap, uint32_t q) {
-        const float eps = S.eps_f;
-        uint64_t mask = 0;
-        uint32_t k = 0;
-        // (no L1 prefetch of the near candidates' payload: measured 9% slower here and 4%
-        // in the walk; the prefetched lines are evicted before phase 2 reads them)
-        for (; k + DEM_SCAN_UNROLL <= m; k += DEM_SCAN_UNROLL) {
-            uint32_t j[DEM_SCAN_UNROLL];
-            float4 pj[DEM_SCAN_UNROLL];
-#pragma unroll
-            for (int u = 0; u < DEM_SCAN_UNROLL; ++u) j[u] = __ldg(&nl[(k + u) * cap + q]);
-#pragma unroll
-            for (int u = 0; u < DEM_SCAN_UNROLL; ++u) pj[u] = __ldg(&s.P0[j[u]]);
-#pragma unroll
-            for (int u = 0; u < DEM_SCAN_UNROLL; ++u)
-                if (near(me, pj[u], eps)) mask |= 1ull << (k + u);
-        }
-        for (; k < m; ++k) {
-            const uint32_t j0 = __ldg(&nl[k * cap + q]);
-            if (near(me, __ldg(&s.P0[j0]), eps)) mask |= 1ull << k;
-        }
-        return mask;
+    // Tile of the list-mode force pass: the planes P0, P1, V, W of its entries.
+    static constexpr uint32_t TILE_BYTES = 64;
+    static __device__ __forceinline__ void tile_fetch(const State& s, uint32_t j, unsigned char* t, uint32_t E,
+                                                      uint32_t i) {
+        float4* p = (float4*)t + i;
+        copy16_async(p, &s.P0[j]);
+        copy16_async(p + E, &s.P1[j]);
+        copy16_async(p + 2 * E, &s.V[j]);
+        copy16_async(p + 3 * E, &s.W[j]);
     }
+    static __device__ __forceinline__ Self tile_self(const State&, uint32_t, const unsigned char* t, uint32_t E,
+                                                     uint32_t i) {
+        const float4* p = (const float4*)t + i;
+        const float4 p0 = p[0], p1 = p[E], v = p[2 * E], w = p[3 * E];
+        Self m;
+        m.hx = p0.x; m.hy = p0.y; m.hz = p0.z; m.r = p0.w;
+        m.lx = p1.x; m.ly = p1.y; m.lz = p1.z;
+        m.v = mk(v.x, v.y, v.z);
+        m.w = mk(w.x, w.y, w.z);
+        m.id = __float_as_uint(p1.w);
+        return m;
+    }
+    static __device__ __forceinline__ Self tile_again(const Self&, const unsigned char* t, uint32_t E, uint32_t i) {
+        const float4* p = (const float4*)t + i;
+        const float4 p0 = lds16(p), p1 = lds16(p + E), v = lds16(p + 2 * E), w = lds16(p + 3 * E);
+        Self m;
+        m.hx = p0.x; m.hy = p0.y; m.hz = p0.z; m.r = p0.w;
+        m.lx = p1.x; m.ly = p1.y; m.lz = p1.z;
+        m.v = mk(v.x, v.y, v.z);
+        m.w = mk(w.x, w.y, w.z);
+        m.id = __float_as_uint(p1.w);
+        return m;
+    }
+    // The own velocity and spin, and the law's constants, as phase 2 of the list pass needs
+    // them: read from the tile each time (held in registers they made the loop spill).
+    static __device__ __forceinline__ V3<float> self_v(const Self&, const unsigned char* t, uint32_t E, uint32_t i) {
+        const float4 v = lds16((const float4*)t + 2 * E + i);
+        return mk(v.x, v.y, v.z);
+    }
+    static __device__ __forceinline__ V3<float> self_w(const Self&, const unsigned char* t, uint32_t E, uint32_t i) {
+        const float4 v = lds16((const float4*)t + 3 * E + i);
+        return mk(v.x, v.y, v.z);
+    }
+    static __device__ __forceinline__ void put_law(const Law<float>& L, unsigned char* s) {
+        float4* p = (float4*)s;
+        p[0] = make_float4(L.dt, L.alpha, L.mu, L.kn);
+        p[1] = make_float4(L.kt, L.cn, L.ct, L.ksp);
+        p[2] = make_float4(L.kda, L.ksh, L.mu_roll, L.alpha_t);
+        p[3] = make_float4(L.kcoh_pi, __int_as_float(L.stiffness), __int_as_float(L.terms), 0.f);
+    }
+    static __device__ __forceinline__ Law<float> law(const Law<float>&, const unsigned char* s) {
+        const float4 a = lds16(s), b = lds16(s + 16), c = lds16(s + 32), d = lds16(s + 48);
+        Law<float> L;
+        L.dt = a.x; L.alpha = a.y; L.mu = a.z; L.kn = a.w;
+        L.kt = b.x; L.cn = b.y; L.ct = b.z; L.ksp = b.w;
+        L.kda = c.x; L.ksh = c.y; L.mu_roll = c.z; L.alpha_t = c.w;
+        L.kcoh_pi = d.x; L.stiffness = __float_as_int(d.y); L.terms = __float_as_int(d.z);
+        return L;
+    }
+    static __device__ __forceinline__ float4 pre(const Self& m) { return make_float4(m.hx, m.hy, m.hz, m.r); }
+    static __device__ __forceinline__ float pre_eps(const SceneDev& S, float4) { return S.eps_f; }
+    static __device__ __forceinline__ float4 pre(const State& s, uint32_t j) { return __ldg(&s.P0[j]); }
     // Neighbour-list test: j may come within contact of i while both move less than
     // skin/2 (FP32 on hi, conservative by eps).
     static __device__ __forceinline__ bool within(const State& s, const Self& me, uint32_t j, float reach_extra) {
@@ -342,6 +428,17 @@ struct PF32 {
         o.p1 = __ldg(&s.P1[j]);
         o.v = __ldg(&s.V[j]);
         o.w = __ldg(&s.W[j]);
+        o.id = __float_as_uint(o.p1.w);
+        return o;
+    }
+    static __device__ __forceinline__ Partner tile_partner(const State&, const unsigned char* t, uint32_t E,
+                                                           uint32_t i) {
+        const float4* p = (const float4*)t + i;
+        Partner o;
+        o.p0 = p[0];
+        o.p1 = p[E];
+        o.v = p[2 * E];
+        o.w = p[3 * E];
         o.id = __float_as_uint(o.p1.w);
         return o;
     }
@@ -612,14 +709,15 @@ struct PF32 {
     static __device__ __forceinline__ V3<double> spin(const Self& m) { return mk((double)m.w.x, (double)m.w.y, (double)m.w.z); }
 };
 
-// Load the stored tangential spring of slot k (partner ids are in shared memory).
+// Stored tangential spring of partner gid (partner ids are in shared memory).
 template <class T>
 __device__ __forceinline__ V3<T> find_spring(const uint32_t* s_oid, uint32_t bd, uint32_t tid, uint32_t cnt_old,
-                                             uint32_t gid, const T* hin_d, size_t maxc, size_t cap, uint32_t src) {
+                                             uint32_t gid, const Spring<T>* hin, size_t cap, uint32_t src) {
     for (uint32_t k = 0; k < cnt_old; ++k)
-        if (s_oid[k * bd + tid] == gid)
-            return mk(__ldg(&hin_d[(0 * maxc + k) * cap + src]), __ldg(&hin_d[(1 * maxc + k) * cap + src]),
-                      __ldg(&hin_d[(2 * maxc + k) * cap + src]));
+        if (s_oid[k * bd + tid] == gid) {
+            const Spring<T> r = load_spring(&hin[k * cap + src]);
+            return mk(r.x, r.y, r.z);
+        }
     return mk(T(0), T(0), T(0));
 }
 

@@ -22,18 +22,21 @@ from . import dem
 
 # device bytes of a batch, as dem_batch_device_bytes counts them: per particle two state
 # sets, two spring buffers of max_contacts slots, the sort arrays, the staging and map
-# buffers, and (list mode) the neighbour list of 64 entries with its count, reference
-# position and window maps; per cell the counts and the starts
+# buffers, and (list mode) the neighbour list of 64 entries as indices and tile entries with
+# its count, reference position, window maps, spring masks and share of the tiles' halos;
+# per cell the counts and the starts (list mode pads a grid by at most half); per scene of
+# list mode the halo of its last, partly filled tile
 LIST_CAP = 64
 BYTES_PER_CELL = 8
+TILE_BYTES = 4 * (768 + 1)
 
 
 def bytes_per_particle(precision: str = "fp32", max_contacts: int = 32, list_mode: bool = False) -> int:
     state, t = (68, 4) if precision == "fp32" else (80, 8)
     m = max_contacts or 32
-    b = 2 * state + 2 * (4 + 4 * m + t * 3 * m) + 20 + 76 + 4
+    b = 2 * state + 2 * (4 + 4 * t * m) + 20 + 76 + 4
     if list_mode:
-        b += 4 + 4 * LIST_CAP + 4 + 16 + 8
+        b += 4 + 6 * LIST_CAP + 4 + 16 + 8 + 16 + 17
     return b
 
 
@@ -58,6 +61,8 @@ def footprint(scene, precision="fp32", max_contacts: int = 32) -> int:
     for a in range(3):
         cells *= max(1, int(np.ceil((p.domain_hi[a] - p.domain_lo[a]) / p.cell_size)))
     per = bytes_per_particle(precision, max_contacts, p.resort_interval != 1)
+    if p.resort_interval != 1:
+        return per * scene.n + BYTES_PER_CELL * (cells + cells // 2 + 1) + TILE_BYTES
     return per * scene.n + BYTES_PER_CELL * cells
 
 
