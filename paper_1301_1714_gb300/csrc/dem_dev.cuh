@@ -19,6 +19,9 @@
 // Neighbour lists of list mode: at most DEM_LIST_CAP candidates per particle (one bit each
 // in the force pass's 64-bit mask); a fuller list is reported, never truncated silently.
 #define DEM_LIST_CAP 64
+// Largest tile of list mode per precision mode (particles, and threads of a block).
+#define DEM_TILE_MAX 512
+#define DEM_TILE_MAX_FP64 128
 // Cell order of list mode: bricks of 2^s x 2^s x 2^s cells, s at most DEM_LIST_BRICK_SHIFT
 // (0 = row-major). Each grid takes the largest s whose padding to whole bricks adds at most
 // 1/8 to its cell count.
@@ -64,7 +67,12 @@ struct SceneDev {
     double alpha_t;             // tangential damping factor
     double kcoh_pi;             // pi * cohesion energy density
     float mu_roll_f, alpha_t_f, kcoh_pi_f;
-    float pad3;
+    float nrkt_f;               // -1 / kt
+    double nrkt;
+    // positions inside [in_lo, in_hi) hash to a cell of the grid, all others are clamped to
+    // it: the smallest coordinates (of the precision mode) whose quotient is >= 0 and >= dims
+    double in_lo[3], in_hi[3];
+    float in_lo_f[3], in_hi_f[3];
     WallDev walls[DEM_MAX_WALLS];
 };
 
@@ -232,17 +240,16 @@ __device__ __forceinline__ float law_div_any(float a, float v2) {
 }
 // The factor mu |F_n| / |F_t| of Eq. 5 from the squared lengths (ft2 > 0). FP32: lengths
 // below 1e-19 N are taken as 1e-19 N, so that the factor stays finite.
-__device__ __forceinline__ double cap_factor(double mu, double fn2, double ft2) { return mu * sqrt(fn2) / sqrt(ft2); }
+// (FP64: one root and one quotient; a call of either is about ten operations of a pipe that
+// does 0.58 T of them per second.)
+__device__ __forceinline__ double cap_factor(double mu, double fn2, double ft2) {
+    return mu > 0.0 ? mu * sqrt(fn2 / ft2) : 0.0;
+}
 __device__ __forceinline__ float cap_factor(float mu, float fn2, float ft2) {
     float r;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fmaxf(ft2, 1.17549435e-38f)));
     return mu * law_sqrt(fn2) * r;
 }
-// Eq. 5's comparison |F_t| > mu |F_n| given that it holds for the squared lengths: FP64 mode
-// decides on the lengths, FP32 mode on the squares.
-__device__ __forceinline__ bool cap_holds(double mu, double fn2, double ft2) { return sqrt(ft2) > mu * sqrt(fn2); }
-__device__ __forceinline__ bool cap_holds(float, float, float) { return true; }
-
 // Symmetric in (a1, b1) <-> (a2, b2): products rounded first, then one rounded sum, so the
 // two threads that evaluate the same pair get the same bits.
 __device__ __forceinline__ float sym_madd(float a1, float b1, float a2, float b2) {
@@ -300,16 +307,17 @@ __device__ __forceinline__ void two_prod(float a, float b, float& p, float& e) {
 template <class T>
 struct Law {
     T dt, kn, kt, cn, ct, alpha, mu, ksp, kda, ksh, mu_roll, alpha_t, kcoh_pi;
+    T nrkt;         // -1 / kt
     int stiffness;  // 0 linear, 1 Hertz
     int terms;      // 1: no attractive normal force, 2: rolling resistance
 };
 __device__ __forceinline__ Law<double> law_of(const SceneDev& s, int stiffness, double) {
     return Law<double>{s.dt,  s.kn,  s.kt,  s.cn,      s.ct,      s.alpha,   s.mu,
-                       s.ksp, s.kda, s.ksh, s.mu_roll, s.alpha_t, s.kcoh_pi, stiffness, s.terms};
+                       s.ksp, s.kda, s.ksh, s.mu_roll, s.alpha_t, s.kcoh_pi, s.nrkt, stiffness, s.terms};
 }
 __device__ __forceinline__ Law<float> law_of(const SceneDev& s, int stiffness, float) {
     return Law<float>{s.dt_f,  s.kn_f,  s.kt_f,  s.cn_f,      s.ct_f,      s.alpha_f,   s.mu_f,
-                      s.ksp_f, s.kda_f, s.ksh_f, s.mu_roll_f, s.alpha_t_f, s.kcoh_pi_f, stiffness, s.terms};
+                      s.ksp_f, s.kda_f, s.ksh_f, s.mu_roll_f, s.alpha_t_f, s.kcoh_pi_f, s.nrkt_f, stiffness, s.terms};
 }
 
 // Practical contact law (Eqs. 2-10) for body i against partner j, seen from i:
@@ -349,9 +357,10 @@ __device__ __forceinline__ void law_practical(const Law<T>& P, V3<T> n, T delta,
     V3<T> Ftt = dt * (-kt) - vt * eta_t;
     // Eq. 5, compared on squared lengths; the lengths are taken only when the cap applies
     const T ft2 = dot(Ftt, Ftt), fn2 = dot(Fn, Fn);
-    if (ft2 > (P.mu * P.mu) * fn2 && ft2 > T(0) && cap_holds(P.mu, fn2, ft2)) {
+    if (ft2 > (P.mu * P.mu) * fn2 && ft2 > T(0)) {
         Ftt = Ftt * cap_factor(P.mu, fn2, ft2);
-        if (kt > T(0)) dt = (Ftt + vt * eta_t) * law_div(T(-1), kt);
+        // (linear stiffness: -1 / k_t is a constant of the scene)
+        if (kt > T(0)) dt = (Ftt + vt * eta_t) * (STIFF == 0 ? P.nrkt : law_div(T(-1), kt));
     }
     F = Fn + Ftt;                                                // Eq. 2
     if (TERMS && (P.terms & 8)) F = F + n * (P.kcoh_pi * Reff * delta);

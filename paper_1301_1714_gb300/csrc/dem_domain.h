@@ -8,12 +8,6 @@
 
 namespace demgb {
 
-// Largest tile of list mode and the force pass's resident blocks of that size per SM.
-#ifndef DEM_TILE_MAX
-#define DEM_TILE_MAX 512
-#define DEM_LIST_MIN_BLOCKS 2
-#endif
-
 // Tiles of list mode: halo entries a tile has room for in shared memory (a dense bed needs
 // 456 / 304 / 202 / 134 on average and at most 614 / 388 / 261 / 182 for tiles of 512 / 256 /
 // 128 / 64 particles). A tile with more reads its partners from global memory.
@@ -100,6 +94,7 @@ struct Domain {
     uint32_t diag_part_cap = 0;
     double* diag_out = nullptr;
 
+    int both_springs = 1; // 1: each pair's spring is stored with both particles (a slab's ghosts have none)
     int in_loop = 0;      // 1 while the step loop is being captured
     cudaGraphConditionalHandle loop_inner{}, loop_outer{};   // of the loop being captured
     int64_t launches = 0;
@@ -148,6 +143,8 @@ cudaError_t run_lists(Domain& d);
 cudaError_t run_tiles(Domain& d, bool always);   // tile entries and spring masks of the lists
 cudaError_t run_wall_masks(Domain& d);   // the wall masks again (after the walls changed)
 cudaError_t run_force_list(Domain& d, bool eval, double* dbgF, double* dbgT);
+// the force pass by contact items (dem_items.cu): FP64 mode and small scenes
+cudaError_t run_force_items(Domain& d, bool eval, double* dbgF, double* dbgT);
 cudaError_t run_export(Domain& d, double* x, double* v, double* w);
 cudaError_t run_diag(Domain& d);   // fills d.diag_out[0..9] (device)
 // batches: springs into sorted order (into the free history buffer), new packed layout,

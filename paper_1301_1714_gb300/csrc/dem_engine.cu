@@ -196,6 +196,34 @@ bool check_wall(const dem_wall& w, int precision, std::string& why) {
     return true;
 }
 
+// The smallest x of type T with fl(fl(x - o) / h) >= c (h > 0; the cell map's quotient with
+// its roundings, which grows with x), by bisection over the ordered values of T.
+template <class T>
+T first_at(T o, T h, T c) {
+    using U = std::conditional_t<sizeof(T) == 8, uint64_t, uint32_t>;
+    const U top = (U)1 << (8 * sizeof(T) - 1);
+    auto value = [&](U k) {   // k-th value in ascending order (0 = -infinity's NaN side)
+        const U b = (k & top) ? (k ^ top) : ~k;
+        T x;
+        std::memcpy(&x, &b, sizeof x);
+        return x;
+    };
+    auto rank = [&](T x) {
+        U b;
+        std::memcpy(&b, &x, sizeof b);
+        return (b & top) ? ~b : (b | top);
+    };
+    U lo = rank(-std::numeric_limits<T>::infinity()), hi = rank(std::numeric_limits<T>::infinity());
+    while (lo < hi) {
+        const U mid = lo + (hi - lo) / 2;
+        volatile T d = value(mid) - o;
+        volatile T q = d / h;
+        if (q >= c) hi = mid;
+        else lo = mid + 1;
+    }
+    return value(lo);
+}
+
 void fill_scene(dem_handle* h, SceneDev& S, uint32_t p0, uint32_t np, uint32_t c0, uint32_t t0 = 0) {
     const dem_config& c = h->cfg;
     S = SceneDev{};
@@ -227,6 +255,14 @@ void fill_scene(dem_handle* h, SceneDev& S, uint32_t p0, uint32_t np, uint32_t c
     S.terms = c.terms;
     S.mu_roll = c.mu_roll;
     S.mu_roll_f = (float)c.mu_roll;
+    S.nrkt = -1.0 / c.kt;
+    S.nrkt_f = -1.0f / (float)c.kt;
+    for (int a = 0; a < 3; ++a) {
+        S.in_lo[a] = first_at(S.origin[a], S.h, 0.0);
+        S.in_hi[a] = first_at(S.origin[a], S.h, (double)S.dims[a]);
+        S.in_lo_f[a] = first_at(S.origin_f[a], S.h_f, 0.0f);
+        S.in_hi_f[a] = first_at(S.origin_f[a], S.h_f, (float)S.dims[a]);
+    }
     S.alpha_t = c.alpha_t;
     S.alpha_t_f = (float)c.alpha_t;
     S.kcoh_pi = c.k_coh * 3.14159265358979323846;
@@ -319,6 +355,7 @@ dem_status alloc_domain(Domain& d, uint32_t n, uint32_t ncells, std::string& err
         AL(d.hs[s], N * 4 * T * (size_t)d.maxc);
     }
     AL(d.key, N * 4); AL(d.rank, N * 4); AL(d.tmp, N * 4); AL(d.perm, N * 4); AL(d.skey, N * 4);
+    if (d.list_mode || d.precision == 0) AL(d.ref, N * 16);
     if (d.list_mode) {
         AL(d.ncnt, N * 4);
         AL(d.nl, N * 4 * (size_t)DEM_LIST_CAP);
@@ -328,7 +365,6 @@ dem_status alloc_domain(Domain& d, uint32_t n, uint32_t ncells, std::string& err
         AL(d.halo, hw * 4);
         AL(d.nhalo, (size_t)d.ntiles * 4);
         AL(d.wmask, N * 4);
-        AL(d.ref, N * 16);
         AL(d.canon, N * 4);
         AL(d.fin, N * 4);
     }
@@ -477,11 +513,19 @@ int choose_bricks(const int64_t dims[3], int64_t nc, int64_t bdims[3], int64_t& 
     return 0;
 }
 
+// Threads per block of the walk's force pass when the configuration leaves it open: 256, and
+// less for few particles, down to one warp, so that the blocks reach every SM.
+int auto_block(const Domain& d, uint32_t n) {
+    int b = 256;
+    while (b > 32 && n / (uint32_t)b < 2u * (uint32_t)(d.sort_blocks / 8)) b /= 2;
+    return b;
+}
+
 // Particles per tile of list mode (a multiple of 32, at most 512; also the threads of a
 // force-pass block): four times the configured block size, and less for few particles, so
 // that the blocks fill the chip.
 uint32_t tile_size(const Domain& d, uint32_t n) {
-    uint32_t t = std::min((uint32_t)DEM_TILE_MAX, 4u * (uint32_t)d.block);
+    uint32_t t = std::min(d.precision == 0 ? (uint32_t)DEM_TILE_MAX_FP64 : (uint32_t)DEM_TILE_MAX, 4u * (uint32_t)d.block);
     while (t > 64 && n / t < 2u * (uint32_t)(d.sort_blocks / 8)) t = t > 256 ? 256 : t / 2;
     return std::max(32u, t & ~31u);
 }
@@ -556,6 +600,7 @@ dem_status load_particles(dem_handle* h, int64_t n64, const double* x, const dou
     if (s != DEM_OK) return s;
     d.n = n;
     d.ncells = (uint32_t)nc;
+    if (h->cfg.block_size == 0 && !d.list_mode) d.block = auto_block(d, n);
     d.tile = tile_size(d, n);
     d.ntiles = (n + d.tile - 1) / d.tile;
     s = ensure_buffers(h, n, (uint32_t)nc);
@@ -1359,6 +1404,7 @@ int64_t dem_device_bytes(const dem_handle* h) {
                (size_t)d.diag_part_cap * 80 + sizeof(StatusDev) + 128 + sizeof(SceneDev) * d.scenes_cap;
     b += (size_t)h->stage_cap * (9 * 8 + 4);
     if (d.list_mode) b += list_bytes(d);
+    else if (d.precision == 0) b += N * 16;
     return (int64_t)b;
 }
 
@@ -1450,6 +1496,7 @@ struct dem_batch {
     uint32_t* d_map = nullptr;
     size_t map_cap = 0;
     int resort_interval = -1;   // sort policy of every scene (set by the first scene added)
+    bool auto_block = false;    // the block size was left open
 };
 
 namespace {
@@ -1542,6 +1589,7 @@ dem_status repack(dem_batch* b) {
     nd.launches = od.launches;
     nd.n = (uint32_t)n_new;
     nd.ncells = (uint32_t)std::max<uint64_t>(c_new, 1);
+    if (b->auto_block && !nd.list_mode) nd.block = auto_block(nd, nd.n);
     nd.tile = tile_size(nd, nd.n);
     uint32_t tiles = 0;
     for (auto* group : {&kept, &fresh})
@@ -1673,6 +1721,7 @@ dem_status dem_batch_create(int precision, int model, int stiffness, int max_con
     d.maxc = max_contacts > 0 ? max_contacts : 32;
     d.maxn = DEM_LIST_CAP;
     d.block = block_size > 0 ? block_size : 256;
+    b->auto_block = block_size == 0;
     d.sort_blocks = sort_blocks_of(device);
     d.stream = (cudaStream_t)cuda_stream;
     if (cudaMalloc(&d.st, sizeof(StatusDev)) != cudaSuccess || cudaMallocHost(&d.st_host, sizeof(StatusDev)) != cudaSuccess ||
@@ -1869,6 +1918,7 @@ int64_t dem_batch_device_bytes(const dem_batch* b) {
     size_t bytes = 2 * state + 2 * (N * 4 + N * 4 * T * M) + 5 * N * 4 + 2 * C * 4 +
                    b->stage_cap * 76 + b->map_cap * 4;
     if (d.list_mode) bytes += list_bytes(d);
+    else if (d.precision == 0) bytes += N * 16;
     return (int64_t)bytes;
 }
 
@@ -2144,6 +2194,7 @@ dem_status dem_slabs_create(const dem_config* cfg, int nslabs, int axis, int dev
             dem_slabs_destroy(S);
             return st;
         }
+        h->d.both_springs = 0;
         h->d.regrow = 0;   // a slab's overflow is reported (its step is part of the exchange)
         S->sl.push_back(h);
     }

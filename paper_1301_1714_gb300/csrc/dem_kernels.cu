@@ -19,14 +19,6 @@
 #include "dem_domain.h"
 #include "dem_policy.cuh"
 
-// Minimum resident 256-thread blocks per SM requested for the force kernel, which caps
-// its registers at 65536 / (256 * value): 64 registers in both modes (measured on
-// GB300: the list-mode pass is 11% faster at 64 than at 80; the walk-mode pass, once it
-// stopped prefetching its candidates' payload, 10% faster; 48 spills and is 19% slower).
-#ifndef DEM_FORCE_MIN_BLOCKS
-#define DEM_FORCE_MIN_BLOCKS 4
-#endif
-
 namespace demgb {
 
 // ======================================================================= force pass
@@ -61,13 +53,14 @@ struct ForceArgs {
 // iterates max-list-length times instead of once per candidate), taking the contact
 // decision, the law (Eq. 1 or Eqs. 2-10) and the springs; then walls, gravity, the
 // update (step 1) and the new cell key with its rank in the cell (step 2).
-// MODEL: 0 the practical law, 1 the simple law (Eq. 1), 2 the practical law with the
-// scene's optional terms (no attraction, rolling resistance).
+// MODEL: 0 the practical law with linear stiffness, 1 the simple law (Eq. 1), 2 the practical
+// law with the scene's optional terms, 3 the practical law with Hertz stiffness.
 template <class PR, int MODEL, bool EVAL>
-__global__ void __launch_bounds__(256, DEM_FORCE_MIN_BLOCKS) k_force(ForceArgs<PR> a) {
+__global__ void __launch_bounds__(256, PR::WALK_BLOCKS) k_force(ForceArgs<PR> a) {
     using T = typename PR::T;
     constexpr bool PRACT = MODEL != 1;
     constexpr bool TERMS = MODEL == 2;
+    constexpr int STIFF = MODEL == 2 ? 2 : (MODEL == 3 ? 1 : 0);
     extern __shared__ uint32_t smem[];
     // a void step (an earlier launch overflowed): nothing to do; one decision per warp
     if (!EVAL && __any_sync(0xffffffffu, (a.ctrl->rebuild & DEM_HALT) != 0)) return;
@@ -169,10 +162,10 @@ __global__ void __launch_bounds__(256, DEM_FORCE_MIN_BLOCKS) k_force(ForceArgs<P
                                 sym_madd(ri, me.w.z, rjT, wj.z));
             const T mj = PR::mass(S, rj);
             const T meff = law_div(mi * mj, mi + mj);
-            const T Reff = law_div(ri * rjT, ri + rjT);
+            const T Reff = STIFF == 0 ? T(0) : law_div(ri * rjT, ri + rjT);
             const V3<T> dold = find_spring(s_oid, bd, tid, cnt_old, gid, a.hin, cap, src);
             V3<T> Fc, Ftc, dnew, Mr;
-            law_practical<TERMS, 2>(L, n, delta, v, rw, Reff, meff, dold, Fc, Ftc, dnew, me.w - wj, Mr);
+            law_practical<TERMS, STIFF>(L, n, delta, v, rw, Reff, meff, dold, Fc, Ftc, dnew, me.w - wj, Mr);
             F = F + Fc;
             Tq = Tq + cross(n, Ftc) * ri;
             if (TERMS) Tq = Tq + Mr;
@@ -198,7 +191,7 @@ __global__ void __launch_bounds__(256, DEM_FORCE_MIN_BLOCKS) k_force(ForceArgs<P
                 const V3<T> rw = me.w * ri;
                 const V3<T> dold = find_spring(s_oid, bd, tid, cnt_old, gid, a.hin, cap, src);
                 V3<T> Fc, Ftc, dnew, Mr;
-                law_practical<TERMS, 2>(L, n, delta, v, rw, ri, mi, dold, Fc, Ftc, dnew, me.w - PR::wall_omega(W), Mr);
+                law_practical<TERMS, STIFF>(L, n, delta, v, rw, ri, mi, dold, Fc, Ftc, dnew, me.w - PR::wall_omega(W), Mr);
                 F = F + Fc;
                 Tq = Tq + cross(n, Ftc) * ri;
                 if (TERMS) Tq = Tq + Mr;
@@ -231,7 +224,7 @@ __global__ void __launch_bounds__(256, DEM_FORCE_MIN_BLOCKS) k_force(ForceArgs<P
         } else {
             bool clamped = false, finite = true;
             float4 pnew;
-            const uint32_t kk = PR::integrate(B, q, me, F, Tq, S, mi, clamped, finite, pnew);
+            const uint32_t kk = PR::template integrate<true>(B, q, me, F, Tq, S, mi, clamped, finite, pnew);
             if (!finite) raise_status(a.st, ST_NONFINITE, (int32_t)q);
             c_clamp = clamped ? 1u : 0u;
             c_disp2 = pnew.w;
@@ -386,7 +379,7 @@ __global__ void k_scatter(uint32_t n, const uint32_t* __restrict__ key, const ui
 
 // (cell, id) order: a particle's place in its cell is the number of cell-mates with a
 // smaller id. Gathers the state from the next set (pre-sort order) into the current one,
-// records the permutation, the cell of each sorted particle and (list mode) its position.
+// records the permutation, the cell of each sorted particle and (FP64) its FP32 position and radius.
 template <class PR>
 __device__ __forceinline__ void reorder_one(uint32_t s, const typename PR::State& A, const typename PR::State& B,
                                             const uint32_t* __restrict__ key, const uint32_t* __restrict__ cs,
@@ -403,7 +396,7 @@ __device__ __forceinline__ void reorder_one(uint32_t s, const typename PR::State
     PR::store(A, q, m);
     perm[q] = p;
     skey[q] = c;
-    if (ref) ref[q] = PR::pos_f(m);
+    if (ref) ref[q] = PR::pre(m);
 }
 
 template <class PR>
@@ -876,7 +869,7 @@ cudaError_t run_rebuild(Domain& d) {
     if (!d.list_mode) {
         if (d.precision == 0)
             k_reorder<PF64><<<sgrid(d, d.n), 256, 0, d.stream>>>(d.n, d.S64[0], d.S64[1], d.ctrl, d.key, d.cs,
-                                                                   d.tmp, d.perm, d.skey, nullptr);
+                                                                   d.tmp, d.perm, d.skey, d.ref);
         else
             k_reorder<PF32><<<sgrid(d, d.n), 256, 0, d.stream>>>(d.n, d.S32[0], d.S32[1], d.ctrl, d.key, d.cs,
                                                                    d.tmp, d.perm, d.skey, nullptr);
@@ -977,19 +970,26 @@ static cudaError_t force_impl(Domain& d, const typename PR::State& S0, const typ
         return cudaSuccess;
     };
     cudaError_t e;
-    const int model = d.model != 0 ? 1 : (d.terms != 0 ? 2 : 0);
+    const int model = d.model != 0 ? 1 : (d.terms != 0 ? 2 : (d.stiffness != 0 ? 3 : 0));
     if (model == 0) e = eval ? launch(k_force<PR, 0, true>) : launch(k_force<PR, 0, false>);
     else if (model == 2) e = eval ? launch(k_force<PR, 2, true>) : launch(k_force<PR, 2, false>);
+    else if (model == 3) e = eval ? launch(k_force<PR, 3, true>) : launch(k_force<PR, 3, false>);
     else e = eval ? launch(k_force<PR, 1, true>) : launch(k_force<PR, 1, false>);
     if (e != cudaSuccess) return e;
     DEM_LAUNCH_CHECK();
     return cudaSuccess;
 }
 
+// Below this many particles the FP32 walk takes its contacts by items (dem_items.cu): a thread
+// per particle then leaves most of the chip idle. Measured per step on dense boxes (items /
+// thread per particle): 2,049 spheres 34 / 47 us, 9,001 37 / 50, 30,001 57 / 52, 100,001 125 /
+// 59. (With neighbour lists the thread per particle wins at any size: 21.2 / 22.3 us at 9,217.)
+constexpr uint32_t WALK_ITEMS_BELOW = 20000;
+
 cudaError_t run_force(Domain& d, bool eval, double* dbgF, double* dbgT) {
     if (d.n == 0) return cudaSuccess;
+    if (d.precision == 0 || (!d.list_mode && d.n < WALK_ITEMS_BELOW)) return run_force_items(d, eval, dbgF, dbgT);
     if (d.list_mode) return run_force_list(d, eval, dbgF, dbgT);
-    if (d.precision == 0) return force_impl<PF64>(d, d.S64[0], d.S64[1], eval, dbgF, dbgT);
     return force_impl<PF32>(d, d.S32[0], d.S32[1], eval, dbgF, dbgT);
 }
 

@@ -1,5 +1,6 @@
 // List mode (re-sort only after some particle moved skin/2): the force pass over the
-// neighbour lists built at each sort (the lists and tiles themselves: dem_nlist.cu).
+// neighbour lists built at each sort (the lists and tiles themselves: dem_nlist.cu), FP32
+// mode (FP64: dem_items.cu).
 //
 //   k_list   steps 5-8 and 1 for one thread block per tile of consecutive stored particles,
 //            one thread per particle. The tile's particles and its halo (the particles
@@ -60,7 +61,7 @@ struct ListArgs {
 // two stiffnesses have a variant each: the other's constants would take registers).
 // EVAL: forces and torques by id instead of the update.
 template <class PR, int MODEL, bool EVAL>
-__global__ void __launch_bounds__(DEM_TILE_MAX, DEM_LIST_MIN_BLOCKS) k_list(ListArgs<PR> a) {
+__global__ void __launch_bounds__(PR::LIST_THREADS, PR::LIST_BLOCKS) k_list(ListArgs<PR> a) {
     using T = typename PR::T;
     constexpr bool PRACT = MODEL != 1;
     constexpr bool TERMS = MODEL == 2;
@@ -297,7 +298,7 @@ __global__ void __launch_bounds__(DEM_TILE_MAX, DEM_LIST_MIN_BLOCKS) k_list(List
         } else {
             bool clamped = false, finite = true;
             float4 pnew;
-            PR::integrate(B, q, me2, F, Tq, S, mi, clamped, finite, pnew);
+            PR::template integrate<false>(B, q, me2, F, Tq, S, mi, clamped, finite, pnew);
             if (!finite) raise_status(a.st, ST_NONFINITE, (int32_t)q);
             c_clamp = clamped ? 1u : 0u;
             c_disp2 = pnew.w;
@@ -400,7 +401,6 @@ static cudaError_t force_list_impl(Domain& d, const typename PR::State& S0, cons
 
 cudaError_t run_force_list(Domain& d, bool eval, double* dbgF, double* dbgT) {
     if (d.n == 0) return cudaSuccess;
-    if (d.precision == 0) return force_list_impl<PF64>(d, d.S64[0], d.S64[1], eval, dbgF, dbgT);
     return force_list_impl<PF32>(d, d.S32[0], d.S32[1], eval, dbgF, dbgT);
 }
 

@@ -45,6 +45,13 @@ __device__ __forceinline__ bool near_f(float4 a, float4 b, float eps) {
     return ax * ax + ay * ay + az * az < Re * Re;
 }
 
+// The opposite, false also for coordinates beyond FP32's range (NaN differences).
+__device__ __forceinline__ bool far_f(float4 a, float4 b, float eps) {
+    const float ax = b.x - a.x, ay = b.y - a.y, az = b.z - a.z;
+    const float Re = (b.w + a.w) + eps;
+    return ax * ax + ay * ay + az * az >= Re * Re;
+}
+
 // ======================================================================= FP64 policy
 struct PF64 {
     using T = double;
@@ -75,48 +82,7 @@ struct PF64 {
         v = mk(__ldg(&s.vx[j]), __ldg(&s.vy[j]), __ldg(&s.vz[j]));
         w = mk(__ldg(&s.wx[j]), __ldg(&s.wy[j]), __ldg(&s.wz[j]));
     }
-    // Contact iff d^2 < R^2 with d^2 = fma(dz,dz, fma(dy,dy, dx*dx)), R = r_i + r_j (exact).
-    static __device__ __forceinline__ bool touches(const Self& me, double xj, double yj, double zj, float rjf) {
-        const double dx = __dsub_rn(xj, me.x), dy = __dsub_rn(yj, me.y), dz = __dsub_rn(zj, me.z);
-        const double d2 = __fma_rn(dz, dz, __fma_rn(dy, dy, __dmul_rn(dx, dx)));
-        const double R = __dadd_rn((double)me.r, (double)rjf);
-        return d2 < __dmul_rn(R, R);
-    }
-    // Phase 1 of the walk: append to the near list every particle of [j0, j1) in contact.
-    static __device__ __forceinline__ void scan_row(const State& s, const Self& me, const SceneDev&, uint32_t j0,
-                                                    uint32_t j1, uint32_t q, uint32_t* lst, uint32_t bd, uint32_t tid,
-                                                    uint32_t maxc, uint32_t& cnt) {
-        for (uint32_t j = j0; j < j1; ++j) {
-            if (j == q) continue;
-            if (touches(me, __ldg(&s.x[j]), __ldg(&s.y[j]), __ldg(&s.z[j]), __ldg(&s.r[j]))) {
-                if (cnt < maxc) lst[cnt * bd + tid] = j;
-                ++cnt;
-            }
-        }
-    }
-    // Tile of the list-mode force pass: (x, y, z, r) of every entry rounded to FP32, and the
-    // stored index. The prefilter runs on the FP32 copies (the FP64 pipe is about 60 times
-    // slower on GB300); the decision and the law read the FP64 state.
-    static constexpr uint32_t TILE_BYTES = 20;
-    static __device__ __forceinline__ void tile_fetch(const State& s, uint32_t j, unsigned char* t, uint32_t E,
-                                                      uint32_t i) {
-        ((float4*)t)[i] = make_float4((float)__ldg(&s.x[j]), (float)__ldg(&s.y[j]), (float)__ldg(&s.z[j]),
-                                      __ldg(&s.r[j]));
-        ((uint32_t*)(t + 16 * E))[i] = j;
-    }
-    static __device__ __forceinline__ Self tile_self(const State& s, uint32_t q, const unsigned char*, uint32_t,
-                                                     uint32_t) {
-        return load(s, q);
-    }
-    static __device__ __forceinline__ Self tile_again(const Self& m, const unsigned char*, uint32_t, uint32_t) { return m; }
-    static __device__ __forceinline__ V3<double> self_v(const Self& m, const unsigned char*, uint32_t, uint32_t) {
-        return m.v;
-    }
-    static __device__ __forceinline__ V3<double> self_w(const Self& m, const unsigned char*, uint32_t, uint32_t) {
-        return m.w;
-    }
-    static __device__ __forceinline__ Law<double> law(const Law<double>& L, const unsigned char*) { return L; }
-    static __device__ __forceinline__ void put_law(const Law<double>&, unsigned char*) {}
+    static __device__ __forceinline__ float radius(const State& s, uint32_t q) { return __ldg(&s.r[q]); }
     // FP32 position and radius of a particle for the prefilter
     static __device__ __forceinline__ float4 pre(const Self& m) {
         return make_float4((float)m.x, (float)m.y, (float)m.z, m.r);
@@ -129,14 +95,6 @@ struct PF64 {
     }
     static __device__ __forceinline__ float4 pre(const State& s, uint32_t j) {
         return make_float4((float)__ldg(&s.x[j]), (float)__ldg(&s.y[j]), (float)__ldg(&s.z[j]), __ldg(&s.r[j]));
-    }
-    // Neighbour-list test: j may come within contact of i while both move less than
-    // skin/2 (FP32 on the rounded positions, conservative by eps).
-    static __device__ __forceinline__ bool within(const State& s, const Self& me, uint32_t j, float reach_extra) {
-        const float ax = (float)__ldg(&s.x[j]) - (float)me.x, ay = (float)__ldg(&s.y[j]) - (float)me.y,
-                    az = (float)__ldg(&s.z[j]) - (float)me.z;
-        const float Re = (__ldg(&s.r[j]) + me.r) + reach_extra;
-        return ax * ax + ay * ay + az * az < Re * Re;
     }
     static __device__ __forceinline__ float4 pos_f(const Self& m) {
         return make_float4((float)m.x, (float)m.y, (float)m.z, 0.f);
@@ -153,10 +111,6 @@ struct PF64 {
         load_vw(s, j, o.v, o.w);
         return o;
     }
-    static __device__ __forceinline__ Partner tile_partner(const State& s, const unsigned char* t, uint32_t E,
-                                                           uint32_t i) {
-        return load_partner(s, ((const uint32_t*)(t + 16 * E))[i]);
-    }
     static __device__ __forceinline__ void partner_vw(const Partner& o, V3<double>& v, V3<double>& w) {
         v = o.v;
         w = o.w;
@@ -165,11 +119,7 @@ struct PF64 {
                                                    V3<double>& n, double& delta, float& rj) {
         return exact_j(s, me, o.j, n, delta, rj);
     }
-    // Phase 2: geometry of a listed contact (the decision is the same as in scan_row).
-    static __device__ __forceinline__ bool exact(const State& s, const Self& me, uint32_t j, const SceneDev&,
-                                                 V3<double>& n, double& delta, float& rj) {
-        return exact_j(s, me, j, n, delta, rj);
-    }
+    // Contact iff d^2 < R^2 with d^2 = fma(dz,dz, fma(dy,dy, dx*dx)), R = r_i + r_j (exact).
     static __device__ __forceinline__ bool exact_j(const State& s, const Self& me, uint32_t j, V3<double>& n,
                                                    double& delta, float& rj) {
         const double dx = __dsub_rn(__ldg(&s.x[j]), me.x);
@@ -179,8 +129,14 @@ struct PF64 {
         const double d2 = __fma_rn(dz, dz, __fma_rn(dy, dy, __dmul_rn(dx, dx)));
         const double R = __dadd_rn((double)me.r, (double)rjf);
         if (!(d2 < __dmul_rn(R, R))) return false;
-        const double d = sqrt(d2);
-        n = mk(dx / d, dy / d, dz / d);
+        // three quotients by the same d: its reciprocal once, then each quotient corrected by
+        // its residual (Markstein 1990, IBM J. Res. Dev. 34: the rounded quotient)
+        const double d = sqrt(d2), inv = __drcp_rn(d);
+        auto over = [&](double a) {
+            const double q = a * inv;
+            return __fma_rn(__fma_rn(-q, d, a), inv, q);
+        };
+        n = mk(over(dx), over(dy), over(dz));
         delta = R - d;
         rj = rjf;
         return true;
@@ -252,7 +208,15 @@ struct PF64 {
     static __device__ __forceinline__ uint32_t key_of(const State& s, const SceneDev& S, uint32_t q, bool& clamped) {
         return cell_key(S, s.x[q], s.y[q], s.z[q], clamped);
     }
+    // Whether the cell map clamps a position to the grid (what cell_key reports, without the
+    // three divisions: the thresholds are exact).
+    static __device__ __forceinline__ bool outside(const SceneDev& S, double x, double y, double z) {
+        return !(x >= S.in_lo[0] && y >= S.in_lo[1] && z >= S.in_lo[2] && x < S.in_hi[0] && y < S.in_hi[1] &&
+                 z < S.in_hi[2]);
+    }
     // Semi-implicit Euler (Sec. 4.2 step 1): v' = v + F dt/m, w' = w + T dt/I, x' = x + v' dt.
+    // KEY: returns the new cell key (else only whether it is clamped).
+    template <bool KEY>
     static __device__ __forceinline__ uint32_t integrate(const State& B, uint32_t q, const Self& me, V3<double> F,
                                                          V3<double> Tq, const SceneDev& S, double m, bool& clamped,
                                                          bool& finite, float4& pnew) {
@@ -268,7 +232,9 @@ struct PF64 {
         B.id[q] = me.id;
         finite = isfinite(xn) && isfinite(yn) && isfinite(zn) && isfinite(vn.x) && isfinite(vn.y) && isfinite(vn.z);
         pnew = make_float4((float)xn, (float)yn, (float)zn, (float)(dot(vn, vn) * (S.dt * S.dt)));
-        return cell_key(S, xn, yn, zn, clamped);
+        if (KEY) return cell_key(S, xn, yn, zn, clamped);
+        clamped = outside(S, xn, yn, zn);
+        return 0;
     }
     static __device__ __forceinline__ V3<double> pos(const Self& m) { return mk(m.x, m.y, m.z); }
     static __device__ __forceinline__ V3<double> vel(const Self& m) { return m.v; }
@@ -285,6 +251,10 @@ __device__ __forceinline__ void ff_diff(float hi, float lo, float phi, float plo
 }
 
 struct PF32 {
+    // Threads and resident blocks the list pass is compiled for (the largest tile), and the
+    // walk: 64 registers in both (measured: 80 or 128 registers lose more warps than they save
+    // spills, 0.61 / 0.69 / 0.85 ms per list pass at 4,194,304 spheres).
+    static constexpr int LIST_THREADS = DEM_TILE_MAX, LIST_BLOCKS = 2, WALK_BLOCKS = 4;
     using T = float;
     using State = StateF32;
     struct Self {
@@ -325,9 +295,9 @@ struct PF32 {
     }
     // Phase 1 of the walk: append to the near list every particle of [j0, j1) that passes
     // the prefilter (two candidates in flight per iteration).
-    static __device__ __forceinline__ void scan_row(const State& s, const Self& me, const SceneDev& S, uint32_t j0,
-                                                    uint32_t j1, uint32_t q, uint32_t* lst, uint32_t bd, uint32_t tid,
-                                                    uint32_t maxc, uint32_t& cnt) {
+    static __device__ __forceinline__ void scan_row(const State& s, const Self& me, const SceneDev& S,
+                                                    uint32_t j0, uint32_t j1, uint32_t q, uint32_t* lst, uint32_t bd,
+                                                    uint32_t tid, uint32_t maxc, uint32_t& cnt) {
         const float eps = S.eps_f;
         uint32_t j = j0;
         for (; j + 2 <= j1; j += 2) {
@@ -394,7 +364,7 @@ struct PF32 {
         p[0] = make_float4(L.dt, L.alpha, L.mu, L.kn);
         p[1] = make_float4(L.kt, L.cn, L.ct, L.ksp);
         p[2] = make_float4(L.kda, L.ksh, L.mu_roll, L.alpha_t);
-        p[3] = make_float4(L.kcoh_pi, __int_as_float(L.stiffness), __int_as_float(L.terms), 0.f);
+        p[3] = make_float4(L.kcoh_pi, __int_as_float(L.stiffness), __int_as_float(L.terms), L.nrkt);
     }
     static __device__ __forceinline__ Law<float> law(const Law<float>&, const unsigned char* s) {
         const float4 a = lds16(s), b = lds16(s + 16), c = lds16(s + 32), d = lds16(s + 48);
@@ -403,19 +373,13 @@ struct PF32 {
         L.kt = b.x; L.cn = b.y; L.ct = b.z; L.ksp = b.w;
         L.kda = c.x; L.ksh = c.y; L.mu_roll = c.z; L.alpha_t = c.w;
         L.kcoh_pi = d.x; L.stiffness = __float_as_int(d.y); L.terms = __float_as_int(d.z);
+        L.nrkt = d.w;
         return L;
     }
+    static __device__ __forceinline__ float radius(const State& s, uint32_t q) { return __ldg(&s.P0[q].w); }
     static __device__ __forceinline__ float4 pre(const Self& m) { return make_float4(m.hx, m.hy, m.hz, m.r); }
     static __device__ __forceinline__ float pre_eps(const SceneDev& S, float4) { return S.eps_f; }
     static __device__ __forceinline__ float4 pre(const State& s, uint32_t j) { return __ldg(&s.P0[j]); }
-    // Neighbour-list test: j may come within contact of i while both move less than
-    // skin/2 (FP32 on hi, conservative by eps).
-    static __device__ __forceinline__ bool within(const State& s, const Self& me, uint32_t j, float reach_extra) {
-        const float4 pj = __ldg(&s.P0[j]);
-        const float ax = pj.x - me.hx, ay = pj.y - me.hy, az = pj.z - me.hz;
-        const float Re = (pj.w + me.r) + reach_extra;
-        return ax * ax + ay * ay + az * az < Re * Re;
-    }
     static __device__ __forceinline__ float4 pos_f(const Self& m) { return make_float4(m.hx, m.hy, m.hz, 0.f); }
     // Everything phase 2 reads of a candidate, loaded together so the latencies overlap.
     struct Partner {
@@ -450,12 +414,8 @@ struct PF32 {
                                                    float& delta, float& rj) {
         return exact_xy(o.p0, o.p1, me, n, delta, rj);
     }
-    // Phase 2: the sign of R^2 - d^2 evaluated with error-free transformations (about
-    // 2^-46 relative to R^2), then delta = (R^2 - d^2)/(R + d) and the unit normal.
-    static __device__ __forceinline__ bool exact(const State& s, const Self& me, uint32_t j, const SceneDev&,
-                                                 V3<float>& n, float& delta, float& rj) {
-        return exact_xy(__ldg(&s.P0[j]), __ldg(&s.P1[j]), me, n, delta, rj);
-    }
+    // The sign of R^2 - d^2 evaluated with error-free transformations (about 2^-46 relative to
+    // R^2), then delta = (R^2 - d^2)/(R + d) and the unit normal.
     static __device__ __forceinline__ bool exact_xy(const float4 pj, const float4 lj, const Self& me, V3<float>& n,
                                                     float& delta, float& rj) {
         float sx, tx, sy, ty, sz, tz;
@@ -682,6 +642,11 @@ struct PF32 {
         const float l2 = __fadd_rn(lo, e);
         two_sum(s, l2, hi, lo);
     }
+    static __device__ __forceinline__ bool outside(const SceneDev& S, float x, float y, float z) {
+        return !(x >= S.in_lo_f[0] && y >= S.in_lo_f[1] && z >= S.in_lo_f[2] && x < S.in_hi_f[0] &&
+                 y < S.in_hi_f[1] && z < S.in_hi_f[2]);
+    }
+    template <bool KEY>
     static __device__ __forceinline__ uint32_t integrate(const State& B, uint32_t q, const Self& me, V3<float> F,
                                                          V3<float> Tq, const SceneDev& S, float m, bool& clamped,
                                                          bool& finite, float4& pnew) {
@@ -700,7 +665,9 @@ struct PF32 {
         B.id[q] = me.id;
         finite = isfinite(hx) && isfinite(hy) && isfinite(hz) && isfinite(vn.x) && isfinite(vn.y) && isfinite(vn.z);
         pnew = make_float4(hx, hy, hz, dot(vn, vn) * (S.dt_f * S.dt_f));
-        return cell_key(S, hx, hy, hz, clamped);
+        if (KEY) return cell_key(S, hx, hy, hz, clamped);
+        clamped = outside(S, hx, hy, hz);
+        return 0;
     }
     static __device__ __forceinline__ V3<double> pos(const Self& m) {
         return mk((double)m.hx + (double)m.lx, (double)m.hy + (double)m.ly, (double)m.hz + (double)m.lz);

@@ -34,7 +34,7 @@ TILE_BYTES = 4 * (768 + 1)
 def bytes_per_particle(precision: str = "fp32", max_contacts: int = 32, list_mode: bool = False) -> int:
     state, t = (68, 4) if precision == "fp32" else (80, 8)
     m = max_contacts or 32
-    b = 2 * state + 2 * (4 + 4 * t * m) + 20 + 76 + 4
+    b = 2 * state + 2 * (4 + 4 * t * m) + 20 + 76 + 4 + (16 if precision == "fp64" and not list_mode else 0)
     if list_mode:
         b += 4 + 6 * LIST_CAP + 4 + 16 + 8 + 16 + 17
     return b
