@@ -12,7 +12,7 @@ namespace demgb {
 // 456 / 304 / 202 / 134 on average and at most 614 / 388 / 261 / 182 for tiles of 512 / 256 /
 // 128 / 64 particles). A tile with more reads its partners from global memory.
 __host__ __device__ inline uint32_t halo_cap(uint32_t tile) {
-    return tile >= 512 ? 768u : tile >= 384 ? 640u : tile >= 256 ? 512u : tile >= 128 ? 384u : 256u;
+    return tile >= 448 ? 768u : tile >= 320 ? 640u : tile >= 192 ? 512u : tile >= 128 ? 384u : 256u;
 }
 constexpr uint32_t HALO_NONE = 0xFFFFFFFFu;
 
