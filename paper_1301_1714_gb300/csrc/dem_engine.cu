@@ -244,6 +244,7 @@ void fill_scene(dem_handle* h, SceneDev& S, uint32_t p0, uint32_t np, uint32_t c
     }
     S.h = h->h;
     S.h_f = (float)h->h;
+    S.inv_h_f = (float)(1.0 / h->h);
     S.active = 1;
     S.nwalls = (int32_t)h->walls.size();
     S.dt = c.dt; S.kn = c.kn; S.kt = c.kt; S.cn = c.cn; S.ct = c.ct; S.alpha = c.alpha; S.mu = c.mu;

@@ -20,6 +20,7 @@
 #include <cuda_runtime.h>
 
 #include "dem.h"
+#include "dem_dev.cuh"
 
 namespace {
 
@@ -47,11 +48,9 @@ void* g_addr[SA_MAX_DEVICES] = {nullptr};
 int g_resident[SA_MAX_DEVICES] = {0};   // blocks of k_sa_sort resident at once
 constexpr int SA_PER_SM = 2;
 
-__device__ __forceinline__ uint32_t sa_axis(double xa, double o, double h, int64_t dim) {
-    const double c = floor(__ddiv_rn(__dsub_rn(xa, o), h));
-    if (!(c >= 0.0)) return 0;
-    if (c >= (double)dim) return (uint32_t)(dim - 1);
-    return (uint32_t)c;
+__device__ __forceinline__ uint32_t sa_axis(double xa, double o, double h, float inv_h, int64_t dim) {
+    bool clamped = false;
+    return demgb::cell_of_axis(__dsub_rn(xa, o), h, inv_h, dim, clamped);
 }
 
 // The whole sort in one cooperative launch: as a memset and six kernels it took 67 us for
@@ -64,8 +63,8 @@ __device__ __forceinline__ uint32_t sa_axis(double xa, double o, double h, int64
 //   cell-mates with a smaller id (each thread reads its whole cell, so the work grows with
 //   the square of the cells' occupancy)
 __global__ void __launch_bounds__(SA_THREADS) k_sa_sort(uint32_t n, const double* __restrict__ x, double ox, double oy,
-                                                        double oz, double h, int64_t nx, int64_t ny, int64_t nz,
-                                                        uint32_t m, uint32_t ntiles, uint32_t* cell_of,
+                                                        double oz, double h, float inv_h, int64_t nx, int64_t ny,
+                                                        int64_t nz, uint32_t m, uint32_t ntiles, uint32_t* cell_of,
                                                         uint32_t* order, uint32_t* cell_start, uint32_t* scratch) {
     cooperative_groups::grid_group grid = cooperative_groups::this_grid();
     __shared__ uint32_t ws[SA_THREADS / 32], s_pre;
@@ -78,9 +77,9 @@ __global__ void __launch_bounds__(SA_THREADS) k_sa_sort(uint32_t n, const double
     for (uint32_t k = first; k < m; k += step) cnt[k] = 0u;
     grid.sync();
     for (uint32_t k = first; k < n; k += step) {
-        const uint32_t i = sa_axis(x[3 * (size_t)k], ox, h, nx);
-        const uint32_t j = sa_axis(x[3 * (size_t)k + 1], oy, h, ny);
-        const uint32_t l = sa_axis(x[3 * (size_t)k + 2], oz, h, nz);
+        const uint32_t i = sa_axis(x[3 * (size_t)k], ox, h, inv_h, nx);
+        const uint32_t j = sa_axis(x[3 * (size_t)k + 1], oy, h, inv_h, ny);
+        const uint32_t l = sa_axis(x[3 * (size_t)k + 2], oz, h, inv_h, nz);
         const uint32_t key = (l * (uint32_t)ny + j) * (uint32_t)nx + i;
         cell_of[k] = key;
         rank[k] = atomicAdd(&cnt[key], 1u);
@@ -195,8 +194,9 @@ extern "C" dem_status dem_sort_cells_static(int64_t n, const double* x, const do
     const uint32_t want = std::max(1u, std::max((std::max(nn, m / SA_ITEMS) + SA_THREADS - 1) / SA_THREADS, nb));
     uint32_t blocks = std::min(want, (uint32_t)resident);
     double ox = origin[0], oy = origin[1], oz = origin[2], h = cell;
+    float inv_h = (float)(1.0 / cell);
     int64_t nx = dims[0], ny = dims[1], nz = dims[2];
-    void* args[] = {&nn, &x, &ox, &oy, &oz, &h, &nx, &ny, &nz, &m, &nb, &cell_of, &order, &cell_start, &scratch};
+    void* args[] = {&nn, &x, &ox, &oy, &oz, &h, &inv_h, &nx, &ny, &nz, &m, &nb, &cell_of, &order, &cell_start, &scratch};
     if (cudaLaunchCooperativeKernel((const void*)k_sa_sort, dim3(blocks), dim3(SA_THREADS), args, 0, st) != cudaSuccess) {
         cudaGetLastError();
         return DEM_ERR_CUDA;

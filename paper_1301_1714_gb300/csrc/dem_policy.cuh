@@ -196,10 +196,7 @@ struct PF64 {
         return S.cmass * rd * rd * rd;
     }
     static __device__ __forceinline__ uint32_t axis_cell(const SceneDev& S, int a, double xa, bool& clamped) {
-        const double c = floor(__ddiv_rn(__dsub_rn(xa, S.origin[a]), S.h));
-        if (!(c >= 0.0)) { clamped = true; return 0; }
-        if (c >= (double)S.dims[a]) { clamped = true; return (uint32_t)(S.dims[a] - 1); }
-        return (uint32_t)c;
+        return cell_of_axis(__dsub_rn(xa, S.origin[a]), S.h, S.inv_h_f, S.dims[a], clamped);
     }
     static __device__ __forceinline__ uint32_t cell_key(const SceneDev& S, double x, double y, double z, bool& clamped) {
         const uint32_t i = axis_cell(S, 0, x, clamped), j = axis_cell(S, 1, y, clamped), k = axis_cell(S, 2, z, clamped);
