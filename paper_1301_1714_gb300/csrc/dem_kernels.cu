@@ -333,13 +333,19 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_down(uint32_t* __restrict
             before = part[tile];
         }
         const uint32_t base = tile * SCAN_TILE + threadIdx.x * SCAN_ITEMS;
+        // a thread's eight entries as two 16-byte loads (and stores below): as 4-byte accesses
+        // of stride 32 bytes they took 21 us for the 1.4 M cells of the 1,000,003-sphere drum
+        const bool whole = base + SCAN_ITEMS <= m;
         uint32_t v[SCAN_ITEMS];
         uint32_t s = 0;
-        for (int i = 0; i < SCAN_ITEMS; ++i) {
-            const uint32_t k = base + i;
-            v[i] = k < m ? cnt[k] : 0u;
-            s += v[i];
+        if (whole) {
+            const uint4 a = *(const uint4*)&cnt[base], b = *(const uint4*)&cnt[base + 4];
+            v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+            v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+        } else {
+            for (int i = 0; i < SCAN_ITEMS; ++i) v[i] = base + i < m ? cnt[base + i] : 0u;
         }
+        for (int i = 0; i < SCAN_ITEMS; ++i) s += v[i];
         // block-exclusive scan of the thread sums
         uint32_t inc = s;
         for (int off = 1; off < 32; off <<= 1) {
@@ -358,13 +364,24 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_down(uint32_t* __restrict
         }
         __syncthreads();
         uint32_t run = before + (inc - s) + (wid > 0 ? ws[wid - 1] : 0u);
-        for (int i = 0; i < SCAN_ITEMS; ++i) {
-            const uint32_t k = base + i;
-            if (k < m) {
-                cs[k] = run;
-                cnt[k] = 0u;
+        if (whole) {
+            uint32_t e[SCAN_ITEMS];
+            for (int i = 0; i < SCAN_ITEMS; ++i) {
+                e[i] = run;
+                run += v[i];
             }
-            run += v[i];
+            *(uint4*)&cs[base] = make_uint4(e[0], e[1], e[2], e[3]);
+            *(uint4*)&cs[base + 4] = make_uint4(e[4], e[5], e[6], e[7]);
+            *(uint4*)&cnt[base] = *(uint4*)&cnt[base + 4] = make_uint4(0u, 0u, 0u, 0u);
+        } else {
+            for (int i = 0; i < SCAN_ITEMS; ++i) {
+                const uint32_t k = base + i;
+                if (k < m) {
+                    cs[k] = run;
+                    cnt[k] = 0u;
+                }
+                run += v[i];
+            }
         }
         __syncthreads();
     }
