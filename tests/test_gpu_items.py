@@ -74,7 +74,8 @@ def test_fp32_walk_across_the_size_limit():
     got = []
     for x, v, w, r in ((sc.x, sc.v, sc.w, sc.r), (x2, v2, w2, r2)):
         p = sc.params.copy(walls=[])
-        with dem.Simulation(p, x, v, w, r) as s:
+        # (24 slots: the block's lists take exactly the default limit of shared memory)
+        with dem.Simulation(p, x, v, w, r, max_contacts=24) as s:
             s.step(20)
             got.append([a[:19000] for a in s.state()])
     for a, b in zip(*got):
