@@ -407,9 +407,10 @@ int64_t dem_device_bytes(const dem_handle* h);
  * dem_step grows up to 64 as needed). */
 int64_t dem_max_contacts_seen(const dem_handle* h);
 
-/* Number of kernel launches the handle has enqueued so far (kernels that a replayed step
- * graph ran conditionally are counted from a device-side counter: the call synchronises
- * the handle's stream). */
+/* Number of kernel launches the handle has enqueued so far. In the step loop of list mode
+ * the three kernels of every step taken and the kernels of every sort that ran are counted
+ * (the sorts from a device-side counter: the call synchronises the handle's stream), not
+ * the launches that idle at the end of a turn. */
 int64_t dem_launch_count(const dem_handle* h);
 
 /* Last error message of the handle ("" if none). Valid until the next call on h. */

@@ -1,17 +1,19 @@
 // Kernels of the GB300 DEM timestep and their launchers.
 //
-//   k_force      steps 5-8 + 1 + 2: 27-cell contact search (Eq. 12) or neighbour list,
-//                contact laws (Eq. 1 or Eqs. 2-10), walls, gravity, semi-implicit Euler,
-//                then the new cell key CM and its rank within the cell (sort every step)
-//                or the displacement test that decides a sort (neighbour lists)
+//   k_force      FP32 walk, steps 5-8 + 1 + 2: 27-cell contact search (Eq. 12), contact laws
+//                (Eq. 1 or Eqs. 2-10), walls, gravity, semi-implicit Euler, then the new cell
+//                key CM and its rank within the cell
 //   k_hash       step 2 for a sort step in list mode
 //   k_scan_*     exclusive scan of per-cell counts -> dense cell-start table
 //   k_scatter    particles into cell-major slots (order within a cell still arbitrary)
 //   k_reorder    step 4: (cell, id) order (Eq. 11) and gather of every property
-//   (list mode: the neighbour lists and the pair-once force pass are in dem_list.cu)
-//   k_end_step   per-step bookkeeping of the device-side step control
+//   k_rank_cell, k_window   the same in list mode, each tile ordered by contact counts
+//   k_sort_end, k_end_step, k_loop_decide, k_loop_end   bookkeeping of the device-side step
+//                control, outside and inside the step loop
 //   k_import / k_export / k_diag* / k_hist_canon / k_repack   set-up, read-out,
 //                diagnostics, batch repacking
+// (list mode's force pass: dem_list.cu, its lists and tiles: dem_nlist.cu; FP64 mode and
+// small FP32 walks: dem_items.cu)
 #include <algorithm>
 
 #include <cuda_runtime.h>

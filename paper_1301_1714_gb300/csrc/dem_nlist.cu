@@ -1,6 +1,7 @@
 // List mode: the neighbour lists of a sort (Eq. 12's 27 cells, candidates within
 // r_i + r_j + skin, in ascending partner id) and the walls each particle can reach before
-// the next sort. The force pass that reads them is in dem_list.cu.
+// the next sort, and the tiles. The force passes that read them: dem_list.cu (FP32),
+// dem_items.cu (FP64).
 #include <algorithm>
 
 #include <cuda_runtime.h>
