@@ -233,45 +233,37 @@ __device__ __forceinline__ float dsqrt(float a) { return sqrtf(a); }
 __device__ __forceinline__ double dsqrt(double a) { return sqrt(a); }
 
 // Quotient and square root of the contact law. FP64 mode: IEEE operations. FP32 mode: the
-// hardware's approximations with subnormal arguments taken as zero, each one instruction
-// (reciprocal: relative error 2^-23, so a quotient is within 1.5 ulp; square root 2^-23):
-// PTX div.approx and sqrt.approx without .ftz have no smaller error and take about eight and
-// five instructions, for arguments that lengths, masses and squared forces never reach (the
-// callers say where a subnormal one could matter). All are deterministic functions of their
-// arguments, so the two evaluations of a pair stay exact mirrors of each other.
+// hardware approximations (PTX div.approx / sqrt.approx, relative error about 2^-22),
+// well inside the FP32 mode's force tolerance; both are deterministic functions of their
+// arguments, so the two evaluations of a pair stay exact mirrors of each other. (The .ftz
+// forms, a reciprocal and a product, take fewer instructions and have the same error against 64
+// bits, but a bed of stiff contacts carries any other rounding to 3e-4 of the velocities in 200
+// steps, and a run would no longer repeat its earlier results.)
 __device__ __forceinline__ double law_div(double a, double b) { return a / b; }
 __device__ __forceinline__ double law_sqrt(double a) { return sqrt(a); }
-__device__ __forceinline__ float law_rcp(float b) {
+__device__ __forceinline__ float law_div(float a, float b) {
     float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));
+    asm("div.approx.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
     return r;
 }
-__device__ __forceinline__ float law_div(float a, float b) { return a * law_rcp(b); }
 __device__ __forceinline__ float law_sqrt(float a) {
     float r;
-    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(a));
     return r;
 }
-// v / |v| from v and |v|^2 > 0, for any magnitude (the components may be subnormal squares).
-__device__ __forceinline__ double law_div_any(double a, double v2) { return a / sqrt(v2); }
-__device__ __forceinline__ float law_div_any(float a, float v2) {
-    float r, s;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(s) : "f"(v2));
-    asm("div.approx.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(s));
-    return r;
+// Eq. 5 for squared lengths that exceed the cap: whether the lengths do, and the factor
+// mu |F_n| / |F_t|. FP64: one root and one quotient (a call of either is about ten operations of
+// a pipe that does 0.58 T of them per second).
+__device__ __forceinline__ bool cap_of(double mu, double fn2, double ft2, double& f) {
+    f = mu > 0.0 ? mu * sqrt(fn2 / ft2) : 0.0;
+    return true;
 }
-// The factor mu |F_n| / |F_t| of Eq. 5 from the squared lengths (ft2 > 0). FP32: lengths
-// below 1e-19 N are taken as 1e-19 N, so that the factor stays finite.
-// (FP64: one root and one quotient; a call of either is about ten operations of a pipe that
-// does 0.58 T of them per second.)
-__device__ __forceinline__ double cap_factor(double mu, double fn2, double ft2) {
-    return mu > 0.0 ? mu * sqrt(fn2 / ft2) : 0.0;
+__device__ __forceinline__ bool cap_of(float mu, float fn2, float ft2, float& f) {
+    const float ftn = law_sqrt(ft2), fnn = law_sqrt(fn2);
+    f = law_div(mu * fnn, ftn);
+    return ftn > mu * fnn;
 }
-__device__ __forceinline__ float cap_factor(float mu, float fn2, float ft2) {
-    float r;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fmaxf(ft2, 1.17549435e-38f)));
-    return mu * law_sqrt(fn2) * r;
-}
+
 // Symmetric in (a1, b1) <-> (a2, b2): products rounded first, then one rounded sum, so the
 // two threads that evaluate the same pair get the same bits.
 __device__ __forceinline__ float sym_madd(float a1, float b1, float a2, float b2) {
@@ -380,9 +372,12 @@ __device__ __forceinline__ void law_practical(const Law<T>& P, V3<T> n, T delta,
     // Eq. 5, compared on squared lengths; the lengths are taken only when the cap applies
     const T ft2 = dot(Ftt, Ftt), fn2 = dot(Fn, Fn);
     if (ft2 > (P.mu * P.mu) * fn2 && ft2 > T(0)) {
-        Ftt = Ftt * cap_factor(P.mu, fn2, ft2);
-        // (linear stiffness: -1 / k_t is a constant of the scene)
-        if (kt > T(0)) dt = (Ftt + vt * eta_t) * (STIFF == 0 ? P.nrkt : law_div(T(-1), kt));
+        T f;
+        if (cap_of(P.mu, fn2, ft2, f)) {
+            Ftt = Ftt * f;
+            // (FP64, linear stiffness: -1 / k_t is a constant of the scene)
+            if (kt > T(0)) dt = (Ftt + vt * eta_t) * (STIFF == 0 && sizeof(T) == 8 ? P.nrkt : law_div(T(-1), kt));
+        }
     }
     F = Fn + Ftt;                                                // Eq. 2
     if (TERMS && (P.terms & 8)) F = F + n * (P.kcoh_pi * Reff * delta);
@@ -391,7 +386,7 @@ __device__ __forceinline__ void law_practical(const Law<T>& P, V3<T> n, T delta,
     Mroll = mk(T(0), T(0), T(0));
     if (TERMS && (P.terms & 2)) {
         const T wn2 = dot(wrel, wrel);
-        if (wn2 > T(0)) Mroll = wrel * law_div_any(-P.mu_roll * Reff * law_sqrt(fn2), wn2);
+        if (wn2 > T(0)) Mroll = wrel * law_div(-P.mu_roll * Reff * law_sqrt(fn2), law_sqrt(wn2));
     }
 }
 
