@@ -224,10 +224,39 @@ struct V3 { T x, y, z; };
 template <class T> __device__ __forceinline__ V3<T> mk(T x, T y, T z) { return V3<T>{x, y, z}; }
 template <class T> __device__ __forceinline__ V3<T> operator+(V3<T> a, V3<T> b) { return {a.x + b.x, a.y + b.y, a.z + b.z}; }
 template <class T> __device__ __forceinline__ V3<T> operator-(V3<T> a, V3<T> b) { return {a.x - b.x, a.y - b.y, a.z - b.z}; }
+template <class T> __device__ __forceinline__ V3<T> operator-(V3<T> a) { return {-a.x, -a.y, -a.z}; }
 template <class T> __device__ __forceinline__ V3<T> operator*(V3<T> a, T s) { return {a.x * s, a.y * s, a.z * s}; }
-template <class T> __device__ __forceinline__ T dot(V3<T> a, V3<T> b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
+// Sums of products as they are rounded: every fused operation is written out, so that each
+// kernel has the same bits. (Left to the compiler, which products of a sum it fuses depends on
+// the code around them, and two kernels, or two versions of one, then differ in the last place;
+// a bed of stiff contacts carries that to 1e-3 of single velocities in a few hundred steps.)
+// a b + c d is fma(a, b, fl(c d)).
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+template <class T> __device__ __forceinline__ T mad2(T a, T b, T c, T d) { return fma_rn(a, b, mul_rn(c, d)); }
+template <class T> __device__ __forceinline__ V3<T> add(V3<T> a, V3<T> b) {
+    return {add_rn(a.x, b.x), add_rn(a.y, b.y), add_rn(a.z, b.z)};
+}
+template <class T> __device__ __forceinline__ V3<T> scale(V3<T> a, T s) {
+    return {mul_rn(a.x, s), mul_rn(a.y, s), mul_rn(a.z, s)};
+}
+// c + a s, fused
+template <class T> __device__ __forceinline__ V3<T> axpy(V3<T> a, T s, V3<T> c) {
+    return {fma_rn(a.x, s, c.x), fma_rn(a.y, s, c.y), fma_rn(a.z, s, c.z)};
+}
+// a s + b t
+template <class T> __device__ __forceinline__ V3<T> mad2(V3<T> a, T s, V3<T> b, T t) {
+    return {mad2(a.x, s, b.x, t), mad2(a.y, s, b.y, t), mad2(a.z, s, b.z, t)};
+}
+template <class T> __device__ __forceinline__ T dot(V3<T> a, V3<T> b) {
+    return fma_rn(a.z, b.z, mad2(a.x, b.x, a.y, b.y));
+}
 template <class T> __device__ __forceinline__ V3<T> cross(V3<T> a, V3<T> b) {
-    return {a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
+    return {fma_rn(a.y, b.z, -mul_rn(a.z, b.y)), fma_rn(a.z, b.x, -mul_rn(a.x, b.z)), fma_rn(a.x, b.y, -mul_rn(a.y, b.x))};
 }
 __device__ __forceinline__ float dsqrt(float a) { return sqrtf(a); }
 __device__ __forceinline__ double dsqrt(double a) { return sqrt(a); }
@@ -237,8 +266,7 @@ __device__ __forceinline__ double dsqrt(double a) { return sqrt(a); }
 // well inside the FP32 mode's force tolerance; both are deterministic functions of their
 // arguments, so the two evaluations of a pair stay exact mirrors of each other. (The .ftz
 // forms, a reciprocal and a product, take fewer instructions and have the same error against 64
-// bits, but a bed of stiff contacts carries any other rounding to 3e-4 of the velocities in 200
-// steps, and a run would no longer repeat its earlier results.)
+// bits, but other last bits.)
 __device__ __forceinline__ double law_div(double a, double b) { return a / b; }
 __device__ __forceinline__ double law_sqrt(double a) { return sqrt(a); }
 __device__ __forceinline__ float law_div(float a, float b) {
@@ -259,9 +287,9 @@ __device__ __forceinline__ bool cap_of(double mu, double fn2, double ft2, double
     return true;
 }
 __device__ __forceinline__ bool cap_of(float mu, float fn2, float ft2, float& f) {
-    const float ftn = law_sqrt(ft2), fnn = law_sqrt(fn2);
-    f = law_div(mu * fnn, ftn);
-    return ftn > mu * fnn;
+    const float ftn = law_sqrt(ft2), lim = __fmul_rn(mu, law_sqrt(fn2));
+    f = law_div(lim, ftn);
+    return ftn > lim;
 }
 
 // Symmetric in (a1, b1) <-> (a2, b2): products rounded first, then one rounded sum, so the
@@ -352,49 +380,51 @@ __device__ __forceinline__ void law_practical(const Law<T>& P, V3<T> n, T delta,
                                               V3<T> dold, V3<T>& F, V3<T>& Ft, V3<T>& dnew, V3<T> wrel,
                                               V3<T>& Mroll) {
     const T vn_s = dot(v, n);                                    // Eq. 6
-    const V3<T> vn = n * vn_s;
-    const V3<T> vt = (v - vn) + cross(rw, n);
-    const T dn = dot(dold, n);                                   // Eq. 7
-    V3<T> dt = (dold - n * dn) + vt * P.dt;
+    const V3<T> vn = scale(n, vn_s);
+    const V3<T> vt = add(add(v, -vn), cross(rw, n));
+    V3<T> dt = axpy(vt, P.dt, axpy(n, -dot(dold, n), dold));     // Eq. 7
     T kn, kt;                                                    // Eqs. 8-9
     if (STIFF == 0 || (STIFF == 2 && P.stiffness == 0)) { kn = P.kn; kt = P.kt; }
     else {
-        const T s = law_sqrt(delta * Reff);
-        kn = P.cn * s;
-        kt = P.ct * s;
+        const T s = law_sqrt(mul_rn(delta, Reff));
+        kn = mul_rn(P.cn, s);
+        kt = mul_rn(P.ct, s);
     }
-    const T eta = P.alpha * law_sqrt(kn * meff);                 // Eq. 10
-    V3<T> Fn = n * (-kn * delta) - vn * eta;                     // Eq. 4
+    const T eta = mul_rn(P.alpha, law_sqrt(mul_rn(kn, meff)));   // Eq. 10
+    V3<T> Fn = mad2(n, mul_rn(-kn, delta), vn, -eta);            // Eq. 4
     if (TERMS && (P.terms & 1) && dot(Fn, n) > T(0)) Fn = mk(T(0), T(0), T(0));
     T eta_t = eta;
-    if (TERMS && (P.terms & 4)) eta_t = P.alpha_t * law_sqrt(kt * meff);
-    V3<T> Ftt = dt * (-kt) - vt * eta_t;
+    if (TERMS && (P.terms & 4)) eta_t = mul_rn(P.alpha_t, law_sqrt(mul_rn(kt, meff)));
+    const V3<T> damp = scale(vt, eta_t);
+    V3<T> Ftt = axpy(dt, -kt, -damp);
     // Eq. 5, compared on squared lengths; the lengths are taken only when the cap applies
     const T ft2 = dot(Ftt, Ftt), fn2 = dot(Fn, Fn);
-    if (ft2 > (P.mu * P.mu) * fn2 && ft2 > T(0)) {
+    if (ft2 > mul_rn(mul_rn(P.mu, P.mu), fn2) && ft2 > T(0)) {
         T f;
         if (cap_of(P.mu, fn2, ft2, f)) {
-            Ftt = Ftt * f;
+            Ftt = scale(Ftt, f);
             // (FP64, linear stiffness: -1 / k_t is a constant of the scene)
-            if (kt > T(0)) dt = (Ftt + vt * eta_t) * (STIFF == 0 && sizeof(T) == 8 ? P.nrkt : law_div(T(-1), kt));
+            if (kt > T(0))
+                dt = scale(add(Ftt, damp), STIFF == 0 && sizeof(T) == 8 ? P.nrkt : law_div(T(-1), kt));
         }
     }
-    F = Fn + Ftt;                                                // Eq. 2
-    if (TERMS && (P.terms & 8)) F = F + n * (P.kcoh_pi * Reff * delta);
+    F = add(Fn, Ftt);                                            // Eq. 2
+    if (TERMS && (P.terms & 8)) F = axpy(n, mul_rn(mul_rn(P.kcoh_pi, Reff), delta), F);
     Ft = Ftt;
     dnew = dt;
     Mroll = mk(T(0), T(0), T(0));
     if (TERMS && (P.terms & 2)) {
         const T wn2 = dot(wrel, wrel);
-        if (wn2 > T(0)) Mroll = wrel * law_div(-P.mu_roll * Reff * law_sqrt(fn2), law_sqrt(wn2));
+        if (wn2 > T(0))
+            Mroll = scale(wrel, law_div(mul_rn(mul_rn(-P.mu_roll, Reff), law_sqrt(fn2)), law_sqrt(wn2)));
     }
 }
 
 // Simple law (Eq. 1): -k_sp delta n - k_da v - k_sh v_t, v_t = v - (v.n) n.
 template <class T>
 __device__ __forceinline__ V3<T> law_simple(const Law<T>& P, V3<T> n, T delta, V3<T> v) {
-    const V3<T> vt = v - n * dot(v, n);
-    return (n * (-P.ksp * delta) - v * P.kda) - vt * P.ksh;
+    const V3<T> vt = axpy(n, -dot(v, n), v);
+    return axpy(vt, -P.ksh, mad2(n, mul_rn(-P.ksp, delta), v, -P.kda));
 }
 
 }  // namespace demgb

@@ -474,14 +474,14 @@ __global__ void __launch_bounds__(ITEM_THREADS, 2) k_items(ItemArgs<PR> a) {
                 const float dl = delta_of[it];
                 if (!(dl >= 0.f)) continue;
                 const T* r = res + it;
-                F = F + mk(r[0], r[ITEM_MAX], r[2 * ITEM_MAX]) * sg;
+                F = axpy(mk(r[0], r[ITEM_MAX], r[2 * ITEM_MAX]), sg, F);
                 if (PRACT) {
-                    Tq = Tq + mk(r[3 * ITEM_MAX], r[4 * ITEM_MAX], r[5 * ITEM_MAX]) * ri;
-                    if (TERMS) Tq = Tq + mk(r[9 * ITEM_MAX], r[10 * ITEM_MAX], r[11 * ITEM_MAX]) * sg;
+                    Tq = axpy(mk(r[3 * ITEM_MAX], r[4 * ITEM_MAX], r[5 * ITEM_MAX]), ri, Tq);
+                    if (TERMS) Tq = axpy(mk(r[9 * ITEM_MAX], r[10 * ITEM_MAX], r[11 * ITEM_MAX]), sg, Tq);
                 }
                 if ((PRACT || EVAL) && nnew < maxc) {
                     const uint32_t j = LIST && !direct ? t_gid[pid_at] : pid_at;
-                    const V3<T> d = PRACT ? mk(r[6 * ITEM_MAX], r[7 * ITEM_MAX], r[8 * ITEM_MAX]) * sg
+                    const V3<T> d = PRACT ? scale(mk(r[6 * ITEM_MAX], r[7 * ITEM_MAX], r[8 * ITEM_MAX]), sg)
                                           : mk(T(0), T(0), T(0));
                     store_spring(&hout[nnew * cap + q], d, __ldg(&A.id[j]));
                     if (LIST) {
@@ -517,7 +517,7 @@ __global__ void __launch_bounds__(ITEM_THREADS, 2) k_items(ItemArgs<PR> a) {
             const V3<T> v = me.v - PR::wall_vel(W, cp);
             const uint32_t gid = DEM_WALL_BASE + (uint32_t)w;
             if (PRACT) {
-                const V3<T> rw = me.w * ri;
+                const V3<T> rw = scale(me.w, ri);
                 V3<T> dold = mk(T(0), T(0), T(0));
                 // (lists: wall springs follow the particles' ones)
                 for (uint32_t k = LIST ? (uint32_t)(__popc(s_om[2 * tid]) + __popc(s_om[2 * tid + 1])) : 0u; k < cold; ++k) {
@@ -526,12 +526,12 @@ __global__ void __launch_bounds__(ITEM_THREADS, 2) k_items(ItemArgs<PR> a) {
                 }
                 V3<T> Fc, Ftc, dnew, Mr;
                 law_practical<TERMS, STIFF>(L, n, delta, v, rw, ri, mi, dold, Fc, Ftc, dnew, me.w - PR::wall_omega(W), Mr);
-                F = F + Fc;
-                Tq = Tq + cross(n, Ftc) * ri;
-                if (TERMS) Tq = Tq + Mr;
+                F = add(F, Fc);
+                Tq = axpy(cross(n, Ftc), ri, Tq);
+                if (TERMS) Tq = add(Tq, Mr);
                 if (nnew < maxc) store_spring(&hout[nnew * cap + q], dnew, gid);
             } else {
-                F = F + law_simple(L, n, delta, v);
+                F = add(F, law_simple(L, n, delta, v));
                 if (EVAL && nnew < maxc) store_spring(&hout[nnew * cap + q], mk(T(0), T(0), T(0)), gid);
             }
             ++nnew;
@@ -549,7 +549,7 @@ __global__ void __launch_bounds__(ITEM_THREADS, 2) k_items(ItemArgs<PR> a) {
             const T gx = sizeof(T) == 8 ? (T)S.g[0] : (T)S.g_f[0];
             const T gy = sizeof(T) == 8 ? (T)S.g[1] : (T)S.g_f[1];
             const T gz = sizeof(T) == 8 ? (T)S.g[2] : (T)S.g_f[2];
-            F = F + mk(gx, gy, gz) * mi;
+            F = axpy(mk(gx, gy, gz), mi, F);
         }
         if (EVAL) {
             const size_t o = 3 * (size_t)me.id;

@@ -168,12 +168,12 @@ __global__ void __launch_bounds__(256, PR::WALK_BLOCKS) k_force(ForceArgs<PR> a)
             const V3<T> dold = find_spring(s_oid, bd, tid, cnt_old, gid, a.hin, cap, src);
             V3<T> Fc, Ftc, dnew, Mr;
             law_practical<TERMS, STIFF>(L, n, delta, v, rw, Reff, meff, dold, Fc, Ftc, dnew, me.w - wj, Mr);
-            F = F + Fc;
-            Tq = Tq + cross(n, Ftc) * ri;
-            if (TERMS) Tq = Tq + Mr;
+            F = add(F, Fc);
+            Tq = axpy(cross(n, Ftc), ri, Tq);
+            if (TERMS) Tq = add(Tq, Mr);
             if (nnew < maxc) store_spring(&a.hout[nnew * cap + q], dnew, gid);
         } else {
-            F = F + law_simple(L, n, delta, v);
+            F = add(F, law_simple(L, n, delta, v));
             if (EVAL && nnew < maxc) store_spring(&a.hout[nnew * cap + q], mk(T(0), T(0), T(0)), gid);
         }
         ++nnew;
@@ -190,16 +190,16 @@ __global__ void __launch_bounds__(256, PR::WALK_BLOCKS) k_force(ForceArgs<PR> a)
             const V3<T> v = me.v - PR::wall_vel(W, cp);
             const uint32_t gid = DEM_WALL_BASE + (uint32_t)w;
             if (PRACT) {
-                const V3<T> rw = me.w * ri;
+                const V3<T> rw = scale(me.w, ri);
                 const V3<T> dold = find_spring(s_oid, bd, tid, cnt_old, gid, a.hin, cap, src);
                 V3<T> Fc, Ftc, dnew, Mr;
                 law_practical<TERMS, STIFF>(L, n, delta, v, rw, ri, mi, dold, Fc, Ftc, dnew, me.w - PR::wall_omega(W), Mr);
-                F = F + Fc;
-                Tq = Tq + cross(n, Ftc) * ri;
-                if (TERMS) Tq = Tq + Mr;
+                F = add(F, Fc);
+                Tq = axpy(cross(n, Ftc), ri, Tq);
+                if (TERMS) Tq = add(Tq, Mr);
                 if (nnew < maxc) store_spring(&a.hout[nnew * cap + q], dnew, gid);
             } else {
-                F = F + law_simple(L, n, delta, v);
+                F = add(F, law_simple(L, n, delta, v));
                 if (EVAL && nnew < maxc) store_spring(&a.hout[nnew * cap + q], mk(T(0), T(0), T(0)), gid);
             }
             ++nnew;
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(256, PR::WALK_BLOCKS) k_force(ForceArgs<PR> a)
             const T gx = sizeof(T) == 8 ? (T)S.g[0] : (T)S.g_f[0];
             const T gy = sizeof(T) == 8 ? (T)S.g[1] : (T)S.g_f[1];
             const T gz = sizeof(T) == 8 ? (T)S.g[2] : (T)S.g_f[2];
-            F = F + mk(gx, gy, gz) * mi;
+            F = axpy(mk(gx, gy, gz), mi, F);
         }
         if (EVAL) {
             const size_t o = 3 * (size_t)me.id;

@@ -225,16 +225,16 @@ __global__ void __launch_bounds__(PR::LIST_THREADS, PR::LIST_BLOCKS) k_list(List
                 const T Reff = (STIFF == 0) ? T(0) : law_div(ri * rjT, ri + rjT);
                 V3<T> Fc, Ftc, dnew, Mr;
                 law_practical<TERMS, STIFF>(Lc, n, delta, v, rw, Reff, meff, dold, Fc, Ftc, dnew, wi - wj, Mr);
-                F = F + Fc;
-                Tq = Tq + cross(n, Ftc) * ri;
-                if (TERMS) Tq = Tq + Mr;
+                F = add(F, Fc);
+                Tq = axpy(cross(n, Ftc), ri, Tq);
+                if (TERMS) Tq = add(Tq, Mr);
                 if (nnew < maxc) {
                     store_spring(op, dnew, pj.id);
                     op += cap;
                     nm |= bit;
                 }
             } else {
-                F = F + law_simple(Lc, n, delta, v);
+                F = add(F, law_simple(Lc, n, delta, v));
                 if (EVAL && nnew < maxc) {
                     store_spring(op, mk(T(0), T(0), T(0)), pj.id);
                     op += cap;
@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(PR::LIST_THREADS, PR::LIST_BLOCKS) k_list(List
             const V3<T> v = me2.v - PR::wall_vel(W, cp);
             const uint32_t gid = DEM_WALL_BASE + (uint32_t)w;
             if (PRACT) {
-                const V3<T> rw = me2.w * ri;
+                const V3<T> rw = scale(me2.w, ri);
                 V3<T> dold = mk(T(0), T(0), T(0));
                 for (uint32_t k = w_first; k < cnt_old; ++k) {
                     const Spring<T> r = load_spring(&hin[k * cap + src]);
@@ -265,12 +265,12 @@ __global__ void __launch_bounds__(PR::LIST_THREADS, PR::LIST_BLOCKS) k_list(List
                 }
                 V3<T> Fc, Ftc, dnew, Mr;
                 law_practical<TERMS, STIFF>(L, n, delta, v, rw, ri, mi, dold, Fc, Ftc, dnew, me2.w - PR::wall_omega(W), Mr);
-                F = F + Fc;
-                Tq = Tq + cross(n, Ftc) * ri;
-                if (TERMS) Tq = Tq + Mr;
+                F = add(F, Fc);
+                Tq = axpy(cross(n, Ftc), ri, Tq);
+                if (TERMS) Tq = add(Tq, Mr);
                 if (nnew < maxc) store_spring(&hout[nnew * cap + q], dnew, gid);
             } else {
-                F = F + law_simple(L, n, delta, v);
+                F = add(F, law_simple(L, n, delta, v));
                 if (EVAL && nnew < maxc) store_spring(&hout[nnew * cap + q], mk(T(0), T(0), T(0)), gid);
             }
             ++nnew;
@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(PR::LIST_THREADS, PR::LIST_BLOCKS) k_list(List
             const T gx = sizeof(T) == 8 ? (T)S.g[0] : (T)S.g_f[0];
             const T gy = sizeof(T) == 8 ? (T)S.g[1] : (T)S.g_f[1];
             const T gz = sizeof(T) == 8 ? (T)S.g[2] : (T)S.g_f[2];
-            F = F + mk(gx, gy, gz) * mi;
+            F = axpy(mk(gx, gy, gz), mi, F);
         }
         if (EVAL) {
             const size_t o = 3 * (size_t)me2.id;

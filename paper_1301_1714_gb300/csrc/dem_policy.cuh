@@ -219,9 +219,9 @@ struct PF64 {
                                                          bool& finite, float4& pnew) {
         const double r = (double)me.r;
         const double I = 0.4 * m * r * r;
-        const V3<double> vn = me.v + F * (S.dt / m);
-        const V3<double> wn = me.w + Tq * (S.dt / I);
-        const double xn = me.x + vn.x * S.dt, yn = me.y + vn.y * S.dt, zn = me.z + vn.z * S.dt;
+        const V3<double> vn = axpy(F, S.dt / m, me.v);
+        const V3<double> wn = axpy(Tq, S.dt / I, me.w);
+        const double xn = __fma_rn(vn.x, S.dt, me.x), yn = __fma_rn(vn.y, S.dt, me.y), zn = __fma_rn(vn.z, S.dt, me.z);
         B.x[q] = xn; B.y[q] = yn; B.z[q] = zn;
         B.r[q] = me.r;
         B.vx[q] = vn.x; B.vy[q] = vn.y; B.vz[q] = vn.z;
@@ -561,7 +561,7 @@ struct PF32 {
             n = mk(-W.nf[0], -W.nf[1], -W.nf[2]);
             delta = d;
             const float s = __fadd_rn(sh, sl);
-            cp = mk((u[0] + ul[0]) - s * W.nf[0], (u[1] + ul[1]) - s * W.nf[1], (u[2] + ul[2]) - s * W.nf[2]);
+            cp = axpy(mk(W.nf[0], W.nf[1], W.nf[2]), -s, mk(u[0] + ul[0], u[1] + ul[1], u[2] + ul[2]));
             return true;
         }
         if (W.kind == 2) return half_plate(W, me, S, n, delta, cp);
@@ -649,8 +649,8 @@ struct PF32 {
                                                          bool& finite, float4& pnew) {
         const float r = me.r;
         const float I = 0.4f * m * r * r;
-        const V3<float> vn = me.v + F * (S.dt_f / m);
-        const V3<float> wn = me.w + Tq * (S.dt_f / I);
+        const V3<float> vn = axpy(F, S.dt_f / m, me.v);
+        const V3<float> wn = axpy(Tq, S.dt_f / I, me.w);
         float hx = me.hx, hy = me.hy, hz = me.hz, lx = me.lx, ly = me.ly, lz = me.lz;
         advance(hx, lx, __fmul_rn(vn.x, S.dt_f));
         advance(hy, ly, __fmul_rn(vn.y, S.dt_f));
