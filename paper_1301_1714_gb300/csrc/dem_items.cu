@@ -115,6 +115,14 @@ struct ItemMem {
     }
 };
 
+// Whether two stored particles touch, as PF64::exact_j decides it (out of line: few blocks ask).
+__device__ __noinline__ bool touch(const double* x, const double* y, const double* z, const float* r, uint32_t i,
+                                   uint32_t j) {
+    const double dx = __dsub_rn(x[j], x[i]), dy = __dsub_rn(y[j], y[i]), dz = __dsub_rn(z[j], z[i]);
+    const double R = __dadd_rn((double)r[i], (double)r[j]);
+    return __fma_rn(dz, dz, __fma_rn(dy, dy, __dmul_rn(dx, dx))) < __dmul_rn(R, R);
+}
+
 template <class PR, bool LIST, int MODEL, bool EVAL>
 __global__ void __launch_bounds__(ITEM_THREADS, 2) k_items(ItemArgs<PR> a) {
     using T = typename PR::T;
@@ -267,7 +275,24 @@ __global__ void __launch_bounds__(ITEM_THREADS, 2) k_items(ItemArgs<PR> a) {
         j1 = __ldg(&a.cs[base + (uint32_t)min(pix + 1, PS.dims[0] - 1) + 1u]);
     };
     auto walk_near = [&](uint32_t j) {
-        return j != q0 + p && !far_f(pp, sizeof(T) == 8 ? __ldg(&a.ref[j]) : PR::pre(A, j), peps);
+        if (sizeof(T) == 4) return j != q0 + p && near_f(pp, PR::pre(A, j), peps);   // (as k_force)
+        return j != q0 + p && !far_f(pp, __ldg(&a.ref[j]), peps);
+    };
+    bool exact = false;   // FP64: candidates are contacts (below)
+    auto touches = [&](uint32_t j) {
+        if constexpr (sizeof(T) == 8) return touch(A.x, A.y, A.z, A.r, q0 + p, j);
+        else return true;
+    };
+    auto count_rows = [&](auto passes) {
+        for (uint32_t r = sub; r < 9u; r += G) {
+            uint32_t c = 0;
+            if (plive) {
+                uint32_t j0, j1;
+                row(r, j0, j1);
+                for (uint32_t j = j0; j < j1; ++j) c += passes(j) ? 1u : 0u;
+            }
+            rows[p * 9u + r] = (uint16_t)min(c, 0xFFFFu);
+        }
     };
     if (LIST) {
         if (!direct) {
@@ -286,15 +311,7 @@ __global__ void __launch_bounds__(ITEM_THREADS, 2) k_items(ItemArgs<PR> a) {
                     atomicOr(&near[2 * p + (k >> 5)], 1u << (k & 31u));
         }
     } else {
-        for (uint32_t r = sub; r < 9u; r += G) {
-            uint32_t c = 0;
-            if (plive) {
-                uint32_t j0, j1;
-                row(r, j0, j1);
-                for (uint32_t j = j0; j < j1; ++j) c += walk_near(j) ? 1u : 0u;
-            }
-            rows[p * 9u + r] = (uint16_t)min(c, 0xFFFFu);
-        }
+        count_rows(walk_near);
         if (PRACT) {
             const uint32_t c = s_cold[p], src = s_src[p];
             for (uint32_t k = sub; k < c; k += G) s_pid[k * P + p] = __ldg(&hin[k * cap + src].pid);
@@ -308,14 +325,27 @@ __global__ void __launch_bounds__(ITEM_THREADS, 2) k_items(ItemArgs<PR> a) {
             mycnt = (uint32_t)(__popc(near[2 * tid]) + __popc(near[2 * tid + 1]));
         } else {
             for (uint32_t r = 0; r < 9u; ++r) mycnt += rows[tid * 9u + r];
-            // more candidates than slots: FP32 counts what passes the prefilter, FP64 contacts
-            // (below); no particle has more than a round holds
-            const uint32_t most = sizeof(T) == 8 ? ITEM_MAX : maxc;
-            if (mycnt > most) {
-                raise_status(a.st, ST_CAPACITY, (int32_t)q);
-                if (!EVAL && a.halt) atomicOr(&s_flag, DEM_HALT);
-                mycnt = most;
-            }
+        }
+    }
+    if (!LIST) {
+        // FP64: the prefilter's margin grows with the coordinates, and far from the origin it
+        // passes spheres that are nowhere near: a block with a particle that has more of them
+        // than a round holds counts contacts instead
+        if (sizeof(T) == 8 && __syncthreads_or(mycnt > ITEM_MAX ? 1 : 0)) {
+            exact = true;
+            count_rows([&](uint32_t j) { return walk_near(j) && touches(j); });
+            __syncthreads();
+            mycnt = 0;
+            if (mine && live)
+                for (uint32_t r = 0; r < 9u; ++r) mycnt += rows[tid * 9u + r];
+        }
+        // more candidates than slots: FP32 counts what passes the prefilter, FP64 contacts
+        // (below); no particle has more than a round holds
+        const uint32_t most = sizeof(T) == 8 ? ITEM_MAX : maxc;
+        if (mycnt > most) {
+            raise_status(a.st, ST_CAPACITY, (int32_t)q);
+            if (!EVAL && a.halt) atomicOr(&s_flag, DEM_HALT);
+            mycnt = most;
         }
     }
     {
@@ -384,7 +414,7 @@ __global__ void __launch_bounds__(ITEM_THREADS, 2) k_items(ItemArgs<PR> a) {
                     if (rows[p * 9u + r] == 0) continue;
                     row(r, j0, j1);
                     for (uint32_t j = j0; j < j1 && k < limit; ++j)
-                        if (walk_near(j)) {
+                        if (walk_near(j) && (!exact || touches(j))) {
                             const uint32_t local = j - q0;
                             add(k++, j, local < P ? local : P, 0u);
                         }
