@@ -523,23 +523,40 @@ int auto_block(const Domain& d, uint32_t n) {
 }
 
 // Particles per tile of list mode (a multiple of 32; in FP32 mode also the threads of a
-// force-pass block): at most four times the configured block size, and by the number of
-// particles the tile that gives the busiest SM the least work, its halo counted at 0.15 of a
-// particle per entry (halo entries per particle of a dense bed beside each size). Measured
-// per pass with 512 or 256 / the choice: 262,144 spheres 2,399 / 2,319 us (448), 131,072 in the
-// hopper 2,185 / 2,053 (448), 100,003 861 / 810 (224). Few particles, and FP64 mode (powers of
-// two): the largest tile that still gives two blocks per SM.
-uint32_t tile_size(const Domain& d, uint32_t n) {
-    const uint32_t most = std::min(d.precision == 0 ? (uint32_t)DEM_TILE_MAX_FP64 : (uint32_t)DEM_TILE_MAX,
-                                   4u * (uint32_t)d.block);
+// force-pass block) for scenes of the given sizes: at most four times the configured block
+// size, and no more than the largest scene fills (every scene has its own tiles: 1,000 scenes of
+// 64 spheres with a tile for their total, 448, took 1,495 us per 20 steps, with 64 824). Then,
+// by the number of particles, the tile that gives the busiest SM the least work, its halo
+// counted at 0.15 of a particle per entry (halo entries per particle of a dense bed beside each
+// size). Measured per pass with 512 or 256 / the choice: 262,144 spheres 2,399 / 2,319 us (448),
+// 131,072 in the hopper 2,185 / 2,053 (448), 100,003 861 / 810 (224). Few particles, and FP64
+// mode (powers of two): the largest tile that still gives two blocks per SM.
+uint32_t tile_size(const Domain& d, const std::vector<uint32_t>& scenes) {
+    uint64_t n = 0;
+    uint32_t largest = 0;
+    for (const uint32_t m : scenes) {
+        n += m;
+        largest = std::max(largest, m);
+    }
+    auto tiles = [&](uint32_t t) {
+        uint64_t k = 0;
+        for (const uint32_t m : scenes) k += (m + t - 1) / t;
+        return k;
+    };
+    const bool f64 = d.precision == 0;
     const uint32_t sms = (uint32_t)(d.sort_blocks / 8);
-    if (d.precision != 0 && n >= 224u * sms) {
+    uint32_t most = std::min(f64 ? (uint32_t)DEM_TILE_MAX_FP64 : (uint32_t)DEM_TILE_MAX, 4u * (uint32_t)d.block) & ~31u;
+    const uint32_t fill = std::max(64u, (largest + 31u) & ~31u);
+    if (!f64) most = std::min(most, fill);
+    else
+        while (most > 64 && most / 2 >= fill) most /= 2;
+    if (!f64 && n >= 224ull * sms) {
         static const struct { uint32_t tile; double halo; } sizes[] = {{512, 0.89}, {448, 0.94}, {320, 1.08}, {224, 1.26}};
-        uint32_t best = most & ~31u;
+        uint32_t best = most;
         double least = 0.0;
         for (const auto& s : sizes) {
             if (s.tile > most) continue;
-            const uint32_t blocks = (n + s.tile - 1) / s.tile, per = (blocks + sms - 1) / sms;
+            const uint64_t per = (tiles(s.tile) + sms - 1) / sms;
             const double work = (double)per * s.tile * (1.0 + 0.15 * s.halo);
             if (least == 0.0 || work < 0.97 * least) {
                 least = work;
@@ -549,8 +566,8 @@ uint32_t tile_size(const Domain& d, uint32_t n) {
         return best;
     }
     uint32_t t = most;
-    while (t > 64 && n / t < 2u * sms) t = t > 256 ? 256 : t / 2;
-    return std::max(32u, t & ~31u);
+    while (t > 64 && tiles(t) < 2u * sms) t = t > 256 ? 256 : std::max(64u, (t / 2) & ~31u);
+    return t;
 }
 
 // Grid of Sec. 4.1 over the configured domain: cell edge >= one diameter of the largest
@@ -624,7 +641,7 @@ dem_status load_particles(dem_handle* h, int64_t n64, const double* x, const dou
     d.n = n;
     d.ncells = (uint32_t)nc;
     if (h->cfg.block_size == 0 && !d.list_mode) d.block = auto_block(d, n);
-    d.tile = tile_size(d, n);
+    d.tile = tile_size(d, {n});
     d.ntiles = (n + d.tile - 1) / d.tile;
     s = ensure_buffers(h, n, (uint32_t)nc);
     if (s != DEM_OK) return s;
@@ -1616,7 +1633,10 @@ dem_status repack(dem_batch* b) {
     nd.n = (uint32_t)n_new;
     nd.ncells = (uint32_t)std::max<uint64_t>(c_new, 1);
     if (b->auto_block && !nd.list_mode) nd.block = auto_block(nd, nd.n);
-    nd.tile = tile_size(nd, nd.n);
+    std::vector<uint32_t> sizes;
+    for (auto* group : {&kept, &fresh})
+        for (const BatchScene* sc : *group) sizes.push_back((uint32_t)sc->n);
+    nd.tile = tile_size(nd, sizes);
     uint32_t tiles = 0;
     for (auto* group : {&kept, &fresh})
         for (BatchScene* sc : *group) {
