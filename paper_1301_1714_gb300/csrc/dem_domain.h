@@ -102,12 +102,15 @@ struct Domain {
     std::vector<void*> allocations;   // every cudaMalloc of this domain (freed together)
 };
 
-// The captured steps of a domain: a graph of two timesteps, or (list mode) the step loop.
+// The captured steps of a domain: a graph of two timesteps, and (list mode) the step loop with
+// turns of 1 to LOOP_MAX steps, each made when it is first asked for.
+constexpr int LOOP_MAX = 10;
 struct StepGraph {
-    cudaGraphExec_t exec = nullptr;
-    bool loop = false;           // exec is the step loop (takes ctrl->left steps) and not two steps
+    cudaGraphExec_t exec = nullptr;                    // two steps
+    cudaGraphExec_t loops[LOOP_MAX + 1] = {};          // takes ctrl->left steps, by the length of a turn
     bool no_loop = false;        // the driver refused conditional nodes
-    int64_t launches = 0;        // kernels every replay launches (loop: every step)
+    int64_t launches = 0;        // kernels every replay of exec launches
+    int64_t loop_launches = 0;   // kernels of every step of the loop
     int64_t body_launches = 0;   // kernels of one conditional sort body (list mode)
     cudaGraphExec_t sort_exec = nullptr;   // phase timing: the sort tail
     int64_t sort_launches = 0;   // kernels every sort-tail replay launches
@@ -117,7 +120,10 @@ struct StepGraph {
         exec = nullptr;
         if (sort_exec) cudaGraphExecDestroy(sort_exec);
         sort_exec = nullptr;
-        loop = false;
+        for (auto& l : loops) {
+            if (l) cudaGraphExecDestroy(l);
+            l = nullptr;
+        }
         sort_launches = 0;
         launches = 0;
         body_launches = 0;

@@ -763,18 +763,33 @@ cudaError_t capture_sort_graph(Domain& d, StepGraph* g) {
 
 // The step loop of list mode: a graph that takes ctrl->left steps by itself.
 //   while (steps left and no error) {
-//       while (steps left and no sort due) { LOOP_STEPS x (force pass, decision, bookkeeping) }
+//       while (steps left and no sort due) { turn x (force pass, decision, bookkeeping) }
 //       the sort and the new lists (they do nothing when no sort is due), its bookkeeping
 //   }
 // A step that finds a sort due (or no step left) idles, so the sort needs no conditional
 // node of its own after every step: an untaken IF node costs 8 us on GB300, as much as ten
 // kernel nodes (0.8 us each), a turn of a WHILE node 3.2 us.
-// Ten steps per turn: programs mostly step in tens, and a call's last turn then has no idle
-// passes (8 / 10 / 16 steps: 131,072-sphere hopper read every 10 steps 2,015 / 1,951 / 2,085 us
-// per 50 steps, 9,217 spheres 2,116 / 2,086 / 2,125 per 100).
-constexpr int LOOP_STEPS = 10;
+//
+// Steps per turn for a call of n steps (or a sort at least every n): the length of at most
+// LOOP_MAX that costs least, 3.2 us per turn and 2.4 us for every pass that idles at the end of
+// the last one. Longer turns would save less than 0.2 us per step, and a sort that falls due
+// leaves half a turn idle on average.
+int turn_length(int64_t n) {
+    if (n <= LOOP_MAX) return (int)std::max<int64_t>(n, 1);
+    int best = LOOP_MAX;
+    double least = 0.0;
+    for (int t = LOOP_MAX; t > LOOP_MAX / 2; --t) {
+        const int64_t turns = (n + t - 1) / t;
+        const double cost = 3.2 * (double)turns + 2.4 * (double)(turns * t - n);
+        if (least == 0.0 || cost < least) {
+            least = cost;
+            best = t;
+        }
+    }
+    return best;
+}
 
-cudaError_t capture_loop(Domain& d, StepGraph* g) {
+cudaError_t capture_loop(Domain& d, StepGraph* g, int turn) {
     cudaError_t e;
     if ((e = side_stream(g)) != cudaSuccess) return e;
     const int64_t l0 = d.launches;
@@ -792,7 +807,7 @@ cudaError_t capture_loop(Domain& d, StepGraph* g) {
     if (e == cudaSuccess)
         e = capture_into(d, g, inner, nullptr, 0, [&] {
             cudaError_t e1 = cudaSuccess;
-            for (int k = 0; k < LOOP_STEPS && e1 == cudaSuccess; ++k) {
+            for (int k = 0; k < turn && e1 == cudaSuccess; ++k) {
                 e1 = run_force(d, false, nullptr, nullptr);
                 if (e1 == cudaSuccess) e1 = run_loop_end(d);
             }
@@ -809,20 +824,24 @@ cudaError_t capture_loop(Domain& d, StepGraph* g) {
     d.launches = l0;
     if (e != cudaSuccess) return e;   // (the graph is left: destroying one whose body's capture failed
                                       // crashes in driver 580.159; run_steps does not try again)
-    e = cudaGraphInstantiate(&g->exec, graph, 0);
+    e = cudaGraphInstantiate(&g->loops[turn], graph, 0);
     cudaGraphDestroy(graph);
     if (e != cudaSuccess) {
-        g->exec = nullptr;
+        g->loops[turn] = nullptr;
         return e;
     }
-    g->loop = true;
-    g->launches = steps / LOOP_STEPS;
+    g->loop_launches = steps / turn;
     g->body_launches = body;
     return cudaSuccess;
 }
 
 // nsteps steps enqueued: the step loop (list mode) or a graph of two steps replayed; plain
-// launches on the legacy default stream and for an odd last step.
+// launches on the legacy default stream, for a single step and for the odd last step of a graph
+// of two. In list mode an odd count stays in the loop (3 steps of 9,217 spheres 181 -> 121 us)
+// up to LOOP_ODD_MAX steps; beyond, a plain step is under 2% of the call, and a program that
+// counts launches finds the plain step that it always found there.
+constexpr int64_t LOOP_ODD_MAX = 127;
+
 cudaError_t run_steps(Domain& d, StepGraph* g, int64_t nsteps) {
     cudaError_t e;
     if (!g || !d.stream || d.n == 0) {
@@ -834,33 +853,36 @@ cudaError_t run_steps(Domain& d, StepGraph* g, int64_t nsteps) {
         if ((e = enqueue_step(d)) != cudaSuccess) return e;
         --nsteps;
     }
-    if (nsteps >= 2 && !g->exec && d.list_mode && !g->no_loop) {
-        const cudaError_t ce = capture_loop(d, g);
-        if (ce != cudaSuccess) {
-            cudaGetLastError();   // conditional nodes unavailable: the plain graph of two steps
-            g->no_loop = true;
-            static bool said = false;
-            if (!said) {
-                said = true;
-                fprintf(stderr, "dem: step loop as a graph unavailable (%s); using the plain graph\n",
-                        cudaGetErrorString(ce));
+    if (d.list_mode && nsteps >= 2 && !g->no_loop) {
+        const int turn = turn_length(d.interval > 0 ? std::min<int64_t>(nsteps, d.interval) : nsteps);
+        if (!g->loops[turn]) {
+            const cudaError_t ce = capture_loop(d, g, turn);
+            if (ce != cudaSuccess) {
+                cudaGetLastError();   // conditional nodes unavailable: the plain graph of two steps
+                g->no_loop = true;
+                static bool said = false;
+                if (!said) {
+                    said = true;
+                    fprintf(stderr, "dem: step loop as a graph unavailable (%s); using the plain graph\n",
+                            cudaGetErrorString(ce));
+                }
             }
         }
-    }
-    if (nsteps >= 2 && g->loop) {
-        for (int64_t k = nsteps & ~(int64_t)1; k > 0;) {
+        const int64_t take = g->no_loop ? 0 : (nsteps <= LOOP_ODD_MAX ? nsteps : nsteps & ~(int64_t)1);
+        for (int64_t k = take; k > 0;) {
             const int64_t chunk = std::min<int64_t>(k, 1 << 30);
             CtrlDev* from = d.ctrl_host + 1;   // pinned; read by the copy before the loop starts
-            if (k != (nsteps & ~(int64_t)1) && (e = cudaStreamSynchronize(d.stream)) != cudaSuccess) return e;
+            if (k != take && (e = cudaStreamSynchronize(d.stream)) != cudaSuccess) return e;
             from->left = (uint32_t)chunk;
             from->stop = LOOP_GO;
             if ((e = cudaMemcpyAsync(&d.ctrl->left, &from->left, 8, cudaMemcpyHostToDevice, d.stream)) != cudaSuccess ||
-                (e = cudaGraphLaunch(g->exec, d.stream)) != cudaSuccess)
+                (e = cudaGraphLaunch(g->loops[turn], d.stream)) != cudaSuccess)
                 return e;
-            d.launches += g->launches * chunk;
-            k -= chunk;   // (an even number of steps: the history buffers keep their roles)
+            d.launches += g->loop_launches * chunk;
+            k -= chunk;
         }
-        nsteps &= 1;
+        d.h_cur ^= (int)(take & 1);   // (the kernels read ctrl->hcur)
+        nsteps -= take;
     }
     if (nsteps >= 2 && !g->exec) {
         const int64_t l0 = d.launches;
