@@ -66,13 +66,15 @@ __global__ void __launch_bounds__(256) k_wall_masks(uint32_t n, const SceneDev* 
 // lanes look the cells up together (one each), number the candidates through by a scan of
 // the counts, read up to NLIST_REGS x 32 of them into registers once, and test all 32 lanes'
 // candidates against one particle of the cell at a time; the accepted ones are ranked by id
-// in shared memory. (One thread per particle walked 27 x 0-5 candidates with its neighbours
+// in shared memory. A warp takes `per` consecutive positions: 32, and less for few particles,
+// whose warps would otherwise walk their 10 to 16 cells one after another with most of the chip
+// idle (9,217 spheres: 49.8 us with 32, 15.0 with 4; 500: 43.2 and 13.3). (One thread per particle walked 27 x 0-5 candidates with its neighbours
 // in the warp on other cells, and sorted its list by insertion in local memory: 2.9 ms per
 // sort of the 4,194,304-sphere bed at 59 candidates and 10 list entries per particle.)
 constexpr int NLIST_REGS = 3;
 
 template <class PR>
-__global__ void __launch_bounds__(256) k_nlist(uint32_t n, const SceneDev* __restrict__ scenes, int nscenes, typename PR::State S0,
+__global__ void __launch_bounds__(256) k_nlist(uint32_t n, uint32_t per, const SceneDev* __restrict__ scenes, int nscenes, typename PR::State S0,
                                                typename PR::State S1, const CtrlDev* ctrl,
                                                const uint32_t* __restrict__ key, const uint32_t* __restrict__ canon,
                                                const uint32_t* __restrict__ cs, const uint32_t* __restrict__ fin,
@@ -89,10 +91,10 @@ __global__ void __launch_bounds__(256) k_nlist(uint32_t n, const SceneDev* __res
     // the lane's cell of the 27 (lanes 27-31: none)
     const int dx = (int)(lane % 3u) - 1, dy = (int)((lane / 3u) % 3u) - 1, dz = (int)(lane / 9u) - 1;
     const uint32_t warps = gridDim.x * (blockDim.x >> 5);
-    for (uint32_t base = (blockIdx.x * (blockDim.x >> 5) + wid) * 32u; base < n; base += warps * 32u) {
-        // 32 (cell, id) positions: stored position, cell and FP32 position of each
+    for (uint32_t base = (blockIdx.x * (blockDim.x >> 5) + wid) * per; base < n; base += warps * per) {
+        // `per` (cell, id) positions: stored position, cell and FP32 position of each
         const uint32_t s = base + lane;
-        const bool valid = s < n;
+        const bool valid = lane < per && s < n;
         uint32_t q = 0, kk = 0xFFFFFFFFu;
         int sidx = 0, ix = 0, iy = 0, iz = 0;
         float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -241,33 +243,42 @@ __global__ void __launch_bounds__(512) k_tile(const SceneDev* scenes, int nscene
             const uint32_t src = valid ? perm[q] : 0u;
             const uint32_t c = valid ? min(hcnt[src], maxc) : 0u;
             uint32_t o = 0, kept = 0, pid = c ? hs[src].pid : DEM_WALL_BASE;
-            for (uint32_t k = 0; k < m; ++k) {
-                const uint32_t j = nl[(size_t)k * cap + q];
-                if (o < c && pid < DEM_WALL_BASE) {
-                    const uint32_t idj = __ldg(&A.id[j]);
-                    while (o < c && pid < idj) {   // a partner that left the list
-                        ++o;
-                        pid = o < c ? hs[(size_t)o * cap + src].pid : DEM_WALL_BASE;
-                    }
-                    if (o < c && pid == idj) {
-                        if (kept != o) hs[(size_t)kept * cap + src] = hs[(size_t)o * cap + src];
-                        ++kept;
-                        mask |= 1ull << k;
-                        ++o;
-                        pid = o < c ? hs[(size_t)o * cap + src].pid : DEM_WALL_BASE;
-                    }
-                }
-                if (j - q0 >= n && *(volatile uint32_t*)&s_n <= hcap) {
-                    uint32_t h = (j * 2654435761u) >> 21;   // 11 bits
-                    for (;;) {
-                        const uint32_t old = atomicCAS(&s_key[h], 0xFFFFFFFFu, j);
-                        if (old == 0xFFFFFFFFu) {
-                            const uint32_t at = atomicAdd(&s_n, 1u);
-                            if (at < hcap) s_list[at] = j;
-                            break;
+            for (uint32_t k0 = 0; k0 < m; k0 += 4) {
+                // four entries and their ids in flight together
+                uint32_t jj[4], id[4];
+#pragma unroll
+                for (uint32_t u = 0; u < 4; ++u) jj[u] = k0 + u < m ? nl[(size_t)(k0 + u) * cap + q] : q0;
+#pragma unroll
+                for (uint32_t u = 0; u < 4; ++u) id[u] = o < c ? __ldg(&A.id[jj[u]]) : 0u;
+#pragma unroll
+                for (uint32_t u = 0; u < 4; ++u) {
+                    const uint32_t k = k0 + u, j = jj[u], idj = id[u];
+                    if (k >= m) break;
+                    if (o < c && pid < DEM_WALL_BASE) {
+                        while (o < c && pid < idj) {   // a partner that left the list
+                            ++o;
+                            pid = o < c ? hs[(size_t)o * cap + src].pid : DEM_WALL_BASE;
                         }
-                        if (old == j) break;
-                        h = (h + 1) & (TILE_HASH - 1);
+                        if (o < c && pid == idj) {
+                            if (kept != o) hs[(size_t)kept * cap + src] = hs[(size_t)o * cap + src];
+                            ++kept;
+                            mask |= 1ull << k;
+                            ++o;
+                            pid = o < c ? hs[(size_t)o * cap + src].pid : DEM_WALL_BASE;
+                        }
+                    }
+                    if (j - q0 >= n && *(volatile uint32_t*)&s_n <= hcap) {
+                        uint32_t h = (j * 2654435761u) >> 21;   // 11 bits
+                        for (;;) {
+                            const uint32_t old = atomicCAS(&s_key[h], 0xFFFFFFFFu, j);
+                            if (old == 0xFFFFFFFFu) {
+                                const uint32_t at = atomicAdd(&s_n, 1u);
+                                if (at < hcap) s_list[at] = j;
+                                break;
+                            }
+                            if (old == j) break;
+                            h = (h + 1) & (TILE_HASH - 1);
+                        }
                     }
                 }
             }
@@ -349,12 +360,16 @@ static inline uint32_t sgrid(const Domain& d, uint32_t n) {
 
 cudaError_t run_lists(Domain& d) {
     if (d.n == 0) return cudaSuccess;
+    // 16 warps per SM, as far as warps of at least four positions reach
+    uint32_t per = 32;
+    while (per > 4 && d.n / per < 2u * (uint32_t)d.sort_blocks) per /= 2;
+    const uint32_t grid = std::max(1u, std::min(nblk(d.n, 8 * per), (uint32_t)std::max(d.sort_blocks, 1)));
     if (d.precision == 0)
-        k_nlist<PF64><<<sgrid(d, d.n), 256, 0, d.stream>>>(d.n, d.d_scenes, d.nscenes, d.S64[0], d.S64[1], d.ctrl, d.key,
-                                                          d.canon, d.cs, d.fin, d.ncnt, d.nl, d.cap, d.wmask, d.st);
+        k_nlist<PF64><<<grid, 256, 0, d.stream>>>(d.n, per, d.d_scenes, d.nscenes, d.S64[0], d.S64[1], d.ctrl, d.key,
+                                                  d.canon, d.cs, d.fin, d.ncnt, d.nl, d.cap, d.wmask, d.st);
     else
-        k_nlist<PF32><<<sgrid(d, d.n), 256, 0, d.stream>>>(d.n, d.d_scenes, d.nscenes, d.S32[0], d.S32[1], d.ctrl, d.key,
-                                                          d.canon, d.cs, d.fin, d.ncnt, d.nl, d.cap, d.wmask, d.st);
+        k_nlist<PF32><<<grid, 256, 0, d.stream>>>(d.n, per, d.d_scenes, d.nscenes, d.S32[0], d.S32[1], d.ctrl, d.key,
+                                                  d.canon, d.cs, d.fin, d.ncnt, d.nl, d.cap, d.wmask, d.st);
     DEM_LAUNCH_CHECK();
     return run_tiles(d, false);
 }
