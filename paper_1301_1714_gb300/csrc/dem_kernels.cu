@@ -999,15 +999,17 @@ static cudaError_t force_impl(Domain& d, const typename PR::State& S0, const typ
     return cudaSuccess;
 }
 
-// Below this many particles the FP32 walk takes its contacts by items (dem_items.cu): a thread
-// per particle then leaves most of the chip idle. Measured per step on dense boxes (items /
-// thread per particle): 2,049 spheres 34 / 47 us, 9,001 37 / 50, 30,001 57 / 52, 100,001 125 /
-// 59. (With neighbour lists the thread per particle wins at any size: 21.2 / 22.3 us at 9,217.)
-constexpr uint32_t WALK_ITEMS_BELOW = 20000;
+// Few particles of the FP32 walk take their contacts by items (dem_items.cu): a thread per
+// particle then leaves most of the chip idle. The line is 128 per SM, from where on the items'
+// blocks hold 128 particles each and barely more than one block per SM is left (19,456 on GB300).
+// Measured per 20 steps, items / thread per particle: 2,048 spheres 599 / 859 us, 9,001 659 / 924,
+// 17,001 806 / 967 and with the simple law 725 / 748; 19,999 1,007 / 934 and 905 / 723. (With
+// neighbour lists the thread per particle wins at any size: 21.2 / 22.3 us at 9,217.)
+static bool walk_by_items(const Domain& d) { return d.n < 128u * (uint32_t)(d.sort_blocks / 8); }
 
 cudaError_t run_force(Domain& d, bool eval, double* dbgF, double* dbgT) {
     if (d.n == 0) return cudaSuccess;
-    if (d.precision == 0 || (!d.list_mode && d.n < WALK_ITEMS_BELOW)) return run_force_items(d, eval, dbgF, dbgT);
+    if (d.precision == 0 || (!d.list_mode && walk_by_items(d))) return run_force_items(d, eval, dbgF, dbgT);
     if (d.list_mode) return run_force_list(d, eval, dbgF, dbgT);
     return force_impl<PF32>(d, d.S32[0], d.S32[1], eval, dbgF, dbgT);
 }
