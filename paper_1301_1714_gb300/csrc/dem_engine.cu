@@ -1305,39 +1305,35 @@ dem_status dem_restore(dem_handle* h, int64_t n, const double* x, const double* 
     // per-particle lists in id order; after the first sort perm[q] is the id position. List
     // mode keeps them in ascending partner id (walls last), whatever order the records have.
     const size_t N = d.cap, M = d.maxc;
-    std::vector<uint32_t> cnt(N, 0);
-    std::vector<HostSpring> sp(M * N, HostSpring{});
-    auto add = [&](uint32_t owner, uint32_t partner, double a, double b, double c) -> bool {
-        if (owner >= (uint32_t)n) return false;
-        uint32_t k = cnt[owner];
-        if (k >= M) return false;
-        cnt[owner] = k + 1;
-        if (d.list_mode)
-            for (; k > 0 && sp[(size_t)(k - 1) * N + owner].pid > partner; --k)
-                sp[(size_t)k * N + owner] = sp[(size_t)(k - 1) * N + owner];
-        sp[(size_t)k * N + owner] = HostSpring{{a, b, c}, partner};
-        return true;
-    };
     const int nw = (int)h->walls.size();
-    for (int64_t k = 0; k < nrec; ++k) {
-        const uint32_t i = ri[k], j = rj[k];
-        const double* dd = rd + 3 * k;
-        bool ok;
-        if (j >= DEM_WALL_BASE) ok = (int)(j - DEM_WALL_BASE) < nw && add(i, j, dd[0], dd[1], dd[2]);
-        else ok = i < j && j < (uint32_t)n && add(i, j, dd[0], dd[1], dd[2]) && add(j, i, -dd[0], -dd[1], -dd[2]);
-        if (!ok) { h->has_particles = false; return fail(h, DEM_ERR_INVALID_ARG, "invalid or excess history record"); }
-    }
-    CK(h, cudaMemcpyAsync(d.hcnt[d.h_cur], cnt.data(), N * 4, cudaMemcpyHostToDevice, d.stream));
     auto put = [&](auto raw) -> dem_status {
         using R = decltype(raw);
         using V = std::remove_reference_t<decltype(raw.d[0])>;
-        std::vector<R> t(M * N);
-        for (size_t k = 0; k < t.size(); ++k) {
-            t[k] = R{};
-            for (int c = 0; c < 3; ++c) t[k].d[c] = (V)sp[k].d[c];
-            t[k].pid = sp[k].pid;
+        std::vector<uint32_t> cnt(N, 0);
+        std::vector<R> sp(M * N, R{});   // as the device holds them, slot-major
+        auto add = [&](uint32_t owner, uint32_t partner, double a, double b, double c) -> bool {
+            if (owner >= (uint32_t)n) return false;
+            uint32_t k = cnt[owner];
+            if (k >= M) return false;
+            cnt[owner] = k + 1;
+            if (d.list_mode)
+                for (; k > 0 && sp[(size_t)(k - 1) * N + owner].pid > partner; --k)
+                    sp[(size_t)k * N + owner] = sp[(size_t)(k - 1) * N + owner];
+            R& e = sp[(size_t)k * N + owner];
+            e.d[0] = (V)a; e.d[1] = (V)b; e.d[2] = (V)c;
+            e.pid = partner;
+            return true;
+        };
+        for (int64_t k = 0; k < nrec; ++k) {
+            const uint32_t i = ri[k], j = rj[k];
+            const double* dd = rd + 3 * k;
+            bool ok;
+            if (j >= DEM_WALL_BASE) ok = (int)(j - DEM_WALL_BASE) < nw && add(i, j, dd[0], dd[1], dd[2]);
+            else ok = i < j && j < (uint32_t)n && add(i, j, dd[0], dd[1], dd[2]) && add(j, i, -dd[0], -dd[1], -dd[2]);
+            if (!ok) { h->has_particles = false; return fail(h, DEM_ERR_INVALID_ARG, "invalid or excess history record"); }
         }
-        CK(h, cudaMemcpyAsync(d.hs[d.h_cur], t.data(), t.size() * sizeof(R), cudaMemcpyHostToDevice, d.stream));
+        CK(h, cudaMemcpyAsync(d.hcnt[d.h_cur], cnt.data(), N * 4, cudaMemcpyHostToDevice, d.stream));
+        CK(h, cudaMemcpyAsync(d.hs[d.h_cur], sp.data(), sp.size() * sizeof(R), cudaMemcpyHostToDevice, d.stream));
         // list mode: which list entries have a spring was found at the sort, before they were set
         if (d.list_mode) CK(h, run_tiles(d, true));
         CK(h, cudaStreamSynchronize(d.stream));
