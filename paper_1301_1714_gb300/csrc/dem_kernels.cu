@@ -56,9 +56,11 @@ struct ForceArgs {
 // decision, the law (Eq. 1 or Eqs. 2-10) and the springs; then walls, gravity, the
 // update (step 1) and the new cell key with its rank in the cell (step 2).
 // MODEL: 0 the practical law with linear stiffness, 1 the simple law (Eq. 1), 2 the practical
-// law with the scene's optional terms, 3 the practical law with Hertz stiffness.
+// law with the scene's optional terms, 3 the practical law with Hertz stiffness. The terms need
+// more registers than the others' 64: with 85 (three blocks per SM) 1,000,001 spheres take 7.88 ms
+// per 20 steps, 30,001 0.96; with 64 10.09 and 1.22, with 128 9.33 and 0.88.
 template <class PR, int MODEL, bool EVAL>
-__global__ void __launch_bounds__(256, PR::WALK_BLOCKS) k_force(ForceArgs<PR> a) {
+__global__ void __launch_bounds__(256, MODEL == 2 ? PR::WALK_BLOCKS - 1 : PR::WALK_BLOCKS) k_force(ForceArgs<PR> a) {
     using T = typename PR::T;
     constexpr bool PRACT = MODEL != 1;
     constexpr bool TERMS = MODEL == 2;
