@@ -202,10 +202,18 @@ __global__ void __launch_bounds__(256) k_nlist(uint32_t n, uint32_t per, const S
 // copies them in nearly coalesced runs), and every list entry is rewritten as a 16-bit index
 // into (tile, halo). A tile whose halo does not fit is marked HALO_NONE. The same pass marks
 // the list entries that have a stored spring: a particle's springs and its list are both in
-// ascending partner id, so it is a merge. A spring whose partner is not on the new list (the
-// pair has moved apart by more than the skin) is dropped, and the ones behind it move up.
+// ascending partner id, so it is a merge. A spring whose partner is not on the new list (the pair
+// has moved apart by more than the skin, or the springs were set from outside) moves behind the
+// wall springs: no contact reads it there, and it is still part of the history.
 constexpr uint32_t TILE_HASH = 2048;   // entries: a tile inserts at most halo_cap + 512 before it stops
 constexpr uint32_t TILE_SORT = 1024;   // >= halo_cap, power of two
+
+template <class T>
+__device__ __forceinline__ void swap_springs(Spring<T>* h, size_t a, size_t b) {
+    const Spring<T> t = h[a];
+    h[a] = h[b];
+    h[b] = t;
+}
 
 template <class PR>
 __global__ void __launch_bounds__(512) k_tile(const SceneDev* scenes, int nscenes, uint32_t tile, uint32_t ntiles,
@@ -213,7 +221,7 @@ __global__ void __launch_bounds__(512) k_tile(const SceneDev* scenes, int nscene
                                               const CtrlDev* ctrl, int always, const uint32_t* __restrict__ ncnt,
                                               const uint32_t* __restrict__ nl, uint2* __restrict__ nl4,
                                               uint32_t* __restrict__ halo, uint32_t* __restrict__ nhalo, size_t cap,
-                                              const uint32_t* __restrict__ perm, uint32_t* hcnt0, uint32_t* hcnt1,
+                                              const uint32_t* __restrict__ perm, const uint32_t* hcnt0, const uint32_t* hcnt1,
                                               Spring<typename PR::T>* hs0, Spring<typename PR::T>* hs1, uint64_t* hm0,
                                               uint64_t* hm1, uint32_t maxc) {
     if (!always && ctrl->rebuild != 1) return;   // no sort this step (or a void step)
@@ -222,7 +230,7 @@ __global__ void __launch_bounds__(512) k_tile(const SceneDev* scenes, int nscene
     __shared__ uint32_t s_n;
     const typename PR::State A = ctrl->cur ? S1 : S0;
     const int hl = ctrl->hlast;
-    uint32_t* hcnt = hl ? hcnt1 : hcnt0;
+    const uint32_t* hcnt = hl ? hcnt1 : hcnt0;
     Spring<typename PR::T>* hs = hl ? hs1 : hs0;
     uint64_t* hm = hl ? hm1 : hm0;
     const uint32_t tid = threadIdx.x, bd = blockDim.x;
@@ -260,7 +268,7 @@ __global__ void __launch_bounds__(512) k_tile(const SceneDev* scenes, int nscene
                             pid = o < c ? hs[(size_t)o * cap + src].pid : DEM_WALL_BASE;
                         }
                         if (o < c && pid == idj) {
-                            if (kept != o) hs[(size_t)kept * cap + src] = hs[(size_t)o * cap + src];
+                            if (kept != o) swap_springs(hs, (size_t)kept * cap + src, (size_t)o * cap + src);
                             ++kept;
                             mask |= 1ull << k;
                             ++o;
@@ -286,10 +294,8 @@ __global__ void __launch_bounds__(512) k_tile(const SceneDev* scenes, int nscene
                 ++o;
                 pid = o < c ? hs[(size_t)o * cap + src].pid : DEM_WALL_BASE;
             }
-            if (kept != o) {   // the wall springs move up
-                for (; o < c; ++o, ++kept) hs[(size_t)kept * cap + src] = hs[(size_t)o * cap + src];
-                hcnt[src] = kept;
-            }
+            if (kept != o)   // the wall springs move up
+                for (; o < c; ++o, ++kept) swap_springs(hs, (size_t)kept * cap + src, (size_t)o * cap + src);
             if (valid) hm[q] = mask;
         }
         __syncthreads();
