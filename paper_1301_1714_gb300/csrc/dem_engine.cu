@@ -1399,15 +1399,15 @@ dem_status dem_debug_snapshot(dem_handle* h, uint32_t* cell, uint32_t* order, in
     if (cell)
         for (size_t q = 0; q < n; ++q) cell[ids[q]] = skey[q];
     if (order) {
-        // storage order; list mode keeps windows ordered by contact count, so the
-        // (cell, id) order is recovered here
-        std::vector<size_t> pos(n);
-        for (size_t q = 0; q < n; ++q) pos[q] = q;
-        if (d.list_mode)
-            std::sort(pos.begin(), pos.end(), [&](size_t a, size_t b) {
-                return skey[a] != skey[b] ? skey[a] < skey[b] : ids[a] < ids[b];
-            });
-        for (size_t q = 0; q < n; ++q) order[q] = ids[pos[q]];
+        // storage order; list mode keeps tiles ordered by contact count, so the (cell, id)
+        // order is recovered here
+        for (size_t q = 0; q < n; ++q) order[q] = ids[q];
+        if (d.list_mode) {
+            std::vector<uint64_t> by(n);
+            for (size_t q = 0; q < n; ++q) by[q] = (uint64_t)skey[q] << 32 | ids[q];
+            std::sort(by.begin(), by.end());
+            for (size_t q = 0; q < n; ++q) order[q] = (uint32_t)by[q];
+        }
     }
     if (npairs) *npairs = 0;
     if (pairs || npairs) {
