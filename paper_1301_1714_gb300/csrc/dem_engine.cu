@@ -1053,7 +1053,8 @@ dem_status dem_step(dem_handle* h, int64_t nsteps) {
         // this attempt did nothing): the state is the one at the start of that step
         int64_t done = left;
         bool void_step = false;
-        if (st == DEM_ERR_CAPACITY && d.st_host->code == ST_CAPACITY && d.regrow) {
+        // (whatever was reported first: another particle of the same step may have overflowed)
+        if (st != DEM_OK && d.regrow) {
             CtrlDev c;
             dem_status s2 = read_ctrl(h, c);
             if (s2 != DEM_OK) return s2;
@@ -1089,6 +1090,7 @@ dem_status dem_step(dem_handle* h, int64_t nsteps) {
         CK(h, cudaMemsetAsync(d.cnt, 0, ((size_t)d.ncells + 1) * 4, d.stream));
         CK(h, cudaStreamSynchronize(d.stream));
         h->graph.reset();
+        if (d.st_host->code != ST_CAPACITY) return st;
         if (d.maxc >= 64) {
             char buf[200];
             snprintf(buf, sizeof buf,
