@@ -241,6 +241,11 @@ dem_status dem_get_diagnostics(dem_handle* h, double* out16);
 dem_status dem_debug_snapshot(dem_handle* h, uint32_t* cell, uint32_t* order, int64_t pair_cap, uint32_t* pairs,
                               int64_t* npairs);
 
+/* How list mode has divided the particles: out[0] particles per tile, out[1] tiles, out[2]
+ * tiles whose neighbours outside them do not fit into shared memory (their force pass reads
+ * those from global memory). Zeros when every step sorts. For tests. */
+dem_status dem_debug_tiles(dem_handle* h, int64_t* out);
+
 /* The grid in use: origin (3), cell edge, and cells per axis (3). */
 dem_status dem_get_grid(const dem_handle* h, double* origin, double* cell, int64_t* dims);
 

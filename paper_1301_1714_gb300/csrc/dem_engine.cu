@@ -1441,6 +1441,24 @@ dem_status dem_debug_snapshot(dem_handle* h, uint32_t* cell, uint32_t* order, in
     return DEM_OK;
 }
 
+dem_status dem_debug_tiles(dem_handle* h, int64_t* out) {
+    if (!h || !out) return DEM_ERR_INVALID_ARG;
+    if (h->broken) return fail(h, DEM_ERR_STATE, "handle is unusable after a CUDA error");
+    if (!h->has_particles) return fail(h, DEM_ERR_STATE, "no particles");
+    DeviceGuard g(h->device);
+    Domain& d = h->d;
+    out[0] = out[1] = out[2] = 0;
+    if (!d.list_mode || d.n == 0) return DEM_OK;
+    std::vector<uint32_t> nh;
+    const dem_status s = download_u32(h, nh, d.nhalo, d.ntiles);
+    if (s != DEM_OK) return s;
+    CK(h, cudaStreamSynchronize(d.stream));
+    out[0] = d.tile;
+    out[1] = d.ntiles;
+    for (const uint32_t k : nh) out[2] += k == HALO_NONE ? 1 : 0;
+    return DEM_OK;
+}
+
 dem_status dem_get_grid(const dem_handle* h, double* origin, double* cell, int64_t* dims) {
     if (!h) return DEM_ERR_INVALID_ARG;
     for (int a = 0; a < 3; ++a) {

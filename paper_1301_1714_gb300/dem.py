@@ -55,7 +55,7 @@ class DemError(RuntimeError):
 
 _lib = None
 _EXPORTS = ["dem_create", "dem_set_particles", "dem_set_walls", "dem_step", "dem_run_until", "dem_get_state", "dem_get_forces",
-            "dem_get_history", "dem_restore", "dem_get_diagnostics", "dem_debug_snapshot", "dem_get_grid",
+            "dem_get_history", "dem_restore", "dem_get_diagnostics", "dem_debug_snapshot", "dem_debug_tiles", "dem_get_grid",
             "dem_device_bytes", "dem_max_contacts_seen", "dem_launch_count", "dem_last_error", "dem_destroy",
             "dem_set_timing",
             "dem_get_phase_times", "dem_sort_cells_static", "dem_batch_create", "dem_batch_add", "dem_batch_run",
@@ -93,6 +93,7 @@ def lib():
     L.dem_restore.argtypes = [P, I64, P, P, P, P, I64, P, P, P]
     L.dem_get_diagnostics.argtypes = [P, P]
     L.dem_debug_snapshot.argtypes = [P, P, P, I64, P, ctypes.POINTER(I64)]
+    L.dem_debug_tiles.argtypes = [P, P]
     L.dem_get_grid.argtypes = [P, P, P, P]
     L.dem_sort_cells_static.argtypes = [I64, P, P, ctypes.c_double, P, P, P, P, P]
     L.dem_batch_create.argtypes = [I32, I32, I32, I32, I32, I32, P, ctypes.POINTER(P)]
@@ -139,8 +140,8 @@ def lib():
         if f.restype is ctypes.c_int or name in ("dem_create", "dem_set_particles", "dem_set_walls", "dem_step",
                                                   "dem_run_until",
                                                   "dem_get_state", "dem_get_forces", "dem_get_history", "dem_restore",
-                                                  "dem_get_diagnostics", "dem_debug_snapshot", "dem_get_grid",
-                                                  "dem_set_timing", "dem_get_phase_times",
+                                                  "dem_get_diagnostics", "dem_debug_snapshot", "dem_debug_tiles",
+                                                  "dem_get_grid", "dem_set_timing", "dem_get_phase_times",
                                                   "dem_sort_cells_static", "dem_batch_create", "dem_batch_add",
                                                   "dem_batch_run", "dem_batch_get_state", "dem_batch_remove",
                                                   "dem_batch_info", "dem_slab_bounds", "dem_slabs_create",
@@ -327,6 +328,13 @@ def dem_debug_snapshot(h, n, with_pairs=True):
     pairs = np.zeros((cnt.value, 2), np.uint32)
     _check(h, lib().dem_debug_snapshot(h, _ptr(cell), _ptr(order), cnt.value, _ptr(pairs), ctypes.byref(cnt)))
     return cell, order, pairs
+
+
+def dem_debug_tiles(h):
+    """(particles per tile, tiles, tiles whose halo did not fit) of list mode; zeros otherwise."""
+    out = np.zeros(3, np.int64)
+    _check(h, lib().dem_debug_tiles(h, _ptr(out)))
+    return tuple(int(k) for k in out)
 
 
 def dem_get_grid(h):
