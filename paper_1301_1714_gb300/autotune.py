@@ -12,10 +12,11 @@ from typing import List, Optional, Sequence, Tuple
 
 from . import dem
 
-# (block size, resort_interval, skin as a fraction of the largest radius)
+# (block size, resort_interval, skin as a fraction of the largest radius). In list mode block
+# sizes of 128 and more give the same tiles (at most four times the block size, at most 512).
 DEFAULT_CANDIDATES: Tuple[Tuple[int, int, float], ...] = (
     (256, 1, 0.0), (128, 1, 0.0),
-    (256, 0, 0.1), (128, 0, 0.05), (128, 0, 0.1), (128, 0, 0.15), (128, 0, 0.2), (96, 0, 0.1),
+    (128, 0, 0.05), (128, 0, 0.1), (128, 0, 0.15), (128, 0, 0.2), (96, 0, 0.1),
 )
 
 
@@ -77,7 +78,7 @@ def tune(params, x, v, w, r, candidates: Sequence[Tuple[int, int, float]] = DEFA
 # candidates for a batch of many small scenes: the whole batch sorts when any particle of
 # any scene has moved half its skin, so larger skins pay off sooner than for one scene
 BATCH_CANDIDATES: Tuple[Tuple[int, int, float], ...] = (
-    (256, 1, 0.0), (128, 0, 0.1), (256, 0, 0.1), (128, 0, 0.2), (128, 0, 0.3),
+    (256, 1, 0.0), (128, 0, 0.1), (128, 0, 0.2), (128, 0, 0.3),
 )
 
 

@@ -68,8 +68,7 @@ struct SceneDev {
     double alpha_t;             // tangential damping factor
     double kcoh_pi;             // pi * cohesion energy density
     float mu_roll_f, alpha_t_f, kcoh_pi_f;
-    float nrkt_f;               // -1 / kt
-    double nrkt;
+    double nrkt;                // -1 / kt (FP64 mode, linear stiffness)
     // positions inside [in_lo, in_hi) hash to a cell of the grid, all others are clamped to
     // it: the smallest coordinates (of the precision mode) whose quotient is >= 0 and >= dims
     double in_lo[3], in_hi[3];
@@ -347,20 +346,31 @@ __device__ __forceinline__ void two_prod(float a, float b, float& p, float& e) {
 
 // ----------------------------------------------------------- law parameters
 template <class T>
-struct Law {
+struct LawBase {
     T dt, kn, kt, cn, ct, alpha, mu, ksp, kda, ksh, mu_roll, alpha_t, kcoh_pi;
-    T nrkt;         // -1 / kt
     int stiffness;  // 0 linear, 1 Hertz
     int terms;      // 1: no attractive normal force, 2: rolling resistance
 };
+template <class T> struct Law : LawBase<T> {};
+template <> struct Law<double> : LawBase<double> {
+    double nrkt;    // -1 / kt
+};
 __device__ __forceinline__ Law<double> law_of(const SceneDev& s, int stiffness, double) {
-    return Law<double>{s.dt,  s.kn,  s.kt,  s.cn,      s.ct,      s.alpha,   s.mu,
-                       s.ksp, s.kda, s.ksh, s.mu_roll, s.alpha_t, s.kcoh_pi, s.nrkt, stiffness, s.terms};
+    return Law<double>{{s.dt,  s.kn,  s.kt,  s.cn,      s.ct,      s.alpha,   s.mu,
+                        s.ksp, s.kda, s.ksh, s.mu_roll, s.alpha_t, s.kcoh_pi, stiffness, s.terms},
+                       s.nrkt};
 }
 __device__ __forceinline__ Law<float> law_of(const SceneDev& s, int stiffness, float) {
-    return Law<float>{s.dt_f,  s.kn_f,  s.kt_f,  s.cn_f,      s.ct_f,      s.alpha_f,   s.mu_f,
-                      s.ksp_f, s.kda_f, s.ksh_f, s.mu_roll_f, s.alpha_t_f, s.kcoh_pi_f, s.nrkt_f, stiffness, s.terms};
+    return Law<float>{{s.dt_f,  s.kn_f,  s.kt_f,  s.cn_f,      s.ct_f,      s.alpha_f,   s.mu_f,
+                       s.ksp_f, s.kda_f, s.ksh_f, s.mu_roll_f, s.alpha_t_f, s.kcoh_pi_f, stiffness, s.terms}};
 }
+// -1 / k_t of a contact (FP64, linear stiffness: a constant of the scene)
+template <int STIFF>
+__device__ __forceinline__ double nrkt_of(const Law<double>& P, double kt) {
+    return STIFF == 0 ? P.nrkt : law_div(-1.0, kt);
+}
+template <int STIFF>
+__device__ __forceinline__ float nrkt_of(const Law<float>&, float kt) { return law_div(-1.f, kt); }
 
 // Practical contact law (Eqs. 2-10) for body i against partner j, seen from i:
 //   n      unit normal from i to j; delta overlap (> 0); v = v_i - v_j (or - wall velocity)
@@ -403,9 +413,7 @@ __device__ __forceinline__ void law_practical(const Law<T>& P, V3<T> n, T delta,
         T f;
         if (cap_of(P.mu, fn2, ft2, f)) {
             Ftt = scale(Ftt, f);
-            // (FP64, linear stiffness: -1 / k_t is a constant of the scene)
-            if (kt > T(0))
-                dt = scale(add(Ftt, damp), STIFF == 0 && sizeof(T) == 8 ? P.nrkt : law_div(T(-1), kt));
+            if (kt > T(0)) dt = scale(add(Ftt, damp), nrkt_of<STIFF>(P, kt));
         }
     }
     F = add(Fn, Ftt);                                            // Eq. 2

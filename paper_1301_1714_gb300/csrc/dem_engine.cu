@@ -257,7 +257,6 @@ void fill_scene(dem_handle* h, SceneDev& S, uint32_t p0, uint32_t np, uint32_t c
     S.mu_roll = c.mu_roll;
     S.mu_roll_f = (float)c.mu_roll;
     S.nrkt = -1.0 / c.kt;
-    S.nrkt_f = -1.0f / (float)c.kt;
     for (int a = 0; a < 3; ++a) {
         S.in_lo[a] = first_at(S.origin[a], S.h, 0.0);
         S.in_hi[a] = first_at(S.origin[a], S.h, (double)S.dims[a]);
@@ -514,11 +513,12 @@ int choose_bricks(const int64_t dims[3], int64_t nc, int64_t bdims[3], int64_t& 
     return 0;
 }
 
-// Threads per block of the walk's force pass when the configuration leaves it open: 256, and
-// less for few particles, down to one warp, so that the blocks reach every SM.
+// Threads per block of the FP32 walk's force pass when the configuration leaves it open: 256, and
+// less for few particles, down to 64 (fewer particles than those fill go by items), so that the
+// blocks reach every SM.
 int auto_block(const Domain& d, uint32_t n) {
     int b = 256;
-    while (b > 32 && n / (uint32_t)b < 2u * (uint32_t)(d.sort_blocks / 8)) b /= 2;
+    while (b > 64 && n / (uint32_t)b < 2u * (uint32_t)(d.sort_blocks / 8)) b /= 2;
     return b;
 }
 

@@ -24,21 +24,20 @@
 namespace demgb {
 
 // ======================================================================= force pass
-template <class PR>
 struct ForceArgs {
     const SceneDev* scenes;
     int nscenes;
     uint32_t n, cap;
     int maxc, stiffness;
-    typename PR::State S0, S1;   // the two state sets; ctrl->cur names the current one
+    StateF32 S0, S1;   // the two state sets; ctrl->cur names the current one
     CtrlDev* ctrl;
     const uint32_t* skey;
     const uint32_t* cs;
     const uint32_t* perm;
     const uint32_t* hin_cnt;
-    const Spring<typename PR::T>* hin;
+    const Spring<float>* hin;
     uint32_t* hout_cnt;
-    Spring<typename PR::T>* hout;
+    Spring<float>* hout;
     uint32_t* key;
     uint32_t* rank;
     uint32_t* cnt;
@@ -59,9 +58,10 @@ struct ForceArgs {
 // law with the scene's optional terms, 3 the practical law with Hertz stiffness. The terms need
 // more registers than the others' 64: with 85 (three blocks per SM) 1,000,001 spheres take 7.88 ms
 // per 20 steps, 30,001 0.96; with 64 10.09 and 1.22, with 128 9.33 and 0.88.
-template <class PR, int MODEL, bool EVAL>
-__global__ void __launch_bounds__(256, MODEL == 2 ? PR::WALK_BLOCKS - 1 : PR::WALK_BLOCKS) k_force(ForceArgs<PR> a) {
-    using T = typename PR::T;
+template <int MODEL, bool EVAL>
+__global__ void __launch_bounds__(256, MODEL == 2 ? PF32::WALK_BLOCKS - 1 : PF32::WALK_BLOCKS) k_force(ForceArgs a) {
+    using PR = PF32;
+    using T = float;
     constexpr bool PRACT = MODEL != 1;
     constexpr bool TERMS = MODEL == 2;
     constexpr int STIFF = MODEL == 2 ? 2 : (MODEL == 3 ? 1 : 0);
@@ -69,8 +69,8 @@ __global__ void __launch_bounds__(256, MODEL == 2 ? PR::WALK_BLOCKS - 1 : PR::WA
     // a void step (an earlier launch overflowed): nothing to do; one decision per warp
     if (!EVAL && __any_sync(0xffffffffu, (a.ctrl->rebuild & DEM_HALT) != 0)) return;
     const int cur = a.ctrl->cur;
-    const typename PR::State A = cur ? a.S1 : a.S0;
-    const typename PR::State B = cur ? a.S0 : a.S1;
+    const StateF32 A = cur ? a.S1 : a.S0;
+    const StateF32 B = cur ? a.S0 : a.S1;
     const bool pv = a.ctrl->perm_valid != 0;
     const uint32_t tid = threadIdx.x;
     const uint32_t bd = blockDim.x;
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(256, MODEL == 2 ? PR::WALK_BLOCKS - 1 : PR::WA
         V3<T> n;
         T delta;
         float rj;
-        const typename PR::Partner o = PR::load_partner(A, j);
+        const PR::Partner o = PR::load_partner(A, j);
         if (!PR::exact_p(A, o, me, n, delta, rj)) continue;
         const uint32_t gid = o.id;
         V3<T> vj, wj;
@@ -216,10 +216,7 @@ __global__ void __launch_bounds__(256, MODEL == 2 ? PR::WALK_BLOCKS - 1 : PR::WA
         if (PRACT || EVAL) a.hout_cnt[q] = min(nnew, maxc);
         // gravity, once per particle
         {
-            const T gx = sizeof(T) == 8 ? (T)S.g[0] : (T)S.g_f[0];
-            const T gy = sizeof(T) == 8 ? (T)S.g[1] : (T)S.g_f[1];
-            const T gz = sizeof(T) == 8 ? (T)S.g[2] : (T)S.g_f[2];
-            F = axpy(mk(gx, gy, gz), mi, F);
+            F = axpy(mk(S.g_f[0], S.g_f[1], S.g_f[2]), mi, F);
         }
         if (EVAL) {
             const size_t o = 3 * (size_t)me.id;
@@ -228,7 +225,7 @@ __global__ void __launch_bounds__(256, MODEL == 2 ? PR::WALK_BLOCKS - 1 : PR::WA
         } else {
             bool clamped = false, finite = true;
             float4 pnew;
-            const uint32_t kk = PR::template integrate<true>(B, q, me, F, Tq, S, mi, clamped, finite, pnew);
+            const uint32_t kk = PR::integrate<true>(B, q, me, F, Tq, S, mi, clamped, finite, pnew);
             if (!finite) raise_status(a.st, ST_NONFINITE, (int32_t)q);
             c_clamp = clamped ? 1u : 0u;
             c_disp2 = pnew.w;
@@ -950,27 +947,25 @@ cudaError_t run_loop_end(Domain& d) {
     return cudaSuccess;
 }
 
-template <class PR>
-static cudaError_t force_impl(Domain& d, const typename PR::State& S0, const typename PR::State& S1, bool eval,
-                              double* dbgF, double* dbgT) {
-    ForceArgs<PR> a;
+static cudaError_t run_force_walk(Domain& d, bool eval, double* dbgF, double* dbgT) {
+    ForceArgs a;
     a.scenes = d.d_scenes;
     a.nscenes = d.nscenes;
     a.n = d.n;
     a.cap = d.cap;
     a.maxc = d.maxc;
     a.stiffness = d.stiffness;
-    a.S0 = S0;
-    a.S1 = S1;
+    a.S0 = d.S32[0];
+    a.S1 = d.S32[1];
     a.ctrl = d.ctrl;
     a.skey = d.skey;
     a.cs = d.cs;
     a.perm = d.perm;
     const int hi = d.h_cur, ho = 1 - d.h_cur;
     a.hin_cnt = d.hcnt[hi];
-    a.hin = (const Spring<typename PR::T>*)d.hs[hi];
+    a.hin = (const Spring<float>*)d.hs[hi];
     a.hout_cnt = d.hcnt[ho];
-    a.hout = (Spring<typename PR::T>*)d.hs[ho];
+    a.hout = (Spring<float>*)d.hs[ho];
     a.key = d.key;
     a.rank = d.rank;
     a.cnt = d.cnt;
@@ -992,10 +987,10 @@ static cudaError_t force_impl(Domain& d, const typename PR::State& S0, const typ
     };
     cudaError_t e;
     const int model = d.model != 0 ? 1 : (d.terms != 0 ? 2 : (d.stiffness != 0 ? 3 : 0));
-    if (model == 0) e = eval ? launch(k_force<PR, 0, true>) : launch(k_force<PR, 0, false>);
-    else if (model == 2) e = eval ? launch(k_force<PR, 2, true>) : launch(k_force<PR, 2, false>);
-    else if (model == 3) e = eval ? launch(k_force<PR, 3, true>) : launch(k_force<PR, 3, false>);
-    else e = eval ? launch(k_force<PR, 1, true>) : launch(k_force<PR, 1, false>);
+    if (model == 0) e = eval ? launch(k_force<0, true>) : launch(k_force<0, false>);
+    else if (model == 2) e = eval ? launch(k_force<2, true>) : launch(k_force<2, false>);
+    else if (model == 3) e = eval ? launch(k_force<3, true>) : launch(k_force<3, false>);
+    else e = eval ? launch(k_force<1, true>) : launch(k_force<1, false>);
     if (e != cudaSuccess) return e;
     DEM_LAUNCH_CHECK();
     return cudaSuccess;
@@ -1013,7 +1008,7 @@ cudaError_t run_force(Domain& d, bool eval, double* dbgF, double* dbgT) {
     if (d.n == 0) return cudaSuccess;
     if (d.precision == 0 || (!d.list_mode && walk_by_items(d))) return run_force_items(d, eval, dbgF, dbgT);
     if (d.list_mode) return run_force_list(d, eval, dbgF, dbgT);
-    return force_impl<PF32>(d, d.S32[0], d.S32[1], eval, dbgF, dbgT);
+    return run_force_walk(d, eval, dbgF, dbgT);
 }
 
 cudaError_t run_export(Domain& d, double* x, double* v, double* w) {

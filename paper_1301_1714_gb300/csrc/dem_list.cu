@@ -26,14 +26,15 @@
 
 namespace demgb {
 
-template <class PR>
+using PR = PF32;
+using T = float;
+
 struct ListArgs {
-    using T = typename PR::T;
     const SceneDev* scenes;
     int nscenes;
     uint32_t cap, tile, hcap;
     int maxc, stiffness;
-    typename PR::State S0, S1;   // the two state sets; ctrl->cur names the current one
+    StateF32 S0, S1;             // the two state sets; ctrl->cur names the current one
     CtrlDev* ctrl;
     const uint32_t* ncnt;        // list lengths
     const uint32_t* nl;          // list entries (stored index), slot-major
@@ -60,9 +61,8 @@ struct ListArgs {
 // law with the scene's optional terms, 3 the practical law with Hertz stiffness (the paper's
 // two stiffnesses have a variant each: the other's constants would take registers).
 // EVAL: forces and torques by id instead of the update.
-template <class PR, int MODEL, bool EVAL>
-__global__ void __launch_bounds__(PR::LIST_THREADS, PR::LIST_BLOCKS) k_list(ListArgs<PR> a) {
-    using T = typename PR::T;
+template <int MODEL, bool EVAL>
+__global__ void __launch_bounds__(PR::LIST_THREADS, PR::LIST_BLOCKS) k_list(ListArgs a) {
     constexpr bool PRACT = MODEL != 1;
     constexpr bool TERMS = MODEL == 2;
     constexpr int STIFF = MODEL == 2 ? 2 : (MODEL == 3 ? 1 : 0);
@@ -79,8 +79,8 @@ __global__ void __launch_bounds__(PR::LIST_THREADS, PR::LIST_BLOCKS) k_list(List
     __syncthreads();
     if (!EVAL && s_void) return;   // an earlier launch (or another block) overflowed: a void step
     const int cur = a.ctrl->cur;
-    const typename PR::State A = cur ? a.S1 : a.S0;
-    const typename PR::State B = cur ? a.S0 : a.S1;
+    const StateF32 A = cur ? a.S1 : a.S0;
+    const StateF32 B = cur ? a.S0 : a.S1;
     const bool pv = a.ctrl->perm_valid != 0;
     const int hi = a.ctrl->hcur, ho = 1 - hi;
     if (!EVAL && blockIdx.x == 0 && tid == 0) {
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(PR::LIST_THREADS, PR::LIST_BLOCKS) k_list(List
     uint32_t c_pp = 0, c_wc = 0, c_clamp = 0, c_nnew = 0;
     float c_maxov = 0.f, c_disp2 = 0.f;
     if (valid) {
-        const typename PR::Self me = PR::tile_self(A, q, t_mem, E, tid);
+        const PR::Self me = PR::tile_self(A, q, t_mem, E, tid);
         // ---- phase 1: list entries that pass the prefilter (near[0]: entries 0-31, near[1]: 32-63)
         uint32_t near0 = 0, near1 = 0;
         {
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(PR::LIST_THREADS, PR::LIST_BLOCKS) k_list(List
             const uint32_t e = (uint32_t)__ffs((int)near0) - 1u;
             const uint32_t bit = 1u << e;
             near0 &= near0 - 1u;
-            typename PR::Partner pj;
+            PR::Partner pj;
             if (!direct)
                 pj = PR::tile_partner(
                     A, t_mem, E, __ldg((const uint16_t*)(a.nl4 + (size_t)((e0 + e) >> 2) * cap + q) + (e & 3u)));
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(PR::LIST_THREADS, PR::LIST_BLOCKS) k_list(List
             c_maxov = fmaxf(c_maxov, (float)delta);
         }
         c_pp = nnew;
-        const typename PR::Self me2 = PR::tile_again(me, t_mem, E, tid);
+        const PR::Self me2 = PR::tile_again(me, t_mem, E, tid);
         // ---- walls (step 8), those the last sort found within reach; their springs follow
         // the particles' ones
         const uint32_t w_first = (uint32_t)(__popc(om_lo) + __popc(om_hi));
@@ -286,10 +286,7 @@ __global__ void __launch_bounds__(PR::LIST_THREADS, PR::LIST_BLOCKS) k_list(List
         if (PRACT && !EVAL) *(uint2*)&mout[q] = e0 ? make_uint2(nm_lo, nm) : make_uint2(nm, 0u);
         // gravity, once per particle
         {
-            const T gx = sizeof(T) == 8 ? (T)S.g[0] : (T)S.g_f[0];
-            const T gy = sizeof(T) == 8 ? (T)S.g[1] : (T)S.g_f[1];
-            const T gz = sizeof(T) == 8 ? (T)S.g[2] : (T)S.g_f[2];
-            F = axpy(mk(gx, gy, gz), mi, F);
+            F = axpy(mk(S.g_f[0], S.g_f[1], S.g_f[2]), mi, F);
         }
         if (EVAL) {
             const size_t o = 3 * (size_t)me2.id;
@@ -298,7 +295,7 @@ __global__ void __launch_bounds__(PR::LIST_THREADS, PR::LIST_BLOCKS) k_list(List
         } else {
             bool clamped = false, finite = true;
             float4 pnew;
-            PR::template integrate<false>(B, q, me2, F, Tq, S, mi, clamped, finite, pnew);
+            PR::integrate<false>(B, q, me2, F, Tq, S, mi, clamped, finite, pnew);
             if (!finite) raise_status(a.st, ST_NONFINITE, (int32_t)q);
             c_clamp = clamped ? 1u : 0u;
             c_disp2 = pnew.w;
@@ -345,11 +342,9 @@ __global__ void __launch_bounds__(PR::LIST_THREADS, PR::LIST_BLOCKS) k_list(List
         if (e_ != cudaSuccess) return e_;           \
     } while (0)
 
-template <class PR>
-static cudaError_t force_list_impl(Domain& d, const typename PR::State& S0, const typename PR::State& S1, bool eval,
-                                   double* dbgF, double* dbgT) {
-    using T = typename PR::T;
-    ListArgs<PR> a;
+cudaError_t run_force_list(Domain& d, bool eval, double* dbgF, double* dbgT) {
+    if (d.n == 0) return cudaSuccess;
+    ListArgs a;
     a.scenes = d.d_scenes;
     a.nscenes = d.nscenes;
     a.cap = d.cap;
@@ -357,8 +352,8 @@ static cudaError_t force_list_impl(Domain& d, const typename PR::State& S0, cons
     a.hcap = halo_cap(d.tile);
     a.maxc = d.maxc;
     a.stiffness = d.stiffness;
-    a.S0 = S0;
-    a.S1 = S1;
+    a.S0 = d.S32[0];
+    a.S1 = d.S32[1];
     a.ctrl = d.ctrl;
     a.ncnt = d.ncnt;
     a.nl = d.nl;
@@ -390,18 +385,13 @@ static cudaError_t force_list_impl(Domain& d, const typename PR::State& S0, cons
         return cudaSuccess;
     };
     cudaError_t e;
-    if (model == 0) e = eval ? launch(k_list<PR, 0, true>) : launch(k_list<PR, 0, false>);
-    else if (model == 2) e = eval ? launch(k_list<PR, 2, true>) : launch(k_list<PR, 2, false>);
-    else if (model == 3) e = eval ? launch(k_list<PR, 3, true>) : launch(k_list<PR, 3, false>);
-    else e = eval ? launch(k_list<PR, 1, true>) : launch(k_list<PR, 1, false>);
+    if (model == 0) e = eval ? launch(k_list<0, true>) : launch(k_list<0, false>);
+    else if (model == 2) e = eval ? launch(k_list<2, true>) : launch(k_list<2, false>);
+    else if (model == 3) e = eval ? launch(k_list<3, true>) : launch(k_list<3, false>);
+    else e = eval ? launch(k_list<1, true>) : launch(k_list<1, false>);
     if (e != cudaSuccess) return e;
     DEM_LAUNCH_CHECK();
     return cudaSuccess;
-}
-
-cudaError_t run_force_list(Domain& d, bool eval, double* dbgF, double* dbgT) {
-    if (d.n == 0) return cudaSuccess;
-    return force_list_impl<PF32>(d, d.S32[0], d.S32[1], eval, dbgF, dbgT);
 }
 
 }  // namespace demgb

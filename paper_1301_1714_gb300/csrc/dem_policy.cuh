@@ -361,7 +361,7 @@ struct PF32 {
         p[0] = make_float4(L.dt, L.alpha, L.mu, L.kn);
         p[1] = make_float4(L.kt, L.cn, L.ct, L.ksp);
         p[2] = make_float4(L.kda, L.ksh, L.mu_roll, L.alpha_t);
-        p[3] = make_float4(L.kcoh_pi, __int_as_float(L.stiffness), __int_as_float(L.terms), L.nrkt);
+        p[3] = make_float4(L.kcoh_pi, __int_as_float(L.stiffness), __int_as_float(L.terms), 0.f);
     }
     static __device__ __forceinline__ Law<float> law(const Law<float>&, const unsigned char* s) {
         const float4 a = lds16(s), b = lds16(s + 16), c = lds16(s + 32), d = lds16(s + 48);
@@ -370,7 +370,6 @@ struct PF32 {
         L.kt = b.x; L.cn = b.y; L.ct = b.z; L.ksp = b.w;
         L.kda = c.x; L.ksh = c.y; L.mu_roll = c.z; L.alpha_t = c.w;
         L.kcoh_pi = d.x; L.stiffness = __float_as_int(d.y); L.terms = __float_as_int(d.z);
-        L.nrkt = d.w;
         return L;
     }
     static __device__ __forceinline__ float radius(const State& s, uint32_t q) { return __ldg(&s.P0[q].w); }
