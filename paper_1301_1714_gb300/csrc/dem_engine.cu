@@ -528,9 +528,10 @@ int auto_block(const Domain& d, uint32_t n) {
 // 64 spheres with a tile for their total, 448, took 1,495 us per 20 steps, with 64 824). Then,
 // by the number of particles, the tile that gives the busiest SM the least work, its halo
 // counted at 0.15 of a particle per entry (halo entries per particle of a dense bed beside each
-// size). Measured per pass with 512 or 256 / the choice: 262,144 spheres 2,399 / 2,319 us (448),
-// 131,072 in the hopper 2,185 / 2,053 (448), 100,003 861 / 810 (224). Few particles, and FP64
-// mode (powers of two): the largest tile that still gives two blocks per SM.
+// size). Measured per pass with 512 / 448 / 320 / 224 particles: 262,144 spheres 3,090 / 3,020 /
+// 3,170 / 3,082 us (448 chosen), 131,072 in the hopper 2,080 / 2,010 / 2,130 / 2,072 (448), 100,003
+// with the terms 979 / 944 / 977 / 914 (224), 500,009 simple 1,810 / 1,876 / 1,843 / 1,880 (512).
+// Few particles, and FP64 mode (powers of two): the largest tile that still gives two blocks per SM.
 uint32_t tile_size(const Domain& d, const std::vector<uint32_t>& scenes) {
     uint64_t n = 0;
     uint32_t largest = 0;

@@ -1,7 +1,7 @@
 // Force pass by contact items: FP64 mode (walk and lists) and the FP32 walk of few particles.
 //
 //   k_items  steps 5-8 and 1 (walk: also the new cell key of step 2) for a block of
-//            ITEM_THREADS threads on `tile` consecutive stored particles (16 to 256).
+//            ITEM_THREADS threads on `tile` consecutive stored particles (16 to 128).
 //            1. all threads search: the particles' list entries, or the 27 cells as 9 rows of
 //               three x-adjacent cells, against the FP32 prefilter;
 //            2. what passes becomes one item per pair, in shared memory: a pair of two
@@ -21,10 +21,9 @@
 // If the items of a block do not fit (ITEM_MAX), it takes its particles in several rounds and
 // evaluates every pair from both sides. The sums do not depend on any of this.
 // Measured (GB300, dense boxes, per step, thread per particle -> items): 2,048 spheres walking
-// 113 -> 54 us, 262,144 with lists 721 -> 547 us, one force evaluation of 65,537 (with load and
-// sort) 439 -> 304 us. Tiles of 64 / 128 / 256 particles take 721 / 547 / 745 us (smaller: fewer
-// pairs inside; larger: more than ITEM_MAX items); 85 registers and three blocks per SM 537 us
-// there, but 10-18% more on the small ones.
+// 230 -> 50 us, 262,144 with lists 1,026 -> 539 us, one force evaluation of 65,537 (with load and
+// sort) 564 -> 301 us. Tiles of 64 particles take 713 us with lists (fewer pairs inside; 256 would
+// be more than ITEM_MAX items), 85 registers and three blocks per SM 563 us and 10% more on 2,048.
 #include <algorithm>
 
 #include <cuda_runtime.h>

@@ -66,11 +66,12 @@ __global__ void __launch_bounds__(256) k_wall_masks(uint32_t n, const SceneDev* 
 // lanes look the cells up together (one each), number the candidates through by a scan of
 // the counts, read up to NLIST_REGS x 32 of them into registers once, and test all 32 lanes'
 // candidates against one particle of the cell at a time; the accepted ones are ranked by id
-// in shared memory. A warp takes `per` consecutive positions: 32, and less for few particles,
-// whose warps would otherwise walk their 10 to 16 cells one after another with most of the chip
-// idle (9,217 spheres: 49.8 us with 32, 15.0 with 4; 500: 43.2 and 13.3). (One thread per particle walked 27 x 0-5 candidates with its neighbours
+// in shared memory. (One thread per particle walked 27 x 0-5 candidates with its neighbours
 // in the warp on other cells, and sorted its list by insertion in local memory: 2.9 ms per
-// sort of the 4,194,304-sphere bed at 59 candidates and 10 list entries per particle.)
+// sort of the 4,194,304-sphere bed at 59 candidates and 10 list entries per particle, 1.6 now.)
+// A warp takes `per` consecutive positions: 32, and less for few particles, whose warps would
+// otherwise walk their 10 to 16 cells one after another with most of the chip idle (9,217
+// spheres: 49.8 us with 32, 15.0 with 4; 500: 43.2 and 13.3).
 constexpr int NLIST_REGS = 3;
 
 template <class PR>
@@ -258,9 +259,12 @@ __global__ void __launch_bounds__(512) k_tile(const SceneDev* scenes, int nscene
                 for (uint32_t u = 0; u < 4; ++u) jj[u] = k0 + u < m ? nl[(size_t)(k0 + u) * cap + q] : q0;
 #pragma unroll
                 for (uint32_t u = 0; u < 4; ++u) id[u] = o < c ? __ldg(&A.id[jj[u]]) : 0u;
-#pragma unroll
+                auto pick = [](const uint32_t (&a)[4], uint32_t u) {
+                    return u == 0 ? a[0] : (u == 1 ? a[1] : (u == 2 ? a[2] : a[3]));
+                };
+#pragma unroll 1   // (unrolled: 94 -> 99 us at 500,009 spheres, 31.6 -> 34.8 at 9,217)
                 for (uint32_t u = 0; u < 4; ++u) {
-                    const uint32_t k = k0 + u, j = jj[u], idj = id[u];
+                    const uint32_t k = k0 + u, j = pick(jj, u), idj = pick(id, u);
                     if (k >= m) break;
                     if (o < c && pid < DEM_WALL_BASE) {
                         while (o < c && pid < idj) {   // a partner that left the list

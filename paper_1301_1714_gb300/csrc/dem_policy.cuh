@@ -249,8 +249,8 @@ __device__ __forceinline__ void ff_diff(float hi, float lo, float phi, float plo
 
 struct PF32 {
     // Threads and resident blocks the list pass is compiled for (the largest tile), and the
-    // walk: 64 registers in both (measured: 80 or 128 registers lose more warps than they save
-    // spills, 0.61 / 0.69 / 0.85 ms per list pass at 4,194,304 spheres).
+    // walk: 64 registers in both (80 or 128 lose more warps than they save spills: 0.66 / 0.80 /
+    // 0.99 ms per list pass at 4,194,304 spheres; the walk with the optional terms: k_force).
     static constexpr int LIST_THREADS = DEM_TILE_MAX, LIST_BLOCKS = 2, WALK_BLOCKS = 4;
     using T = float;
     using State = StateF32;

@@ -51,3 +51,23 @@ def test_counts_and_intervals_against_plain_launches(stream, interval):
             got.append((*s.state(), s.history(), d["sorts"], d["steps"]))
     for a, b in zip(*got):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_scenes_join_a_batch_after_an_odd_number_of_steps(stream, precision):
+    """The springs of the scenes that stay are taken from the buffer the last step wrote."""
+    sc, v, p = _scene(0, 0.3)
+    p = p.copy(precision=precision)
+    b = dem.dem_batch_create(precision=precision, cuda_stream=stream.cuda_stream)
+    slots = [dem.dem_batch_add(b, p, sc.x, v, sc.w, sc.r, 1000)]
+    for k in (7, 3, 12):
+        dem.dem_batch_run(b, k)
+        slots.append(dem.dem_batch_add(b, p, sc.x, v, sc.w, sc.r, 1000))
+    dem.dem_batch_run(b, 9)
+    got = [dem.dem_batch_get_state(b, s, 1501) for s in slots]
+    dem.dem_batch_destroy(b)
+    for out, steps in zip(got, (31, 24, 21, 9)):
+        with dem.Simulation(p, sc.x, v, sc.w, sc.r) as s:
+            s.step(steps)
+            for a, c in zip(out, s.state()):
+                assert np.array_equal(a, c)
