@@ -94,9 +94,11 @@ enum { DEM_TERM_NO_ATTRACTION = 1, DEM_TERM_ROLLING = 2, DEM_TERM_ETA_T = 4, DEM
  *              candidates in ascending partner id (a fuller one makes dem_step return
  *              DEM_ERR_CAPACITY), so a particle's contacts are summed in that order and
  *              results do not depend on when the sorts happened.
- *  block_size  threads per block of the force kernel (32..256); 0 = automatic (256). List
- *              mode works in tiles of at most four times as many particles (at most 512;
- *              smaller tiles for few particles), one thread each. Results do not depend on it.
+ *  block_size  threads per block of the force kernel (32..256); 0 = automatic (256, fewer for
+ *              few particles). List mode works in tiles of at most four times as many
+ *              particles (64 to 512; smaller tiles for few particles and for small scenes of a
+ *              batch), one thread each. FP64 mode and FP32 walks of few particles work by
+ *              contacts and do not use it. Results do not depend on it.
  *  terms       optional force terms added to Eqs. 2-10 (none is in the paper; its force
  *              is built from separable terms so that terms can be added, Sec. 3), an OR of:
  *              DEM_TERM_NO_ATTRACTION  the normal force never pulls: F_n = 0 when
