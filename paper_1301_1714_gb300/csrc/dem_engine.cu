@@ -1220,11 +1220,7 @@ static dem_status download_u32(dem_handle* h, std::vector<uint32_t>& out, const 
     return DEM_OK;
 }
 
-// Spring records as the host sees them, and the device layout of either precision.
-struct HostSpring {
-    double d[3];
-    uint32_t pid;
-};
+// Spring records in the device layout of either precision.
 struct Raw32 {
     float d[3];
     uint32_t pid;
@@ -1234,21 +1230,23 @@ struct Raw64 {
     uint32_t pid, pad;
 };
 
-// The first mx slots of every particle of history buffer b.
-static dem_status download_springs(dem_handle* h, std::vector<HostSpring>& out, int b, uint32_t mx) {
+// The first mx slots of every particle of history buffer b, handed to use(records, slot-major).
+extern "C++" {
+template <class F>
+static dem_status with_springs(dem_handle* h, int b, uint32_t mx, F use) {
     Domain& d = h->d;
     const size_t count = (size_t)mx * d.cap;
-    out.resize(count);
     auto get = [&](auto raw) -> dem_status {
         std::vector<decltype(raw)> t(count);
         if (count)
             CK(h, cudaMemcpyAsync(t.data(), d.hs[b], count * sizeof(raw), cudaMemcpyDeviceToHost, d.stream));
         CK(h, cudaStreamSynchronize(d.stream));
-        for (size_t k = 0; k < count; ++k) out[k] = HostSpring{{(double)t[k].d[0], (double)t[k].d[1], (double)t[k].d[2]}, t[k].pid};
+        use(t);
         return DEM_OK;
     };
     return d.precision == 0 ? get(Raw64{}) : get(Raw32{});
 }
+}  // extern "C++"
 
 dem_status dem_get_history(dem_handle* h, int64_t cap, uint32_t* oi, uint32_t* oj, double* od, int64_t* nout) {
     if (!h || !nout || cap < 0) return DEM_ERR_INVALID_ARG;
@@ -1271,18 +1269,20 @@ dem_status dem_get_history(dem_handle* h, int64_t cap, uint32_t* oi, uint32_t* o
         for (size_t q = 0; q < n; ++q) perm[q] = (uint32_t)q;
     uint32_t mx = 0;
     for (size_t q = 0; q < n; ++q) mx = std::max(mx, slots_of(d, cnt[perm[q]]));
-    std::vector<HostSpring> sp;
-    if ((s = download_springs(h, sp, d.h_cur, mx)) != DEM_OK) return s;
     struct Rec { uint32_t i, j; double d[3]; };
     std::vector<Rec> recs;
-    for (size_t q = 0; q < n; ++q) {
-        const uint32_t src = perm[q], owner = ids[q];
-        const uint32_t c = slots_of(d, cnt[src]);
-        for (uint32_t k = 0; k < c; ++k) {
-            const HostSpring& f = sp[(size_t)k * N + src];
-            if (f.pid >= DEM_WALL_BASE || owner < f.pid) recs.push_back(Rec{owner, f.pid, {f.d[0], f.d[1], f.d[2]}});
+    s = with_springs(h, d.h_cur, mx, [&](const auto& sp) {
+        for (size_t q = 0; q < n; ++q) {
+            const uint32_t src = perm[q], owner = ids[q];
+            const uint32_t c = slots_of(d, cnt[src]);
+            for (uint32_t k = 0; k < c; ++k) {
+                const auto& f = sp[(size_t)k * N + src];
+                if (f.pid >= DEM_WALL_BASE || owner < f.pid)
+                    recs.push_back(Rec{owner, f.pid, {(double)f.d[0], (double)f.d[1], (double)f.d[2]}});
+            }
         }
-    }
+    });
+    if (s != DEM_OK) return s;
     std::sort(recs.begin(), recs.end(), [](const Rec& a, const Rec& b) { return a.i != b.i ? a.i < b.i : a.j < b.j; });
     *nout = (int64_t)recs.size();
     for (size_t k = 0; k < recs.size() && (int64_t)k < cap; ++k) {
@@ -1421,16 +1421,17 @@ dem_status dem_debug_snapshot(dem_handle* h, uint32_t* cell, uint32_t* order, in
         CK(h, cudaStreamSynchronize(d.stream));
         uint32_t mx = 0;
         for (size_t q = 0; q < n; ++q) mx = std::max(mx, slots_of(d, cnt[q]));
-        std::vector<HostSpring> sp;
-        if ((s = download_springs(h, sp, ho, mx)) != DEM_OK) return s;
         std::vector<std::pair<uint32_t, uint32_t>> pr;
-        for (size_t q = 0; q < n; ++q) {
-            const uint32_t c = slots_of(d, cnt[q]);
-            for (uint32_t k = 0; k < c; ++k) {
-                const uint32_t p = sp[(size_t)k * N + q].pid;
-                if (p < DEM_WALL_BASE && ids[q] < p) pr.emplace_back(ids[q], p);
+        s = with_springs(h, ho, mx, [&](const auto& sp) {
+            for (size_t q = 0; q < n; ++q) {
+                const uint32_t c = slots_of(d, cnt[q]);
+                for (uint32_t k = 0; k < c; ++k) {
+                    const uint32_t p = sp[(size_t)k * N + q].pid;
+                    if (p < DEM_WALL_BASE && ids[q] < p) pr.emplace_back(ids[q], p);
+                }
             }
-        }
+        });
+        if (s != DEM_OK) return s;
         std::sort(pr.begin(), pr.end());
         if (npairs) *npairs = (int64_t)pr.size();
         if (pairs)
